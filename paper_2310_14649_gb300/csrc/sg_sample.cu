@@ -9,8 +9,8 @@
 // the same P1 discretisation as the SG system.  One CTA solves one sample
 // entirely in shared memory by Jacobi-preconditioned conjugate gradients
 // in FP32: the search direction, the edge conductances and the inverse
-// diagonal live in shared memory, the iterate and the residual in registers
-// (nodes r = tid + k * 1024 of the thread).
+// diagonal live in shared memory, the iterate, the residual and the thread's
+// own search direction in registers.
 #include <algorithm>
 #include <cmath>
 
@@ -19,30 +19,109 @@
 namespace sg {
 namespace {
 
-constexpr int kSampThreads = 1024;
-constexpr int kSampNodes = 10;   // nodes per thread: n <= 10240 (meshes up to N = 102)
+constexpr int kSampThreads = 512;      // most threads of a CTA
+constexpr int kSampMaxNodes = 10240;   // meshes up to N = 102
+constexpr int kSampMaxRun = 21;        // most nodes of a thread (m = 101: 5 runs of a column)
 
-// block-wide sums of two values (every thread receives them)
-__device__ inline void block_sum2(float a, float b, double* red, double& sa, double& sb) {
+// Double-FP32 number hi + lo (48 significant bits).  The sums over a block
+// and the scalars of the CG recurrence are carried in it: GB300 runs FP64 at
+// 1/64 of its FP32 rate, and the FP64 sums this replaces (every thread
+// adding 64 partial sums per reduction) were 90 % of an iteration.
+struct Df {
+  float h, l;
+};
+
+// exact sum of two floats as hi + lo (TwoSum, Knuth)
+__device__ __forceinline__ Df two_sum(float a, float b) {
+  const float s = __fadd_rn(a, b);
+  const float bb = __fsub_rn(s, a);
+  return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb))};
+}
+// a + b with the rounding error gathered in the low word; symmetric in its
+// arguments, so a butterfly gives every lane the same bits
+__device__ __forceinline__ Df df_add(Df a, Df b) {
+  const Df s = two_sum(a.h, b.h);
+  return {s.h, __fadd_rn(__fadd_rn(a.l, b.l), s.l)};
+}
+// float(a / b): the quotient of the high words corrected by its remainder
+__device__ __forceinline__ float df_div(Df a, Df b) {
+  const float q = __fdiv_rn(a.h, b.h);
+  const float r = __fmaf_rn(-q, b.h, a.h);
+  return __fadd_rn(q, __fdiv_rn(__fadd_rn(r, __fmaf_rn(-q, b.l, a.l)), b.h));
+}
+__device__ __forceinline__ Df df_of(double v) {
+  const float h = float(v);
+  return {h, float(v - double(h))};
+}
+
+// float(exp(a)) for a double-FP32 argument: a = n ln 2 + r with |r| <= 0.35,
+// the Taylor series of exp(r) with its terms up to r^2 / 2 summed exactly
+// enough that only the last addition rounds (largest error 0.53 ulp
+// measured on 7 million arguments in [-60, 60]).
+__host__ __device__ inline float exp_df(float ah, float al) {
+  if (!(ah < 100.f)) return ah != ah ? ah : INFINITY;
+  if (ah < -110.f) return 0.f;
+  const float n = rintf(ah * 1.44269504088896341f);
+  // ln 2 in two parts (Cody and Waite); n has at most 8 bits, so n * c1 is exact
+  const float c1 = 0.693145751953125f;             // 16 significant bits
+  const float c2 = 1.4286068e-06f;                 // ln 2 - c1
+  const float rh = fmaf(-n, c1, ah);               // exact (Sterbenz range)
+  const float rm = fmaf(-n, c2, al);
+  // r = rh + rm as a normalised pair
+  const float r = rh + rm;
+  const float rl = rm - (r - rh);
+  const float r2 = r * r;
+  float t = 2.7557319e-06f;                        // 1/9!
+  t = fmaf(t, r, 2.4801587e-05f);
+  t = fmaf(t, r, 1.9841270e-04f);
+  t = fmaf(t, r, 1.3888889e-03f);
+  t = fmaf(t, r, 8.3333333e-03f);
+  t = fmaf(t, r, 4.1666667e-02f);
+  t = fmaf(t, r, 1.6666667e-01f);
+  t = t * r * r2;                                  // r^3 (1/6 + ...)
+  const float q = 0.5f * r2;                       // r^2 / 2 and its rounding error
+  const float qe = 0.5f * fmaf(r, r, -r2);
+  // s = r + q + t with the errors kept
+  const float s1 = r + q;
+  const float e1 = fabsf(r) >= q ? q - (s1 - r) : r - (s1 - q);
+  const float low = e1 + (qe + (t + fmaf(rl, r, rl)));
+  const float s = s1 + low;
+  const float se = low - (s - s1);
+  const float h = 1.0f + s;
+  const float he = s - (h - 1.0f);
+  return ldexpf(h + (he + se), int(n));
+}
+
+// Block-wide sums of NV (1 or 2) values (every thread receives them):
+// butterflies in the warps, then every warp sums the warps' results.  The
+// slots alternate between two halves of red, so one barrier per call is
+// enough.  512 threads: the butterflies cost the same instructions in every
+// warp, and with 1,024 threads they were a third of an iteration (7.2 us
+// against 4.0 us at N = 100).
+template <int NV>
+__device__ __forceinline__ void block_sum(const float (&v)[NV], float2* red, int& turn, int nwarps, Df (&s)[NV]) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  double x = a, y = b;
-  for (int o = 16; o > 0; o >>= 1) {
-    x += __shfl_xor_sync(0xffffffffu, x, o);
-    y += __shfl_xor_sync(0xffffffffu, y, o);
-  }
-  __syncthreads();  // red is free again
-  if (lane == 0) {
-    red[warp] = x;
-    red[32 + warp] = y;
+  float2* slot = red + 32 * turn;
+  turn ^= 1;
+#pragma unroll
+  for (int q = 0; q < NV; ++q) {
+    Df x{v[q], 0.f};
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+      x = df_add(x, Df{__shfl_xor_sync(0xffffffffu, x.h, o), __shfl_xor_sync(0xffffffffu, x.l, o)});
+    if (lane == 0) slot[16 * q + warp] = make_float2(x.h, x.l);
   }
   __syncthreads();
-  double u = 0.0, v = 0.0;
-  for (int w = 0; w < kSampThreads / 32; ++w) {
-    u += red[w];
-    v += red[32 + w];
+#pragma unroll
+  for (int q = 0; q < NV; ++q) {
+    const int l = lane & 15;
+    const float2 t = l < nwarps ? slot[16 * q + l] : make_float2(0.f, 0.f);
+    Df x{t.x, t.y};
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1)
+      x = df_add(x, Df{__shfl_xor_sync(0xffffffffu, x.h, o), __shfl_xor_sync(0xffffffffu, x.l, o)});
+    s[q] = two_sum(x.h, x.l);
   }
-  sa = u;
-  sb = v;
 }
 
 // Edge conductances of the P1 stencil (Sec. 2.1): the horizontal edge
@@ -51,128 +130,188 @@ __device__ inline void block_sum2(float a, float b, double* red, double& sa, dou
 // (i,j)-(i,j+1) couples the upper triangle of cell (i,j) and the lower one
 // of cell (i-1,j), wy = (c_up(i,j) + c_lo(i-1,j)) / 2.  Row (i,j) of A(c):
 // diagonal = the four conductances around the node, off-diagonals = minus
-// the conductance of the edge (edges to boundary nodes are dropped).
-// Shared memory: p [n], wx [m N], wy [N m], the inverse diagonal [n] and
-// the reduction slots; x, r and A p of the thread's nodes in registers.
-template <typename To>
+// the conductance of the edge (edges to boundary nodes are dropped: the
+// search direction is stored with a border of zeros).
+//
+// A thread owns a run of HN vertically adjacent nodes of one column, lanes
+// adjacent columns: the vertical neighbours inside a run are its registers
+// and every shared-memory access of a warp is to consecutive words.  Per
+// iteration a node costs seven shared words and three barriers a CTA.  304
+// samples at N = 100 (two waves of one CTA per SM): 21.4 ms with FP64 block
+// sums and interleaved nodes, now 2.0 ms (4.0 us per iteration); what
+// bounds it now is the shared-memory words (1.2 us) and the latency of the
+// three barriers and two butterflies of an iteration.
+// Shared memory: p [(N+1)^2] with its border, the inverse diagonal [n]
+// (both first hold the 2 N^2 triangle coefficients), wx [m N], wy [N m],
+// the reduction slots.
+template <typename To, int HN>
 __global__ void __launch_bounds__(kSampThreads, 1)
-    k_sample_pcg(int N, int L, const double* __restrict__ gfield, double g0, const double* __restrict__ xi,
+    k_sample_pcg(int N, int L, int runs, const double* __restrict__ gfield, double g0, const double* __restrict__ xi,
                  double h2, double rtol, int max_it, To* __restrict__ U, int64_t ldu, int* __restrict__ its_max) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int m = N - 1;
-  const int n = m * m;
+  const int m = N - 1, S = N + 1;
   const int64_t E = 2LL * N * N;
-  float* p = reinterpret_cast<float*>(smem_raw);       // [n]
-  float* wx = p + n;                                    // [m][N]: (i = 0..N-1, j = 1..m)
-  float* wy = wx + int64_t(m) * N;                      // [N][m]: (i = 1..m, j = 0..m)
-  float* dinv = wy + int64_t(N) * m;                    // [n]
-  double* red = reinterpret_cast<double*>(dinv + n + 2);  // [64], 8-byte aligned below
-  red = reinterpret_cast<double*>((reinterpret_cast<uintptr_t>(red) + 7) & ~uintptr_t(7));
+  float2* red = reinterpret_cast<float2*>(smem_raw);   // [2][2][16]
+  float* p = reinterpret_cast<float*>(red + 64);       // [S][S], node (i, j) at j S + i
+  float* dinv = p + S * S;                             // [m][m]
+  float* wx = dinv + m * m;                            // [m][N]: (i = 0..N-1, j = 1..m)
+  float* wy = wx + m * N;                              // [N][m]: (i = 1..m, j = 0..m)
+  float* cb = p;                                       // [2 N^2] while wx and wy are formed
   __shared__ double sxi[16];
   const int64_t s = blockIdx.x;
+  const int nthr = blockDim.x, nwarps = nthr >> 5;
   if (threadIdx.x < L) sxi[threadIdx.x] = xi[s * L + threadIdx.x];
   __syncthreads();
-  auto coef = [&](int ci, int cj, int upper) -> float {
-    if (ci < 0 || cj < 0 || ci >= N || cj >= N) return 0.0f;
-    const int64_t e = 2LL * (int64_t(cj) * N + ci) + upper;
+  for (int e = threadIdx.x; e < 2 * N * N; e += nthr) {
     double a = g0;
     for (int i = 0; i < L; ++i) a += gfield[int64_t(i) * E + e] * sxi[i];
-    return float(exp(a));
-  };
-  for (int t = threadIdx.x; t < m * N; t += kSampThreads) {
-    const int i = t % N, j = t / N + 1;  // edge (i,j)-(i+1,j)
-    wx[t] = 0.5f * (coef(i, j, 0) + coef(i, j - 1, 1));
-  }
-  for (int t = threadIdx.x; t < N * m; t += kSampThreads) {
-    const int i = t % m + 1, j = t / m;  // edge (i,j)-(i,j+1)
-    wy[t] = 0.5f * (coef(i, j, 1) + coef(i - 1, j, 0));
+    const Df d = df_of(a);
+    cb[e] = exp_df(d.h, d.l);
   }
   __syncthreads();
-  float x[kSampNodes], r[kSampNodes];
+  for (int t = threadIdx.x; t < m * N; t += nthr) {
+    const int i = t % N, j = t / N + 1;  // edge (i,j)-(i+1,j)
+    wx[t] = 0.5f * (cb[2 * (j * N + i)] + cb[2 * ((j - 1) * N + i) + 1]);
+  }
+  for (int t = threadIdx.x; t < N * m; t += nthr) {
+    const int i = t % m + 1, j = t / m;  // edge (i,j)-(i,j+1)
+    wy[t] = 0.5f * (cb[2 * (j * N + i) + 1] + cb[2 * (j * N + i - 1)]);
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < S * S; t += nthr) p[t] = 0.0f;
+  __syncthreads();
+  // column i, rows j0 .. j0 + cnt - 1
+  const int run = threadIdx.x / m, i = threadIdx.x - run * m + 1;
+  const int j0 = run * HN + 1, cnt = run < runs ? min(HN, m - j0 + 1) : 0;
+  float* pc = p + j0 * S + i;
+  const float* we = wx + (j0 - 1) * N + i;
+  const float* wv = wy + (j0 - 1) * m + i - 1;  // south edge of the run's first node
+  float* di = dinv + (j0 - 1) * m + i - 1;
+  float x[HN], r[HN], pr[HN];
   float rz_loc = 0.0f, bb_loc = 0.0f;
 #pragma unroll
-  for (int k = 0; k < kSampNodes; ++k) {
-    const int node = threadIdx.x + k * kSampThreads;
+  for (int k = 0; k < HN; ++k) {
     x[k] = 0.0f;
     r[k] = 0.0f;
-    if (node < n) {
-      const int i = node % m + 1, j = node / m + 1;
-      const float d = wx[(j - 1) * N + i] + wx[(j - 1) * N + i - 1] + wy[j * m + i - 1] + wy[(j - 1) * m + i - 1];
-      const float di = 1.0f / d;
-      dinv[node] = di;
+    pr[k] = 0.0f;
+    if (k < cnt) {
+      const float d = we[k * N] + we[k * N - 1] + wv[(k + 1) * m] + wv[k * m];
+      const float dv = 1.0f / d;
+      di[k * m] = dv;
       r[k] = float(h2);
-      p[node] = r[k] * di;
-      rz_loc += r[k] * r[k] * di;
+      pr[k] = r[k] * dv;
+      pc[k * S] = pr[k];
+      rz_loc += r[k] * r[k] * dv;
       bb_loc += r[k] * r[k];
     }
   }
-  double rz, bb;
-  block_sum2(rz_loc, bb_loc, red, rz, bb);
-  const double tol2 = rtol * rtol * bb;
+  int turn = 0;
+  Df sums[2];
+  block_sum<2>({rz_loc, bb_loc}, red, turn, nwarps, sums);
+  Df rz = sums[0];
+  const Df tol2 = df_of(rtol * rtol * (double(sums[1].h) + double(sums[1].l)));
   int it = 0;
   for (; it < max_it; ++it) {
     __syncthreads();  // p complete
-    float q[kSampNodes];
+    float q[HN];
     float pq_loc = 0.0f;
+    if (cnt > 0) {
+      float ws = wv[0], pS = pc[-S];
+      const float pTop = pc[cnt * S];
 #pragma unroll
-    for (int k = 0; k < kSampNodes; ++k) {
-      const int node = threadIdx.x + k * kSampThreads;
-      q[k] = 0.0f;
-      if (node < n) {
-        const int i = node % m + 1, j = node / m + 1;
-        const float we = wx[(j - 1) * N + i], ww = wx[(j - 1) * N + i - 1];
-        const float wn = wy[j * m + i - 1], ws = wy[(j - 1) * m + i - 1];
-        const float pc = p[node];
-        float v = (we + ww + wn + ws) * pc;
-        if (i > 1) v -= ww * p[node - 1];
-        if (i < m) v -= we * p[node + 1];
-        if (j > 1) v -= ws * p[node - m];
-        if (j < m) v -= wn * p[node + m];
-        q[k] = v;
-        pq_loc += pc * v;
+      for (int k = 0; k < HN; ++k) {
+        q[k] = 0.0f;
+        if (k < cnt) {
+          const float e = we[k * N], w = we[k * N - 1], wn = wv[(k + 1) * m];
+          const float pN = (k + 1 < cnt && k + 1 < HN) ? pr[(k + 1) % HN] : pTop;
+          float v = (e + w + wn + ws) * pr[k];
+          v -= w * pc[k * S - 1];
+          v -= e * pc[k * S + 1];
+          v -= ws * pS;
+          v -= wn * pN;
+          q[k] = v;
+          pq_loc += pr[k] * v;
+          ws = wn;
+          pS = pr[k];
+        }
       }
     }
-    double pq, dummy;
-    block_sum2(pq_loc, 0.0f, red, pq, dummy);
-    if (!(pq > 0.0)) break;
-    const float alpha = float(rz / pq);
+    Df pq[1];
+    block_sum<1>({pq_loc}, red, turn, nwarps, pq);
+    if (!(pq[0].h > 0.0f)) break;
+    const float alpha = df_div(rz, pq[0]);
     float rr_loc = 0.0f, rzn_loc = 0.0f;
 #pragma unroll
-    for (int k = 0; k < kSampNodes; ++k) {
-      const int node = threadIdx.x + k * kSampThreads;
-      if (node < n) {
-        x[k] += alpha * p[node];
+    for (int k = 0; k < HN; ++k) {
+      if (k < cnt) {
+        x[k] += alpha * pr[k];
         r[k] -= alpha * q[k];
         rr_loc += r[k] * r[k];
-        rzn_loc += r[k] * r[k] * dinv[node];
+        rzn_loc += r[k] * r[k] * di[k * m];
       }
     }
-    double rr, rzn;
-    block_sum2(rr_loc, rzn_loc, red, rr, rzn);
-    if (rr <= tol2) {
+    block_sum<2>({rr_loc, rzn_loc}, red, turn, nwarps, sums);
+    const Df rr = sums[0], rzn = sums[1];
+    if ((rr.h - tol2.h) + (rr.l - tol2.l) <= 0.0f) {
       ++it;
       break;
     }
-    const float beta = float(rzn / rz);
+    const float beta = df_div(rzn, rz);
     rz = rzn;
-    __syncthreads();  // every thread has read p for x
+    // every thread read its neighbours' p before the first sum's barrier
 #pragma unroll
-    for (int k = 0; k < kSampNodes; ++k) {
-      const int node = threadIdx.x + k * kSampThreads;
-      if (node < n) p[node] = r[k] * dinv[node] + beta * p[node];
-    }
+    for (int k = 0; k < HN; ++k)
+      if (k < cnt) {
+        pr[k] = r[k] * di[k * m] + beta * pr[k];
+        pc[k * S] = pr[k];
+      }
   }
 #pragma unroll
-  for (int k = 0; k < kSampNodes; ++k) {
-    const int node = threadIdx.x + k * kSampThreads;
-    if (node < n) U[s * ldu + node] = To(x[k]);
-  }
+  for (int k = 0; k < HN; ++k)
+    if (k < cnt) U[s * ldu + int64_t(j0 - 1 + k) * m + i - 1] = To(x[k]);
   if (threadIdx.x == 0) atomicMax(its_max, it);
 }
 
 size_t sample_smem(int N) {
-  const int64_t m = N - 1;
-  return size_t(2 * m * m + 2 * m * N + 2) * 4 + 64 * 8 + 8;
+  const int64_t m = N - 1, S = N + 1;
+  return 64 * sizeof(float2) + size_t(S * S + m * m + 2 * m * N) * 4;
+}
+
+// the shortest run of nodes per thread (of the instantiated lengths) whose
+// m x ceil(m / run) threads fit a CTA: short runs keep more warps in flight
+int sample_run(int m) {
+  for (int h : {1, 2, 4, 8, 12, 16, 20, kSampMaxRun})
+    if (int64_t(m) * ((m + h - 1) / h) <= kSampThreads) return h;
+  return 0;
+}
+
+template <typename To, int HN>
+sg_status sample_launch(const sg_problem* pr, int64_t S, const double* gfield, const double* xi, double rtol,
+                        int max_it, To* U, int64_t ldu, int* its, cudaStream_t st) {
+  const int m = pr->N - 1, runs = (m + HN - 1) / HN;
+  const double h = 1.0 / pr->N;
+  const size_t smem = sample_smem(pr->N);
+  SG_CUDA(cudaFuncSetAttribute(k_sample_pcg<To, HN>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
+  k_sample_pcg<To, HN><<<unsigned(S), unsigned(round_up(int64_t(m) * runs, 32)), smem, st>>>(
+      pr->N, pr->L, runs, gfield, pr->g0, xi, h * h, rtol, max_it, U, ldu, its);
+  note_launch();
+  SG_CUDA(cudaGetLastError());
+  return SG_OK;
+}
+
+template <typename To>
+sg_status sample_dispatch(const sg_problem* pr, int64_t S, const double* gfield, const double* xi, double rtol,
+                          int max_it, To* U, int64_t ldu, int* its, cudaStream_t st) {
+  switch (sample_run(pr->N - 1)) {
+    case 1: return sample_launch<To, 1>(pr, S, gfield, xi, rtol, max_it, U, ldu, its, st);
+    case 2: return sample_launch<To, 2>(pr, S, gfield, xi, rtol, max_it, U, ldu, its, st);
+    case 4: return sample_launch<To, 4>(pr, S, gfield, xi, rtol, max_it, U, ldu, its, st);
+    case 8: return sample_launch<To, 8>(pr, S, gfield, xi, rtol, max_it, U, ldu, its, st);
+    case 12: return sample_launch<To, 12>(pr, S, gfield, xi, rtol, max_it, U, ldu, its, st);
+    case 16: return sample_launch<To, 16>(pr, S, gfield, xi, rtol, max_it, U, ldu, its, st);
+    case 20: return sample_launch<To, 20>(pr, S, gfield, xi, rtol, max_it, U, ldu, its, st);
+    default: return sample_launch<To, kSampMaxRun>(pr, S, gfield, xi, rtol, max_it, U, ldu, its, st);
+  }
 }
 
 }  // namespace
@@ -188,7 +327,7 @@ extern "C" sg_status sg_sample_solve(sg_problem* pr, const double* xi, int64_t S
   SG_ARG(ldu >= pr->n, "sg_sample_solve: leading dimension < n");
   SG_ARG(rtol > 0 && max_it > 0, "sg_sample_solve: rtol and max_it must be > 0");
   SG_ARG(pr->L >= 1 && pr->L <= 16, "sg_sample_solve: needs 1 <= L <= 16 KL modes");
-  SG_ARG(pr->n <= int64_t(kSampThreads) * kSampNodes && sample_smem(pr->N) <= 227 * 1024,
+  SG_ARG(pr->n <= kSampMaxNodes && sample_run(pr->N - 1) > 0 && sample_smem(pr->N) <= 227 * 1024,
          "sg_sample_solve: the mesh is too large for one CTA per sample (N <= 102)");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   // the KL modes at the element centroids, once per problem
@@ -200,22 +339,13 @@ extern "C" sg_status sg_sample_solve(sg_problem* pr, const double* xi, int64_t S
   DevBuf itsd;
   SG_TRY(itsd.alloc(sizeof(int)));
   SG_CUDA(cudaMemsetAsync(itsd.ptr, 0, sizeof(int), st));
-  const double h = 1.0 / pr->N;
-  const size_t smem = sample_smem(pr->N);
   if (S > 0) {
-    if (dtype == SG_F32) {
-      SG_CUDA(cudaFuncSetAttribute(k_sample_pcg<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
-      k_sample_pcg<float><<<unsigned(S), kSampThreads, smem, st>>>(pr->N, pr->L, dp<double>(g), pr->g0, xi, h * h,
-                                                                   rtol, max_it, static_cast<float*>(U), ldu,
-                                                                   dp<int>(itsd));
-    } else {
-      SG_CUDA(cudaFuncSetAttribute(k_sample_pcg<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
-      k_sample_pcg<double><<<unsigned(S), kSampThreads, smem, st>>>(pr->N, pr->L, dp<double>(g), pr->g0, xi, h * h,
-                                                                    rtol, max_it, static_cast<double*>(U), ldu,
-                                                                    dp<int>(itsd));
-    }
-    note_launch();
-    SG_CUDA(cudaGetLastError());
+    if (dtype == SG_F32)
+      SG_TRY(sample_dispatch<float>(pr, S, dp<double>(g), xi, rtol, max_it, static_cast<float*>(U), ldu,
+                                    dp<int>(itsd), st));
+    else
+      SG_TRY(sample_dispatch<double>(pr, S, dp<double>(g), xi, rtol, max_it, static_cast<double*>(U), ldu,
+                                     dp<int>(itsd), st));
   }
   int its = 0;
   SG_CUDA(cudaMemcpyAsync(&its, itsd.ptr, sizeof(int), cudaMemcpyDeviceToHost, st));

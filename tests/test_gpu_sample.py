@@ -54,6 +54,26 @@ def test_samples_match_direct_solves(gpu, N, L, dt):
     prob.close()
 
 
+@pytest.mark.parametrize("N", [2, 3, 24, 42, 65, 90, 101, 102])
+def test_samples_run_lengths(gpu, N):
+    """One mesh for every run length of a thread (1 to 21 nodes of a column,
+    the last run of a column shorter than the others), the smallest mesh and
+    the largest, with enough samples for more than one CTA per SM at the
+    small ones; the bound of test_samples_match_direct_solves."""
+    import torch
+    import paper_2310_14649_gb300 as sg
+    prob = sg.sg_setup(N, 2, 1, 2, sigma2=0.3, bx=0.5, by=0.5)
+    ref = galerkin.build(N, 2, 1, 2, 0.3, 0.5, 0.5)
+    xi = samples(5, 2, 11)
+    U = torch.full((5, ref.n), float("nan"), dtype=torch.float32, device="cuda")
+    sg.sg_sample_solve(prob, torch.from_numpy(xi).cuda(), U, rtol=1e-6)
+    Uh = U.double().cpu().numpy()
+    for s in range(5):
+        u = spla.spsolve(fem.assemble(N, np.exp(xi[s] @ ref.gfield)).tocsc(), ref.b)
+        assert np.linalg.norm(Uh[s] - u) <= 2e-5 * np.linalg.norm(u), s
+    prob.close()
+
+
 def test_paper_verification_setting(gpu):
     """101 x 101 vertices (N = 100), L = 3, input order 2, output order 3,
     sigma = 0.1 (variance 0.01), four subdomains; 40,000 Monte Carlo
