@@ -229,22 +229,27 @@ sg_status sg_residual_refine(sg_problem* prob, const double* F_dev, int64_t ldf,
 sg_status sg_apply_config(sg_problem* prob, int which, int rows, int groups, int igroups, int sgroups,
                           int prefetch, int min_blocks, int stages, int cgroups, int warps);
 
-/* Edge-flux form of the fine FP32 operator (Sec. 2.1, Eq. Galerkin_L_exp
- * in Kronecker form, the stiffness written edge by edge): on this mesh the
+/* Edge form of the FP32 operators (Sec. 2.1, Eq. Galerkin_L_exp in
+ * Kronecker form, the stiffness written edge by edge): on this mesh the
  * rows of every A_k are
  *     (A_k x)_r = sum over the four edges (r, r') of w_k(r, r') (x_r - x_r'),
  * x_r' = 0 at a Dirichlet node, with one conductance w_k per edge (half the
  * sum of c_k over the two triangles sharing it).  Storing the K
  * conductances of the 2 N (N - 1) edges instead of the K values of five
  * stencil slots per node reads 2.5 times fewer matrix bytes per apply, and
- * four edge passes replace five slot passes.  mode 0: the five-slot form
- * (the autotuner may not choose the edge form); 1: the edge form now (its
- * K x 2 N (N - 1) FP32 conductances are built on first use); 2 (default):
- * the autotuner (sg_apply_autotune, fine FP32 family) times both forms and
- * keeps the faster; -1: no change.  on (may be NULL) receives 1 when fine
- * FP32 applies use the edge form.  sg_apply_config selects the slot form.
- * Coarse and FP64 applies are unaffected.  A change drops recorded
- * coarse-solve graphs; recorded batches of this problem then refuse to run.
+ * each edge's flux is formed once for both its nodes; the differences are
+ * formed before any product, so the rounding error is smaller too.  It is
+ * the default of sg_apply and sg_residual in FP32, of the nonlinear
+ * operators, and of FP32 solves up to P = 48 (above that a solve keeps the
+ * five-slot form unless the fine family was configured or tuned: the
+ * rounding of the FP32 operator shows in the returned solution there).
+ * mode 0: the five-slot form of the fine operator (the autotuner may not
+ * choose the edge form); 1: the edge form, in solves at any P; 2: the
+ * autotuner (sg_apply_autotune, fine FP32 family) may choose the edge form;
+ * -1: no change.  on (may be NULL) receives 1 when fine FP32 applies use the
+ * edge form.  sg_apply_config selects the slot form of its family.  FP64
+ * applies are unaffected.  A change drops recorded coarse-solve graphs;
+ * recorded batches of this problem then refuse to run.
  * Errors: SG_ERR_ARG (mode out of range; mode 1 without the specialised
  * kernel), SG_ERR_NOMEM, SG_ERR_CUDA. */
 sg_status sg_apply_flux(sg_problem* prob, int mode, int* on);

@@ -389,8 +389,9 @@ def sg_apply_config(prob, rows=1, groups=1, igroups=1, sgroups=1, prefetch=8, mi
 
 
 def sg_apply_flux(prob, mode=-1):
-    """Edge-flux form of the fine FP32 operator: 0 slot form, 1 edge form,
-    2 autotuner decides, -1 query.  Returns 1 when the edge form is used."""
+    """Edge form of the fine FP32 operator (the default): 0 slot form, 1 edge
+    form (in solves at any P), 2 the autotuner may choose it, -1 query.
+    Returns 1 when fine FP32 applies use the edge form."""
     on = ctypes.c_int(0)
     call("sg_apply_flux", prob.handle, mode, ctypes.byref(on))
     return on.value

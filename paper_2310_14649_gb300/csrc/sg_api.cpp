@@ -71,7 +71,7 @@ sg_status sg_destroy(sg_problem* pr) {
   solver_free(pr);
   cnn_free(pr);
   newton_free(pr);
-  for (int w = 0; w < kJitFamilies; ++w) jit_free(pr, w);
+  for (int w = 0; w < kJitAllFamilies; ++w) jit_free(pr, w);
   pr->mdot_partial.free_();
   pr->mdot_counter.free_();
   pr->fine.col.free_();
@@ -117,20 +117,13 @@ sg_status sg_apply_config(sg_problem* pr, int which, int rows, int groups, int i
 
 sg_status sg_apply_flux(sg_problem* pr, int mode, int* on) {
   SG_ARG(pr && mode >= -1 && mode <= 2, "sg_apply_flux: NULL handle or mode not in [-1, 2]");
-  if (mode >= 0) pr->flux_allowed = mode != 0;
-  if (mode == 0 || mode == 1) {
-    SG_ARG(jit_eligible(pr) || mode == 0, "sg_apply_flux: the edge-flux form needs the specialised kernel");
-    JitConfig c = pr->jit_cfg_set[0] ? pr->jit_cfg[0] : jit_default_config(pr, 0);
-    if (mode == 1 && (c.rows != 1 || c.stages != 0 || c.cgroups != 1)) {
-      c.rows = 1;
-      c.stages = 0;
-      c.cgroups = 1;
-      c.prefetch = std::max(c.prefetch, 8);
-    }
-    c.flux = mode;
-    if (pr->flux_on != c.flux || !pr->jit_cfg_set[0]) SG_TRY(jit_configure(pr, 0, c));
+  SG_ARG(mode != 1 || jit_eligible(pr), "sg_apply_flux: the edge form needs the specialised kernel");
+  if (mode >= 0) {
+    const JitConfig was = jit_config(pr, 0);
+    pr->flux_allowed = mode != 0;
+    if ((mode == 0 || mode == 1) && was.flux != mode) SG_TRY(jit_configure(pr, 0, jit_default_config(pr, 0)));
   }
-  if (on) *on = pr->flux_on;
+  if (on) *on = jit_eligible(pr) && jit_config(pr, 0).flux;
   return SG_OK;
 }
 
@@ -141,7 +134,7 @@ sg_status sg_apply_autotune(sg_problem* pr, int which, int force, double* best_m
 
 sg_status sg_apply_info(const sg_problem* pr, int which, int* cfg10, double* compile_s) {
   SG_ARG(pr && which >= 0 && which < kJitFamilies, "sg_apply_info: NULL handle or which not in [0, 3]");
-  const JitConfig c = pr->jit_cfg_set[which] ? pr->jit_cfg[which] : jit_default_config(pr, which);
+  const JitConfig c = jit_config(pr, which);
   if (cfg10) {
     cfg10[0] = c.rows;
     cfg10[1] = c.groups;

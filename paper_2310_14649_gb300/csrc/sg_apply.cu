@@ -305,9 +305,20 @@ sg_status apply_asm64(const sg_problem* pr, const Ell& A, const AsmBlocks& B, co
   return SG_OK;
 }
 
+bool solver_edge(const sg_problem* pr) {
+  return jit_eligible(pr) && (pr->jit_cfg_user[0] ? pr->jit_cfg[0].flux != 0 : pr->flux_allowed && pr->P <= 48);
+}
+
+// generated family of an FP32 apply: a solve on the slot form while the fine
+// family's own (untuned) form is the edge form has a family for it
+static int fp32_family(const sg_problem* pr, bool coarse, bool solver) {
+  if (coarse) return 1;
+  return solver && jit_config(pr, 0).flux && !solver_edge(pr) ? 6 : 0;
+}
+
 template <typename T>
 sg_status apply_any(sg_problem* pr, bool coarse, const T* X, int64_t ldx, const T* F, int64_t ldf, T* Y,
-                    int64_t ldy, cudaStream_t st) {
+                    int64_t ldy, cudaStream_t st, bool solver) {
   const Ell& A = coarse ? coarse_ell(pr) : pr->fine;
   if (sizeof(T) == 8) {
     const AsmBlocks& B = coarse ? coarse_asm(pr) : pr->asm_fine;
@@ -316,35 +327,46 @@ sg_status apply_any(sg_problem* pr, bool coarse, const T* X, int64_t ldx, const 
                          ldf, reinterpret_cast<double*>(Y), ldy, st);
   }
   if (pr->apply_mode != 1 && jit_eligible(pr)) {
-    // the edge-flux form of the fine FP32 operator when the family is configured for it
-    const bool flux = !coarse && sizeof(T) == 4 && pr->flux_on;
-    return jit_apply_launch(pr, (coarse ? 1 : 0) + (sizeof(T) == 8 ? 2 : 0), flux ? pr->flux : A, X, ldx, F, ldf, Y,
-                            ldy, st);
+    const int which = sizeof(T) == 8 ? 2 + coarse : fp32_family(pr, coarse, solver);
+    if (sizeof(T) == 4 && jit_config(pr, which).flux)
+      return jit_edge_launch<T>(pr, which, coarse ? coarse_edge(pr) : pr->edge, X, ldx, F, ldf, Y, ldy, st);
+    if (sizeof(T) == 4) SG_TRY(ell_f32(A, pr->K, st));
+    return jit_apply_launch(pr, which, A, X, ldx, F, ldf, Y, ldy, st);
   }
+  if (sizeof(T) == 4) SG_TRY(ell_f32(A, pr->K, st));
   return apply_ell<T>(A, coarse ? coarse_tri(pr) : pr->tri, pr->P, pr->K, X, ldx, F, ldf, Y, ldy, st);
 }
 
+sg_status apply_prepare32(sg_problem* pr, bool coarse, cudaStream_t st) {
+  if (pr->apply_mode != 1 && jit_eligible(pr)) {
+    const int which = fp32_family(pr, coarse, true);
+    SG_TRY(jit_apply_build(pr, which));
+    if (jit_config(pr, which).flux) return SG_OK;
+  }
+  return ell_f32(coarse ? coarse_ell(pr) : pr->fine, pr->K, st);
+}
+
 template sg_status apply_any<double>(sg_problem*, bool, const double*, int64_t, const double*, int64_t, double*,
-                                     int64_t, cudaStream_t);
+                                     int64_t, cudaStream_t, bool);
 template sg_status apply_any<float>(sg_problem*, bool, const float*, int64_t, const float*, int64_t, float*,
-                                    int64_t, cudaStream_t);
+                                    int64_t, cudaStream_t, bool);
 
 template <typename T>
 sg_status apply_op(sg_problem* pr, bool coarse, const T* X, int64_t ldx, const T* F, int64_t ldf, T* Y,
-                   int64_t ldy, cudaStream_t st) {
+                   int64_t ldy, cudaStream_t st, bool solver) {
   if (sizeof(T) == 8) SG_TRY(asm_prepare(pr, coarse ? coarse_ell(pr) : pr->fine, coarse ? coarse_asm(pr) : pr->asm_fine, st));
   size_t slot = 0;
   const bool on = pr->prof.on;
   if (on) SG_TRY(pr->prof.begin((coarse ? 2 : 0) + (sizeof(T) == 8 ? 1 : 0), st, slot));
-  SG_TRY(apply_any<T>(pr, coarse, X, ldx, F, ldf, Y, ldy, st));
+  SG_TRY(apply_any<T>(pr, coarse, X, ldx, F, ldf, Y, ldy, st, solver));
   if (on) SG_TRY(pr->prof.end(slot, st));
   return SG_OK;
 }
 
 template sg_status apply_op<double>(sg_problem*, bool, const double*, int64_t, const double*, int64_t, double*,
-                                    int64_t, cudaStream_t);
+                                    int64_t, cudaStream_t, bool);
 template sg_status apply_op<float>(sg_problem*, bool, const float*, int64_t, const float*, int64_t, float*,
-                                   int64_t, cudaStream_t);
+                                   int64_t, cudaStream_t, bool);
 
 template sg_status apply_ell<double>(const Ell&, const TripleTables&, int, int, const double*, int64_t,
                                      const double*, int64_t, double*, int64_t, cudaStream_t);

@@ -60,7 +60,7 @@ __global__ void k_cbar(const double* __restrict__ gfield, const int* __restrict_
 // Five-slot ELL values for input terms [k0, k0 + kn).  Slot order (ascending
 // column): south, west, centre, east, north.  Thread per (row, term).
 __global__ void k_fine_ell(const double* __restrict__ cb, int N, int64_t n, int64_t ldr, int k0,
-                           int kn, double* __restrict__ v64, float* __restrict__ v32) {
+                           int kn, double* __restrict__ v64) {
   const int m = N - 1;
   const int64_t E = 2LL * N * N;
   int64_t total = int64_t(kn) * n;
@@ -76,86 +76,179 @@ __global__ void k_fine_ell(const double* __restrict__ cb, int N, int64_t n, int6
     for (int s = 0; s < 5; ++s) {
       int64_t idx = (int64_t(k) * 5 + s) * ldr + r;
       v64[idx] = v[s];
-      v32[idx] = float(v[s]);
     }
   }
 }
 
-// Conductances of the edge-flux form for input terms [k0, k0 + kn): the
-// horizontal edge (i,j)-(i+1,j) (i = 0..N-1, j = 1..N-1) at (j-1) N + i,
-// half the sum of the lower triangle of cell (i,j) and the upper one of
-// cell (i,j-1); the vertical edge (i,j)-(i,j+1) (i = 1..N-1, j = 0..N-1) at
-// N (N-1) + j (N-1) + i - 1, half the sum of the upper triangle of cell
-// (i,j) and the lower one of cell (i-1,j).  A row of A_k is then the sum
-// over its four edges of w (x_r - x_neighbour) (the rows of the P1 element
-// matrices sum to zero).  Thread per (term, edge).
+// conductance of edge e of a mesh of N x N cells with the coefficient field
+// c over its triangles: the horizontal edge (i,j)-(i+1,j) (i = 0..N-1, j =
+// 1..N-1) at (j-1) N + i, half the sum of the lower triangle of cell (i,j)
+// and the upper one of cell (i,j-1); the vertical edge (i,j)-(i,j+1) (i =
+// 1..N-1, j = 0..N-1) at N (N-1) + j (N-1) + i - 1, half the sum of the
+// upper triangle of cell (i,j) and the lower one of cell (i-1,j).  A row of
+// A(c) is then the sum over its four edges of w (x_r - x_neighbour) (the
+// rows of the P1 element matrices sum to zero).
 template <typename T>
-__global__ void k_flux_values(const double* __restrict__ cb, int N, int64_t vkst, int k0, int kn,
-                              T* __restrict__ v32) {
+__device__ __forceinline__ T edge_conductance(const T* c, int N, int64_t e) {
   const int m = N - 1;
-  const int64_t E = 2LL * N * N, ne = 2LL * N * m, total = int64_t(kn) * ne;
+  auto lo = [&](int ci, int cj) { return c[2LL * (int64_t(cj) * N + ci)]; };
+  auto up = [&](int ci, int cj) { return c[2LL * (int64_t(cj) * N + ci) + 1]; };
+  if (e < int64_t(N) * m) {
+    const int i = int(e % N), j = int(e / N) + 1;
+    return T(0.5) * (lo(i, j) + up(i, j - 1));
+  }
+  const int64_t e2 = e - int64_t(N) * m;
+  const int i = int(e2 % m) + 1, j = int(e2 / m);
+  return T(0.5) * (up(i, j) + lo(i - 1, j));
+}
+
+// FP64 conductances of input terms [k0, k0 + kn), w[k * vkst + e]; thread
+// per (term, edge)
+__global__ void k_flux_values64(const double* __restrict__ cb, int N, int64_t vkst, int k0, int kn,
+                                double* __restrict__ w) {
+  const int64_t E = 2LL * N * N, ne = 2LL * N * (N - 1), total = int64_t(kn) * ne;
   for (int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; t < total;
        t += int64_t(gridDim.x) * blockDim.x) {
     const int kl = int(t / ne);
     const int64_t e = t - int64_t(kl) * ne;
+    w[int64_t(k0 + kl) * vkst + e] = edge_conductance(cb + int64_t(kl) * E, N, e);
+  }
+}
+
+// conductances of input terms [k0, k0 + kn) into the edge form's blocks
+// (EdgeVals), every position of the term; lanes without an edge get zero
+template <typename Tc>
+__global__ void k_edge_values(const Tc* __restrict__ cb, int N, int KT, const int* __restrict__ off,
+                              const int* __restrict__ pos, const double* __restrict__ scale, int k0, int kn,
+                              float* __restrict__ v32, double* __restrict__ v64) {
+  const int m = N - 1, ntile = (N + 30) / 31;
+  const int64_t E = 2LL * N * N, per = int64_t(N) * ntile * 64, total = int64_t(kn) * per;
+  for (int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; t < total;
+       t += int64_t(gridDim.x) * blockDim.x) {
+    const int kl = int(t / per);
+    const int64_t q = t - int64_t(kl) * per;  // ((j ntile + tile) 2 + vertical) 32 + lane
+    const int lane = int(q & 31), ver = int(q >> 5) & 1;
+    const int64_t b = q >> 6;
+    const int tile = int(b % ntile), j = int(b / ntile), e = 31 * tile + lane;
+    int64_t edge = -1;
+    if (ver) {
+      if (lane < 31 && e + 1 <= m) edge = int64_t(N) * m + int64_t(j) * m + e;
+    } else if (j >= 1 && e < N) {
+      edge = int64_t(j - 1) * N + e;
+    }
+    const double w = edge >= 0 ? scale[k0 + kl] * double(edge_conductance(cb + int64_t(kl) * E, N, edge)) : 0.0;
+    for (int u = off[k0 + kl]; u < off[k0 + kl + 1]; ++u) {
+      const int64_t at = (((q >> 5) * (KT / 4) + pos[u] / 4) * 32 + lane) * 4 + pos[u] % 4;
+      if (v32) v32[at] = float(w);
+      if (v64) v64[at] = w;
+    }
+  }
+}
+
+__global__ void k_round_values(const double* __restrict__ v64, float* __restrict__ v32, int64_t len) {
+  for (int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; t < len; t += int64_t(gridDim.x) * blockDim.x)
+    v32[t] = float(v64[t]);
+}
+
+// Coefficients of the triangles of the nested 2h mesh: the mean over the
+// four fine triangles inside (the gradients of the coarse basis are constant
+// on a coarse triangle, so R_0 A(c) R_0^T is the P1 stiffness of that mean).
+// Coarse cell (I, J), fine cell (i, j) = (2I, 2J): its lower triangle holds
+// lo(i, j), lo(i+1, j), up(i+1, j), lo(i+1, j+1), its upper triangle
+// up(i, j), up(i, j+1), lo(i, j+1), up(i+1, j+1).
+__global__ void k_coarse_coef(const double* __restrict__ cb, int N, int kn, double* __restrict__ out) {
+  const int Nc = N / 2;
+  const int64_t E = 2LL * N * N, Ec = 2LL * Nc * Nc, total = int64_t(kn) * Nc * Nc;
+  for (int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; t < total; t += int64_t(gridDim.x) * blockDim.x) {
+    const int kl = int(t / (int64_t(Nc) * Nc));
+    const int64_t cell = t - int64_t(kl) * Nc * Nc;
+    const int i = 2 * int(cell % Nc), j = 2 * int(cell / Nc);
     const double* c = cb + int64_t(kl) * E;
     auto lo = [&](int ci, int cj) { return c[2LL * (int64_t(cj) * N + ci)]; };
     auto up = [&](int ci, int cj) { return c[2LL * (int64_t(cj) * N + ci) + 1]; };
-    double v;
-    if (e < int64_t(N) * m) {
-      const int i = int(e % N), j = int(e / N) + 1;
-      v = 0.5 * (lo(i, j) + up(i, j - 1));
-    } else {
-      const int64_t e2 = e - int64_t(N) * m;
-      const int i = int(e2 % m) + 1, j = int(e2 / m);
-      v = 0.5 * (up(i, j) + lo(i - 1, j));
-    }
-    v32[int64_t(k0 + kl) * vkst + e] = T(v);
+    double* o = out + int64_t(kl) * Ec + 2 * cell;
+    o[0] = 0.25 * (lo(i, j) + lo(i + 1, j) + up(i + 1, j) + lo(i + 1, j + 1));
+    o[1] = 0.25 * (up(i, j) + up(i, j + 1) + lo(i, j + 1) + up(i + 1, j + 1));
   }
 }
 
 }  // namespace
 
-sg_status flux_build(sg_problem* pr) {
-  Ell& A = pr->flux;
+sg_status ell_f32(const Ell& A, int K, cudaStream_t st) {
   if (A.v32.ptr) return SG_OK;
-  const int S = 4, K = pr->K, N = pr->N, m = N - 1;
-  const int64_t n = pr->n, E = pr->E, ldr = pr->fine.ldr, ne = 2LL * N * m;
-  A.S = S;
-  A.n = n;
-  A.ldr = ldr;
-  A.vkst = round_up(ne, 64);
-  std::vector<int32_t> col(size_t(S) * ldr, -1), vidx(size_t(S) * ldr, 0);
-  for (int64_t r = 0; r < n; ++r) {
-    const int i = int(r % m) + 1, j = int(r / m) + 1;
-    col[0 * ldr + r] = int32_t(i < m ? r + 1 : -1);
-    vidx[0 * ldr + r] = int32_t(int64_t(j - 1) * N + i);
-    col[1 * ldr + r] = int32_t(i > 1 ? r - 1 : -1);
-    vidx[1 * ldr + r] = int32_t(int64_t(j - 1) * N + i - 1);
-    col[2 * ldr + r] = int32_t(j < m ? r + m : -1);
-    vidx[2 * ldr + r] = int32_t(int64_t(N) * m + int64_t(j) * m + i - 1);
-    col[3 * ldr + r] = int32_t(j > 1 ? r - m : -1);
-    vidx[3 * ldr + r] = int32_t(int64_t(N) * m + int64_t(j - 1) * m + i - 1);
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (st) SG_CUDA(cudaStreamIsCapturing(st, &cs));
+  if (cs != cudaStreamCaptureStatusNone) {
+    set_error("the FP32 slot values must exist before a capture");
+    return SG_ERR_ARG;
   }
-  SG_TRY(A.col.alloc(col.size() * 4));
-  SG_TRY(A.vidx.alloc(vidx.size() * 4));
-  SG_CUDA(cudaMemcpy(A.col.ptr, col.data(), col.size() * 4, cudaMemcpyHostToDevice));
-  SG_CUDA(cudaMemcpy(A.vidx.ptr, vidx.data(), vidx.size() * 4, cudaMemcpyHostToDevice));
+  const int64_t len = int64_t(K) * A.S * A.ldr;
   DevBuf v;
-  SG_TRY(v.alloc(size_t(K) * A.vkst * 4));
-  SG_CUDA(cudaMemset(v.ptr, 0, size_t(K) * A.vkst * 4));
-  const int KC = 32;
-  DevBuf dcb;
-  SG_TRY(dcb.alloc(size_t(KC) * E * sizeof(double)));
+  SG_TRY(v.alloc(size_t(len) * 4));
+  k_round_values<<<4 * 152, 256, 0, st>>>(A.v64.as<double>(), v.as<float>(), len);
+  note_launch();
+  SG_CUDA(cudaGetLastError());
+  SG_CUDA(cudaStreamSynchronize(st));
+  A.v32 = std::move(v);
+  return SG_OK;
+}
+
+sg_status edge_alloc(const sg_problem* pr, int N, bool f32, bool f64, EdgeVals& out) {
+  out.N = N;
+  const size_t len = size_t(N) * ((N + 30) / 31) * 64 * pr->edge_terms.KT;
+  if (f32 && !out.v32.ptr) SG_TRY(out.v32.alloc(len * sizeof(float)));
+  if (f64 && !out.v64.ptr) SG_TRY(out.v64.alloc(len * sizeof(double)));
+  return SG_OK;
+}
+
+template <typename Tc>
+sg_status edge_values(const sg_problem* pr, const Tc* coef, int k0, int kn, EdgeVals& out, cudaStream_t st) {
+  const EdgeTerms& T = pr->edge_terms;
+  k_edge_values<Tc><<<8 * 152, 256, 0, st>>>(coef, out.N, T.KT, T.off.as<int>(), T.pos.as<int>(), T.scale.as<double>(),
+                                             k0, kn, out.v32.as<float>(), out.v64.as<double>());
+  note_launch();
+  SG_CUDA(cudaGetLastError());
+  return SG_OK;
+}
+template sg_status edge_values<float>(const sg_problem*, const float*, int, int, EdgeVals&, cudaStream_t);
+template sg_status edge_values<double>(const sg_problem*, const double*, int, int, EdgeVals&, cudaStream_t);
+
+static sg_status edge_terms_build(sg_problem* pr) {
+  const std::vector<int> term = jit_edge_terms(pr);
+  std::vector<int> off(pr->K + 1, 0), pos(term.size());
+  for (int k : term)
+    if (k >= 0) ++off[k + 1];
+  for (int k = 0; k < pr->K; ++k) off[k + 1] += off[k];
+  std::vector<int> at(off.begin(), off.end() - 1);
+  for (size_t q = 0; q < term.size(); ++q)
+    if (term[q] >= 0) pos[at[term[q]]++] = int(q);
+  EdgeTerms& T = pr->edge_terms;
+  T.KT = int(term.size());
+  T.R = jit_edge_rotations(pr);
+  SG_TRY(T.off.alloc(off.size() * 4));
+  SG_TRY(T.pos.alloc(pos.size() * 4));
+  SG_CUDA(cudaMemcpy(T.off.ptr, off.data(), off.size() * 4, cudaMemcpyHostToDevice));
+  const std::vector<double> scale = jit_edge_scale(pr);
+  SG_TRY(T.scale.alloc(scale.size() * 8));
+  SG_CUDA(cudaMemcpy(T.scale.ptr, scale.data(), scale.size() * 8, cudaMemcpyHostToDevice));
+  SG_CUDA(cudaMemcpy(T.pos.ptr, pos.data(), pos.size() * 4, cudaMemcpyHostToDevice));
+  return SG_OK;
+}
+
+sg_status coarse_edge_build(sg_problem* pr, EdgeVals& out) {
+  const int K = pr->K, N = pr->N, Nc = N / 2, KC = 32;
+  SG_TRY(edge_alloc(pr, Nc, true, false, out));
+  DevBuf dcb, dcc;
+  SG_TRY(dcb.alloc(size_t(KC) * pr->E * sizeof(double)));
+  SG_TRY(dcc.alloc(size_t(KC) * 2 * Nc * Nc * sizeof(double)));
   for (int k0 = 0; k0 < K; k0 += KC) {
     const int kn = std::min(KC, K - k0);
     SG_TRY(element_coefficients(pr, k0, kn, dcb.as<double>(), nullptr));
-    k_flux_values<float><<<4 * 152, 256>>>(dcb.as<double>(), N, A.vkst, k0, kn, v.as<float>());
+    k_coarse_coef<<<4 * 152, 256>>>(dcb.as<double>(), N, kn, dcc.as<double>());
     note_launch();
-    SG_CUDA(cudaGetLastError());
+    SG_TRY(edge_values<double>(pr, dcc.as<double>(), k0, kn, out, nullptr));
   }
   SG_CUDA(cudaDeviceSynchronize());
-  A.v32 = std::move(v);
   return SG_OK;
 }
 
@@ -166,7 +259,7 @@ sg_status flux_values64(sg_problem* pr, double* w, int64_t vkst) {
   for (int k0 = 0; k0 < K; k0 += KC) {
     const int kn = std::min(KC, K - k0);
     SG_TRY(element_coefficients(pr, k0, kn, dcb.as<double>(), nullptr));
-    k_flux_values<double><<<4 * 152, 256>>>(dcb.as<double>(), N, vkst, k0, kn, w);
+    k_flux_values64<<<4 * 152, 256>>>(dcb.as<double>(), N, vkst, k0, kn, w);
     note_launch();
     SG_CUDA(cudaGetLastError());
   }
@@ -199,7 +292,12 @@ sg_status assemble_fine(sg_problem* pr) {
   SG_TRY(A.col.alloc(col.size() * sizeof(int32_t)));
   SG_CUDA(cudaMemcpy(A.col.ptr, col.data(), col.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
   SG_TRY(A.v64.alloc(size_t(K) * S * ldr * sizeof(double)));
-  SG_TRY(A.v32.alloc(size_t(K) * S * ldr * sizeof(float)));
+  // the conductances of the edge form from the same coefficients
+  const bool edges = jit_eligible(pr) && n > 0;
+  if (edges) {
+    SG_TRY(edge_terms_build(pr));
+    SG_TRY(edge_alloc(pr, N, true, false, pr->edge));
+  }
 
   const int KC = 32;
   DevBuf dcb;
@@ -207,39 +305,45 @@ sg_status assemble_fine(sg_problem* pr) {
   for (int k0 = 0; k0 < K; k0 += KC) {
     int kn = std::min(KC, K - k0);
     SG_TRY(element_coefficients(pr, k0, kn, dcb.as<double>(), nullptr));
-    k_fine_ell<<<4 * 152, 256>>>(dcb.as<double>(), N, n, ldr, k0, kn, A.v64.as<double>(),
-                                 A.v32.as<float>()); note_launch();
+    k_fine_ell<<<4 * 152, 256>>>(dcb.as<double>(), N, n, ldr, k0, kn, A.v64.as<double>());
+    note_launch();
+    if (edges) SG_TRY(edge_values<double>(pr, dcb.as<double>(), k0, kn, pr->edge, nullptr));
     SG_CUDA(cudaGetLastError());
   }
   SG_CUDA(cudaDeviceSynchronize());
   return SG_OK;
 }
 
+sg_status gfield_upload(sg_problem* pr) {
+  DevBuf& g = pr->gfield_dev;
+  if (g.ptr) return SG_OK;
+  SG_TRY(g.alloc(std::max<size_t>(1, pr->gfield.size()) * 8));
+  if (!pr->gfield.empty()) SG_CUDA(cudaMemcpy(g.ptr, pr->gfield.data(), pr->gfield.size() * 8, cudaMemcpyHostToDevice));
+  return SG_OK;
+}
+
 sg_status element_coefficients(sg_problem* pr, int k0, int kn, double* out, cudaStream_t st) {
   const int K = pr->K, L = pr->L;
-  const int64_t E = pr->E;
-  DevBuf dg, dmi, disf;
-  std::vector<double> isf(K, 1.0);
-  std::vector<int32_t> mi = pr->mi_in;
-  if (L == 0) mi.assign(1, 0);
-  for (int k = 0; k < K; ++k) {
-    double f = 1.0;
-    for (int i = 0; i < L; ++i)
-      for (int v = 2; v <= mi[size_t(k) * L + i]; ++v) f *= v;
-    isf[k] = 1.0 / std::sqrt(f);
+  if (!pr->mi_in_dev.ptr) {
+    std::vector<double> isf(K, 1.0);
+    std::vector<int32_t> mi = pr->mi_in;
+    if (L == 0) mi.assign(1, 0);
+    for (int k = 0; k < K; ++k) {
+      double f = 1.0;
+      for (int i = 0; i < L; ++i)
+        for (int v = 2; v <= mi[size_t(k) * L + i]; ++v) f *= v;
+      isf[k] = 1.0 / std::sqrt(f);
+    }
+    SG_TRY(gfield_upload(pr));
+    SG_TRY(pr->isf_dev.alloc(isf.size() * sizeof(double)));
+    SG_CUDA(cudaMemcpy(pr->isf_dev.ptr, isf.data(), isf.size() * sizeof(double), cudaMemcpyHostToDevice));
+    SG_TRY(pr->mi_in_dev.alloc(mi.size() * sizeof(int32_t)));
+    SG_CUDA(cudaMemcpy(pr->mi_in_dev.ptr, mi.data(), mi.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
   }
-  SG_TRY(dg.alloc(std::max<size_t>(1, pr->gfield.size()) * sizeof(double)));
-  if (!pr->gfield.empty())
-    SG_CUDA(cudaMemcpy(dg.ptr, pr->gfield.data(), pr->gfield.size() * sizeof(double),
-                       cudaMemcpyHostToDevice));
-  SG_TRY(dmi.alloc(mi.size() * sizeof(int32_t)));
-  SG_CUDA(cudaMemcpy(dmi.ptr, mi.data(), mi.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
-  SG_TRY(disf.alloc(isf.size() * sizeof(double)));
-  SG_CUDA(cudaMemcpy(disf.ptr, isf.data(), isf.size() * sizeof(double), cudaMemcpyHostToDevice));
-  k_cbar<<<4 * 152, 256, 0, st>>>(dg.as<double>(), dmi.as<int>(), disf.as<double>(), L, E, pr->g0, k0, kn, out);
+  k_cbar<<<4 * 152, 256, 0, st>>>(pr->gfield_dev.as<double>(), pr->mi_in_dev.as<int>(), pr->isf_dev.as<double>(), L,
+                                  pr->E, pr->g0, k0, kn, out);
   note_launch();
   SG_CUDA(cudaGetLastError());
-  SG_CUDA(cudaStreamSynchronize(st));
   return SG_OK;
 }
 

@@ -332,7 +332,7 @@ struct SolverCtx {
   }
 
   sg_status apply_fine(const T* X, T* Y, const T* F, cudaStream_t st) {
-    return apply_op<T>(pr, false, X, ld, F, ld, Y, ld, st);
+    return apply_op<T>(pr, false, X, ld, F, ld, Y, ld, st, true);
   }
   sg_status apply_coarse(const T* X, T* Y, cudaStream_t st) {
     return apply_op<T>(pr, true, X, ldc, nullptr, 0, Y, ldc, st);
@@ -375,7 +375,7 @@ struct SolverCtx {
 
   // fine apply without the profiler (Y = F - A X when F, else A X)
   sg_status apply_raw_fine(const T* X, T* Y, const T* F, cudaStream_t st) {
-    return apply_any<T>(pr, false, X, ld, F, ld, Y, ld, st);
+    return apply_any<T>(pr, false, X, ld, F, ld, Y, ld, st, true);
   }
   // iteration counters summed over solves (device): fine FGMRES, coarse GMRES
   sg_status clear_counters(cudaStream_t st) {
@@ -439,9 +439,12 @@ struct SolverCtx {
       SG_TRY(asm_prepare(pr, pc->co.ell, pc->co.asm_c, nullptr));
       SG_TRY(resid_prepare(pr, nullptr));
     }
-    if (pr->apply_mode != 1 && jit_eligible(pr)) {
-      SG_TRY(jit_apply_build(pr, sizeof(T) == 8 ? 2 : 0));
-      SG_TRY(jit_apply_build(pr, sizeof(T) == 8 ? 3 : 1));
+    if (sizeof(T) == 4) {
+      SG_TRY(apply_prepare32(pr, false, nullptr));
+      SG_TRY(apply_prepare32(pr, true, nullptr));
+    } else if (pr->apply_mode != 1 && jit_eligible(pr)) {
+      SG_TRY(jit_apply_build(pr, 2));
+      SG_TRY(jit_apply_build(pr, 3));
     }
     SG_TRY(kernel_attrs_init());
     if (pr->cnn) SG_TRY(pr->cnn->reserve(pr->P));

@@ -82,13 +82,27 @@ struct Ell {
   int64_t n = 0, ldr = 0;
   DevBuf col;      // int32 S x ldr
   DevBuf v64;      // double K x S x ldr
-  DevBuf v32;      // float  K x S x ldr
-  // edge-flux form (fine FP32 operator only): col[s * ldr + r] is the
-  // neighbour across edge s of row r or -1 (a Dirichlet node), vidx[s * ldr
-  // + r] the offset of that edge's conductance within a term's block, the
-  // conductances of term k at v32[k * vkst + vidx]
-  DevBuf vidx;     // int32 S x ldr
-  int64_t vkst = 0;
+  mutable DevBuf v32;  // float  K x S x ldr, rounded from v64 on first use (ell_f32)
+};
+
+// The same family in the edge form: one conductance per edge of a mesh of
+// N x N cells, in the order the generated kernel reads them.  Tile t of a
+// node row j holds the horizontal edges (e, j)-(e + 1, j), e = 31 t + lane,
+// of its 32 lanes (the last one again in the next tile) and the vertical
+// edges (e + 1, j)-(e + 1, j + 1) above them, every position kk of the
+// kernel's order of input terms (EdgeTerms):
+//     v[((((j ntile + t) 2 + vertical) KT / 4 + kk / 4) 32 + lane) 4 + kk % 4],  ntile = ceil(N / 31),
+// KT a multiple of 4, the values scaled as the kernel wants them (EdgeTerms).
+struct EdgeVals {
+  int N = 0;
+  DevBuf v32, v64;  // v64: nonlinear operators only
+};
+// Where the conductances of input term k go: positions pos[off[k]] ..
+// pos[off[k + 1] - 1] of KT.
+struct EdgeTerms {
+  int KT = 0, R = 1;  // positions; turns of the kernel's loop over orbits (KT / R positions each)
+  DevBuf off, pos;        // int32 K + 1, KT
+  DevBuf scale;           // double K: factor of the stored conductances
 };
 
 // The Galerkin operator summed per stencil edge into its P x P block (FP64),
@@ -173,10 +187,14 @@ struct ProfScope {
 };
 
 // Register-specialised apply compiled at setup time (sg_jit.cpp).  Four
-// families: which = 0 fine FP32, 1 coarse FP32, 2 fine FP64, 3 coarse FP64.
+// families: which = 0 fine FP32, 1 coarse FP32, 2 fine FP64, 3 coarse FP64,
+// and of the library's own: 4 and 5, the nonlinear operators in FP32 and FP64
+// (edge form), 6 the fine FP32 operator of solves in the slot form
+// (solver_edge).
 constexpr int kJitFamilies = 4;
+constexpr int kJitAllFamilies = 7;
 constexpr int kJitMaxP = 128;
-constexpr int kJitGeneratorVersion = 10;  // bump when the generated code changes
+constexpr int kJitGeneratorVersion = 11;  // bump when the generated code changes
 constexpr int64_t kJitMaxT = 40000;
 struct JitConfig {
   int rows = 1;        // rows per thread (2: paired FP32 FMA)
@@ -190,8 +208,9 @@ struct JitConfig {
   int cgroups = 1;     // output groups as separate 128-thread CTAs (no register cap from wide CTAs)
   int warps = 4;       // warps per group (rows per group = 32 x warps x rows): narrow groups keep
                        // several slot or input groups within one register-rich CTA
-  int flux = 0;        // 1: edge-flux form (fine FP32 family): y_r = sum over the four edges of
-                       // sum_k w_k G_k (x_r - x_neighbour), conductances stored once per edge
+  int flux = 0;        // 1: edge form (FP32 families): each edge's flux sum_k w_k G_k (x_hi - x_lo)
+                       // formed once, conductances stored once per edge
+  int strip = 4;       // edge form: node rows a lane marches over
 };
 struct JitApply {
   cudaLibrary_t lib = nullptr;
@@ -222,17 +241,19 @@ struct sg_problem {
   sg::SolverState* solver = nullptr;   // preconditioner + solver workspaces
   sg::Cnn* cnn = nullptr;              // learned smoother network
   sg::NewtonWork* nl = nullptr;        // nonlinear problem: coefficients, operators, triple lists
-  sg::DevBuf gfield_dev;               // KL modes at the element centroids (sampled solves)
+  sg::DevBuf gfield_dev;               // KL modes at the element centroids
+  sg::DevBuf mi_in_dev, isf_dev;       // input multi-indices, 1 / sqrt(k!) (element_coefficients)
   sg::Profiler prof;
-  sg::JitApply* jit[sg::kJitFamilies] = {};     // specialised apply per family (fine/coarse x f32/f64)
-  sg::JitConfig jit_cfg[sg::kJitFamilies];
-  bool jit_cfg_set[sg::kJitFamilies] = {};
+  sg::JitApply* jit[sg::kJitAllFamilies] = {};     // specialised apply per family (fine/coarse x f32/f64)
+  sg::JitConfig jit_cfg[sg::kJitAllFamilies];
+  bool jit_cfg_set[sg::kJitAllFamilies] = {};
+  bool jit_cfg_user[sg::kJitAllFamilies] = {};  // configured or tuned by the program
   sg::DevBuf mdot_partial, mdot_counter;  // scratch of sg_mdot
   int apply_mode = 0;                  // 0 auto, 1 shared-memory kernel, 2 specialised
   sg::AsmBlocks asm_fine;              // assembled FP64 blocks of the fine operator
-  sg::Ell flux;                        // edge-flux form of the fine operator (FP32 conductances)
-  int flux_on = 0;                     // fine FP32 applies use the edge-flux form
-  bool flux_allowed = true;            // the autotuner may choose the edge-flux form
+  sg::EdgeVals edge;                   // edge form of the fine operator (FP32 conductances)
+  sg::EdgeTerms edge_terms;            // order of the input terms in the edge form
+  bool flux_allowed = true;            // fine FP32 applies may use the edge form
   int wait_limit = 1 << 22;            // mbarrier polls of a tcgen05 completion wait
   int asm_mode = 0;                    // FP64 applies: 0 auto, 1 never assembled, 2 always
   sg::FluxDf fdf;                      // double-FP32 edge blocks of the fine operator
@@ -248,21 +269,41 @@ sg_status build_host(sg_problem* pr, const sg_kl_desc* kl);
 // device assembly (sg_assemble.cu)
 sg_status assemble_fine(sg_problem* pr);
 // lognormal input coefficients c_bar_k(e) of terms [k0, k0 + kn) at every
-// element, written as out[(k - k0) E + e] (FP64 device array); synchronous
+// element, written as out[(k - k0) E + e] (FP64 device array) on `st`; the
+// field modes and index tables go to the device on the first call
+sg_status gfield_upload(sg_problem* pr);
 sg_status element_coefficients(sg_problem* pr, int k0, int kn, double* out, cudaStream_t st);
-// edge-flux form of the fine operator: neighbours, offsets and the FP32
-// conductances of every input term on every edge (allocated on first use)
-sg_status flux_build(sg_problem* pr);
 // the edge conductances of every input term in FP64, w[k * vkst + e] (the
-// edge numbering of the edge-flux form); synchronous
+// edge numbering of EdgeVals); synchronous
 sg_status flux_values64(sg_problem* pr, double* w, int64_t vkst);
+// FP32 conductances of the coarse operator R_0 A_k R_0^T on the nested 2h
+// mesh (its triangles carry the mean of the four fine triangles inside);
+// synchronous
+sg_status coarse_edge_build(sg_problem* pr, EdgeVals& out);
+// storage of the edge form on a mesh of N x N cells (either precision), and
+// its values from coefficients [kn][2 N^2] over the triangles of that mesh,
+// input terms [k0, k0 + kn); v32 and v64 where allocated
+sg_status edge_alloc(const sg_problem* pr, int N, bool f32, bool f64, EdgeVals& out);
+template <typename Tc>
+sg_status edge_values(const sg_problem* pr, const Tc* coef, int k0, int kn, EdgeVals& out, cudaStream_t st);
+// the FP32 five- or seven-slot values of an ELL family (rounded from the
+// FP64 ones on first use; synchronous then, never while `st` is capturing)
+sg_status ell_f32(const Ell& A, int K, cudaStream_t st);
 sg_status build_triple_tables(sg_problem* pr, TripleTables& t, int S);
 // apply (sg_apply.cu)
 template <typename T>
 sg_status apply_ell(const Ell& A, const TripleTables& tri, int P, int K, const T* X, int64_t ldx,
                     const T* F, int64_t ldf, T* Y, int64_t ldy, cudaStream_t st);
 std::string jit_apply_source(const sg_problem* pr, const JitConfig& c, bool fp64 = false);
+std::string jit_edge_source(const sg_problem* pr, const JitConfig& c, bool fp64);
 JitConfig jit_default_config(const sg_problem* pr, int which);
+// turns of the edge form's loop, and the input term at each position of its
+// conductance blocks
+int jit_edge_rotations(const sg_problem* pr);
+std::vector<int> jit_edge_terms(const sg_problem* pr);  // -1: padding
+std::vector<double> jit_edge_scale(const sg_problem* pr);
+// the configuration in use (or to be used) by one family
+JitConfig jit_config(const sg_problem* pr, int which);
 size_t jit_smem_bytes(const sg_problem* pr, const JitConfig& c, bool fp64 = false);
 sg_status jit_autotune(sg_problem* pr, int which, int force, double* best_ms);
 sg_status jit_apply_build(sg_problem* pr, int which);
@@ -273,6 +314,22 @@ sg_status jit_apply_launch(sg_problem* pr, int which, const Ell& A, const double
                            int64_t ldf, double* Y, int64_t ldy, cudaStream_t st);
 sg_status jit_apply_launch(sg_problem* pr, int which, const Ell& A, const float* X, int64_t ldx, const float* F,
                            int64_t ldf, float* Y, int64_t ldy, cudaStream_t st);
+// the same over the edge form (the family's configuration has flux = 1)
+template <typename T>
+sg_status jit_edge_launch(sg_problem* pr, int which, const EdgeVals& A, const T* X, int64_t ldx, const T* F,
+                          int64_t ldf, T* Y, int64_t ldy, cudaStream_t st);
+// Whether FP32 solves run on the edge form: what the program configured or
+// tuned for the fine family, else P <= 48.  Above that the five-slot form
+// was the default, and a mixed solve that stops at a relative residual of
+// 1e-8 carries the rounding error of its FP32 operator: 1.1e-9 of the
+// solution at 384^2, P = 70 (2e-11 in the edge form; below 2e-11 in either
+// form up to P = 35), so a change of form there would move the returned
+// solutions by more than their FP64 results may move.  The edge form is
+// several times faster (345 us against 2.1 ms an apply): sg_apply_flux(prob,
+// 1) selects it.
+bool solver_edge(const sg_problem* pr);
+// FP32 values the applies of a solve need, built before any capture
+sg_status apply_prepare32(sg_problem* pr, bool coarse, cudaStream_t st);
 // assembled FP64 blocks (sg_apply.cu): build per the problem's policy (no-op
 // once tried; never while `st` is capturing), and the apply over them
 sg_status asm_prepare(sg_problem* pr, const Ell& A, AsmBlocks& B, cudaStream_t st);
@@ -290,14 +347,15 @@ sg_status refine_residual(sg_problem* pr, const double* F, int64_t ldf, const do
                           int64_t ldr, cudaStream_t st);
 sg_status apply_asm64(const sg_problem* pr, const Ell& A, const AsmBlocks& B, const double* X, int64_t ldx,
                       const double* F, int64_t ldf, double* Y, int64_t ldy, cudaStream_t st);
+// (solver: the form FP32 solves use, solver_edge)
 // the operator apply without timing: assembled blocks (FP64, when built),
 // else the specialised kernel, else the shared-memory kernel
 template <typename T>
 sg_status apply_any(sg_problem* pr, bool coarse, const T* X, int64_t ldx, const T* F, int64_t ldf, T* Y,
-                    int64_t ldy, cudaStream_t st);
+                    int64_t ldy, cudaStream_t st, bool solver = false);
 // apply_ell on the fine (coarse = false) or coarse family of a problem,
 // timed when the problem's profiler is on
 template <typename T>
 sg_status apply_op(sg_problem* pr, bool coarse, const T* X, int64_t ldx, const T* F, int64_t ldf, T* Y,
-                   int64_t ldy, cudaStream_t st);
+                   int64_t ldy, cudaStream_t st, bool solver = false);
 }  // namespace sg

@@ -38,6 +38,7 @@ struct NewtonWork {
   DevBuf coef64, dcoef64, dcoef32;   // [K][E]: ctil(U); dctil of a Jacobian apply
   Ell op;                            // A(U): values of sum_j A(ctil_j) (FP64 and FP32)
   Ell dop;                           // A(dctil), the Jacobian's derivative part
+  EdgeVals eop, edop;                // the same in the edge form (where the specialised kernel runs)
   DevBuf ppp_off, ppp_ab, ppp_m64, ppp_m32;  // <psi_a psi_b psi_f> by rows f
   DevBuf kfj_off, kfj_kf, kfj_m64, kfj_m32;  // <psi_k psi_f psi_j> by rows j (k | f << 16)
   DevBuf u64, u32, f64, r64, r32, d32, d64, tmp32, tmp64, one, scal;
@@ -177,14 +178,12 @@ sg_status upload(DevBuf& d, const void* src, size_t bytes) {
   return SG_OK;
 }
 
-sg_status ell_like(const Ell& src, Ell& dst, bool v64, bool v32, int K) {
+sg_status ell_like(const Ell& src, Ell& dst) {
   dst.S = src.S;
   dst.n = src.n;
   dst.ldr = src.ldr;
   SG_TRY(dst.col.alloc(src.col.bytes));
   SG_CUDA(cudaMemcpy(dst.col.ptr, src.col.ptr, src.col.bytes, cudaMemcpyDeviceToDevice));
-  if (v64) SG_TRY(dst.v64.alloc(size_t(K) * src.S * src.ldr * 8));
-  if (v32) SG_TRY(dst.v32.alloc(size_t(K) * src.S * src.ldr * 4));
   return SG_OK;
 }
 
@@ -274,8 +273,8 @@ sg_status newton_prepare(sg_problem* pr) {
   SG_CUDA(cudaGetLastError());
   SG_TRY(w->coef64.alloc(size_t(KE) * 8));
   SG_TRY(w->dcoef32.alloc(size_t(KE) * 4));
-  SG_TRY(ell_like(pr->fine, w->op, true, true, K));
-  SG_TRY(ell_like(pr->fine, w->dop, false, true, K));
+  SG_TRY(ell_like(pr->fine, w->op));
+  SG_TRY(ell_like(pr->fine, w->dop));
   const size_t len = size_t(P) * pr->ld;
   for (DevBuf* b : {&w->u64, &w->f64, &w->r64, &w->d64, &w->tmp64}) SG_TRY(b->alloc(len * 8));
   for (DevBuf* b : {&w->u32, &w->r32, &w->d32, &w->tmp32}) SG_TRY(b->alloc(len * 4));
@@ -306,8 +305,22 @@ sg_status nl_coef(sg_problem* pr, const T* U, const T* dU, const T* base, T* out
   return SG_OK;
 }
 
+// the nonlinear operators run on the generated kernels over the edge form
+// (2.5 times fewer values to write and read than five slots), else on the
+// shared-memory kernel over five-slot values
+bool nl_edge(const sg_problem* pr) { return pr->apply_mode != 1 && jit_eligible(pr); }
+
+// values of sum_j A(coef_j): A in five slots or E in the edge form, in FP32
+// and / or FP64 (allocated on first use)
 template <typename Tc>
-sg_status nl_ell(sg_problem* pr, const Tc* coef, Ell& A, cudaStream_t st) {
+sg_status nl_values(sg_problem* pr, const Tc* coef, Ell& A, EdgeVals& E, bool f32, bool f64, cudaStream_t st) {
+  if (nl_edge(pr)) {
+    SG_TRY(edge_alloc(pr, pr->N, f32, f64, E));
+    return edge_values<Tc>(pr, coef, 0, pr->K, E, st);
+  }
+  const size_t len = size_t(pr->K) * A.S * A.ldr;
+  if (f64 && !A.v64.ptr) SG_TRY(A.v64.alloc(len * 8));
+  if (f32 && !A.v32.ptr) SG_TRY(A.v32.alloc(len * 4));
   const int64_t total = int64_t(pr->K) * pr->n;
   k_nl_ell<Tc><<<grid_len(total), 256, 0, st>>>(coef, pr->N, pr->n, A.ldr, pr->K, dp<double>(A.v64),
                                                  dp<float>(A.v32));
@@ -319,12 +332,9 @@ sg_status nl_ell(sg_problem* pr, const Tc* coef, Ell& A, cudaStream_t st) {
 // Y = F - A X (F given) or A X with the values of A (same pattern and
 // triples as the linear operator)
 template <typename T>
-sg_status nl_apply(sg_problem* pr, const Ell& A, const T* X, const T* F, T* Y, cudaStream_t st) {
+sg_status nl_apply(sg_problem* pr, const Ell& A, const EdgeVals& E, const T* X, const T* F, T* Y, cudaStream_t st) {
   const int64_t ld = pr->ld;
-  // the fine FP32 family may be generated for the edge-flux storage, which
-  // these per-step value arrays do not have: the shared-memory kernel then
-  if (pr->apply_mode != 1 && jit_eligible(pr) && !(sizeof(T) == 4 && pr->flux_on))
-    return jit_apply_launch(pr, sizeof(T) == 8 ? 2 : 0, A, X, ld, F, ld, Y, ld, st);
+  if (nl_edge(pr)) return jit_edge_launch<T>(pr, sizeof(T) == 8 ? 5 : 4, E, X, ld, F, ld, Y, ld, st);
   return apply_ell<T>(A, pr->tri, pr->P, pr->K, X, ld, F, ld, Y, ld, st);
 }
 
@@ -332,7 +342,7 @@ sg_status nl_apply(sg_problem* pr, const Ell& A, const T* X, const T* F, T* Y, c
 sg_status nl_operator(sg_problem* pr, const double* U64, cudaStream_t st) {
   NewtonWork& w = *pr->nl;
   SG_TRY(nl_coef<double>(pr, U64, nullptr, dp<double>(w.cbar64), dp<double>(w.coef64), st));
-  return nl_ell<double>(pr, dp<double>(w.coef64), w.op, st);
+  return nl_values<double>(pr, dp<double>(w.coef64), w.op, w.eop, true, true, st);
 }
 
 // Y = J(U) X = A(U) X + A(dctil(U; X)) U, with A(U) already in w.op and U
@@ -344,16 +354,15 @@ sg_status nl_jacobian(sg_problem* pr, const T* U, const T* X, T* Y, cudaStream_t
   T* dcoef = sizeof(T) == 8 ? reinterpret_cast<T*>(w.dcoef64.ptr) : reinterpret_cast<T*>(w.dcoef32.ptr);
   T* tmp = sizeof(T) == 8 ? reinterpret_cast<T*>(w.tmp64.ptr) : reinterpret_cast<T*>(w.tmp32.ptr);
   SG_TRY(nl_coef<T>(pr, U, X, nullptr, dcoef, st));
-  SG_TRY(nl_ell<T>(pr, dcoef, w.dop, st));
-  SG_TRY(nl_apply<T>(pr, w.op, X, nullptr, Y, st));
-  SG_TRY(nl_apply<T>(pr, w.dop, U, nullptr, tmp, st));
+  SG_TRY(nl_values<T>(pr, dcoef, w.dop, w.edop, sizeof(T) == 4, sizeof(T) == 8, st));
+  SG_TRY(nl_apply<T>(pr, w.op, w.eop, X, nullptr, Y, st));
+  SG_TRY(nl_apply<T>(pr, w.dop, w.edop, U, nullptr, tmp, st));
   return vec_axpy_multi<T>(tmp, 0, 1, dp<double>(w.one), Y, len, st);
 }
 
 sg_status ensure_fp64_jacobian(sg_problem* pr) {
   NewtonWork& w = *pr->nl;
   if (!w.dcoef64.ptr) SG_TRY(w.dcoef64.alloc(size_t(w.K) * w.E * 8));
-  if (!w.dop.v64.ptr) SG_TRY(w.dop.v64.alloc(size_t(w.K) * w.dop.S * w.dop.ldr * 8));
   return SG_OK;
 }
 
@@ -433,7 +442,7 @@ sg_status newton_impl(sg_problem* pr, double* X, int64_t ldx, double tol_update,
   for (int it = 0; it < max_newton && nF > 0.0; ++it) {
     // R = F - A(U) U in FP64
     SG_TRY(nl_operator(pr, U, st));
-    SG_TRY(nl_apply<double>(pr, w.op, U, F, R, st));
+    SG_TRY(nl_apply<double>(pr, w.op, w.eop, U, F, R, st));
     double nR = 0.0;
     SG_TRY(norm_host(pr, R, len, nR, st, c64));
     if (!std::isfinite(nR)) {
@@ -493,7 +502,7 @@ sg_status newton_impl(sg_problem* pr, double* X, int64_t ldx, double tol_update,
   double nR = 0.0;
   if (nF > 0.0) {
     SG_TRY(nl_operator(pr, U, st));
-    SG_TRY(nl_apply<double>(pr, w.op, U, F, R, st));
+    SG_TRY(nl_apply<double>(pr, w.op, w.eop, U, F, R, st));
     SG_TRY(norm_host(pr, R, len, nR, st, c64));
   } else {
     SG_CUDA(cudaMemsetAsync(U, 0, len * 8, st));
@@ -558,7 +567,7 @@ sg_status sg_nonlinear_residual(sg_problem* pr, const double* F, int64_t ldf, co
   SG_TRY(load_rhs(pr, F, ldf, dp<double>(w.f64), st));
   SG_TRY(load_block<double>(pr, X, ldx, dp<double>(w.u64), st));
   SG_TRY(nl_operator(pr, dp<double>(w.u64), st));
-  SG_TRY(nl_apply<double>(pr, w.op, dp<double>(w.u64), dp<double>(w.f64), dp<double>(w.r64), st));
+  SG_TRY(nl_apply<double>(pr, w.op, w.eop, dp<double>(w.u64), dp<double>(w.f64), dp<double>(w.r64), st));
   SG_CUDA(cudaMemcpy2DAsync(R, ldr * 8, w.r64.ptr, pr->ld * 8, pr->n * 8, pr->P, cudaMemcpyDeviceToDevice, st));
   return SG_OK;
 }

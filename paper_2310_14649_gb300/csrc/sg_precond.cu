@@ -498,7 +498,7 @@ __global__ void __launch_bounds__(128) k_node_transform_reg(float* __restrict__ 
 // Coarse ELL values of all K terms from the fine ELL values by the RAP plan.
 __global__ void k_coarse_values(const double* __restrict__ fine, int64_t fine_kstride, const int* __restrict__ rp,
                                 const int64_t* __restrict__ src, const double* __restrict__ w, int64_t npos,
-                                int K, double* __restrict__ v64, float* __restrict__ v32) {
+                                int K, double* __restrict__ v64) {
   int64_t total = npos * K;
   for (int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; t < total; t += int64_t(gridDim.x) * blockDim.x) {
     int k = int(t / npos);
@@ -507,7 +507,6 @@ __global__ void k_coarse_values(const double* __restrict__ fine, int64_t fine_ks
     double acc = 0.0;
     for (int u = rp[q]; u < rp[q + 1]; ++u) acc += w[u] * fk[src[u]];
     v64[t] = acc;
-    v32[t] = float(acc);
   }
 }
 
@@ -1002,13 +1001,13 @@ sg_status precond_setup_coarse_plan(sg_problem* pr, Precond& pc, const CoarsePla
     SG_CUDA(cudaMemcpy(w.ptr, plan.w.data(), plan.w.size() * 8, cudaMemcpyHostToDevice));
   }
   SG_TRY(C.ell.v64.alloc(size_t(K) * npos * 8));
-  SG_TRY(C.ell.v32.alloc(size_t(K) * npos * 4));
   k_coarse_values<<<4 * 152, 256>>>(pr->fine.v64.as<double>(), int64_t(pr->fine.S) * pr->fine.ldr, rp.as<int>(),
-                                    src.as<int64_t>(), w.as<double>(), npos, K, C.ell.v64.as<double>(),
-                                    C.ell.v32.as<float>()); note_launch();
+                                    src.as<int64_t>(), w.as<double>(), npos, K, C.ell.v64.as<double>());
+  note_launch();
   SG_CUDA(cudaGetLastError());
   SG_CUDA(cudaDeviceSynchronize());
   SG_TRY(build_triple_tables(pr, C.tri, S));
+  if (jit_eligible(pr)) SG_TRY(coarse_edge_build(pr, C.edge));
   return SG_OK;
 }
 

@@ -331,11 +331,8 @@ extern "C" sg_status sg_sample_solve(sg_problem* pr, const double* xi, int64_t S
          "sg_sample_solve: the mesh is too large for one CTA per sample (N <= 102)");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   // the KL modes at the element centroids, once per problem
-  DevBuf& g = pr->gfield_dev;
-  if (!g.ptr) {
-    SG_TRY(g.alloc(pr->gfield.size() * 8));
-    SG_CUDA(cudaMemcpy(g.ptr, pr->gfield.data(), pr->gfield.size() * 8, cudaMemcpyHostToDevice));
-  }
+  SG_TRY(gfield_upload(pr));
+  const DevBuf& g = pr->gfield_dev;
   DevBuf itsd;
   SG_TRY(itsd.alloc(sizeof(int)));
   SG_CUDA(cudaMemsetAsync(itsd.ptr, 0, sizeof(int), st));

@@ -14,6 +14,7 @@ namespace sg {
 
 const Ell& coarse_ell(const sg_problem* pr) { return pr->solver->pc.co.ell; }
 const TripleTables& coarse_tri(const sg_problem* pr) { return pr->solver->pc.co.tri; }
+const EdgeVals& coarse_edge(const sg_problem* pr) { return pr->solver->pc.co.edge; }
 AsmBlocks& coarse_asm(sg_problem* pr) { return pr->solver->pc.co.asm_c; }
 
 // Recorded graphs (the coarse-solve graphs of the solver contexts) hold the

@@ -74,6 +74,7 @@ struct CoarseData {
   int64_t nc = 0, ldc = 0;
   std::vector<int32_t> rowptr, colidx;     // coarse CSR pattern (host)
   Ell ell;                                 // coarse A_k in ELL form (device)
+  EdgeVals edge;                           // the same in the edge form (FP32 conductances)
   TripleTables tri;
   DevCsr RT, R;                            // interpolation (n x nc) and restriction
   AsmBlocks asm_c;                         // assembled FP64 blocks of the coarse operator
@@ -131,6 +132,7 @@ sg_status precond_setup_host(sg_problem* pr, Precond& pc);
 sg_status amg_setup_fine(const sg_problem* pr, AmgHier& h);
 const Ell& coarse_ell(const sg_problem* pr);
 const TripleTables& coarse_tri(const sg_problem* pr);
+const EdgeVals& coarse_edge(const sg_problem* pr);
 AsmBlocks& coarse_asm(sg_problem* pr);
 // drops the solver contexts and their recorded graphs after a change of
 // apply kernel (recorded batches of the problem then refuse to run)

@@ -392,3 +392,64 @@ def check_flux(prob, ref, X):
     bound, m = flux_bound(ref, X)
     assert np.all(np.abs(Y - Yr) <= gamma(m, U32) * bound + 1e-30)
     assert np.linalg.norm(Y - Yr) <= 1e-5 * np.linalg.norm(Yr)
+
+
+@pytest.mark.parametrize("N,L,p,q", [(2, 2, 2, 4), (3, 4, 3, 6), (31, 3, 3, 6), (32, 4, 3, 6), (33, 3, 4, 8), (63, 2, 4, 8),
+                                     (62, 1, 6, 12), (24, 5, 3, 6), (22, 4, 4, 8), (16, 6, 3, 6), (9, 5, 4, 4),
+                                     (17, 3, 3, 2), (9, 0, 0, 0)])
+def test_edge_form_tiles_and_rotations(gpu, N, L, p, q):
+    """The edge form at the edges of its 31-node tiles, with strips of one
+    and more rows marched up and down, one to six turns of the orbit loop
+    (L / R shifts of 1 to 6 variables, orbits shorter than R included), two
+    output groups (P = 126), fewer input than output terms, ragged leading
+    dimensions, and as a residual in place; against the oracle within the
+    rounding bound of the form."""
+    import torch
+    import paper_2310_14649_gb300 as sg
+    prob, ref = setup_pair(N, L, p, q)
+    assert sg.sg_apply_flux(prob, -1) == 1                    # the default
+    X = random_block(ref.n, ref.P, seed=91).astype(np.float32).astype(np.float64)
+    check_flux(prob, ref, X)
+    F = random_block(ref.n, ref.P, seed=92).astype(np.float32).astype(np.float64)
+    Xd, Fd = to_dev(X, torch.float32, ref.n + 5), to_dev(F, torch.float32, ref.n + 2)
+    sg.sg_residual(prob, Fd, Xd, Fd)
+    torch.cuda.synchronize()
+    bound, m = flux_bound(ref, X)
+    err = np.abs(from_dev(Fd, ref.n) - (F - galerkin.apply(ref, X)))
+    assert np.all(err <= gamma(m + 1, U32) * (bound + np.abs(F)) + 1e-30)
+    prob.close()
+
+
+def test_edge_form_nan_stays_local(gpu):
+    """A NaN at one node reaches that node and the ends of its four edges,
+    and nothing else."""
+    import torch
+    import paper_2310_14649_gb300 as sg
+    N = 40
+    prob = sg.sg_setup(N, 2, 2, 4)
+    X = torch.zeros((prob.P, prob.n), dtype=torch.float32, device="cuda")
+    m = N - 1
+    r = 20 * m + 30                                           # lane 30 of its tile: the shuffle's end
+    X[0, r] = float("nan")
+    Y = torch.zeros_like(X)
+    sg.sg_apply(prob, X, Y)
+    hit = torch.isnan(Y).any(0).nonzero()[:, 0].tolist()
+    assert hit == sorted([r - m, r - 1, r, r + 1, r + m])
+    prob.close()
+
+
+def test_solves_above_48_modes_keep_the_slot_form(gpu):
+    """At P > 48 an untuned mixed solve returns the five-slot operator's
+    solution bit for bit while sg_apply runs the edge form; sg_apply_flux(1)
+    moves the solve to the edge form."""
+    import torch
+    import paper_2310_14649_gb300 as sg
+    prob = sg.sg_setup(24, 5, 3, 6)
+    sg.sg_precond_setup(prob, 2, 2, 1, inner_rtol=0.5)
+    X = [torch.zeros((prob.P, prob.n), dtype=torch.float64, device="cuda") for _ in range(3)]
+    for x, mode in zip(X, (2, 0, 1)):
+        assert sg.sg_apply_flux(prob, mode) == (mode != 0)
+        sg.sg_solve(prob, x, rtol=1e-9, mode=1)
+    assert torch.equal(X[0], X[1])
+    assert not torch.equal(X[0], X[2]) and (X[0] - X[2]).norm() <= 1e-7 * X[0].norm()
+    prob.close()
