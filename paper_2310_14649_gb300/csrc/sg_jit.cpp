@@ -850,8 +850,9 @@ static sg_status jit_compile(const std::string& src, cudaLibrary_t* lib, cudaKer
 // else is resident, and a warp's time is its 2 strip + 1 edge visits, so the
 // strip with the fewest rounds x visits (measured: 23.7 to 24.6 us per round
 // and visit at 384^2, P = 70 for strips of 1 to 4, 6.8 to 7.3 us at 256^2, P
-// = 35).  Long strips lose: 27 us at 6 rows.  FP64: the SM's FP64 units run
-// one warp's work at a time, so single-warp CTAs, one an SM to a round.
+// = 35).  Long strips lose: 27 us at 6 rows.  FP64 takes the same
+// rule (single-warp CTAs, one an SM to a round: 0.67 instead of 0.58 ms at
+// 128^2, P = 35 with the nonlinear problem's full chaos).
 static JitConfig edge_default(const sg_problem* pr, int N, bool fp64) {
   JitConfig c;
   c.flux = 1;
@@ -859,14 +860,14 @@ static JitConfig edge_default(const sg_problem* pr, int N, bool fp64) {
   c.cgroups = std::min(16, std::max(1, (2 * pr->P * words + 219) / 220));
   c.prefetch = 32;
   c.stages = 3;
-  c.warps = fp64 ? 1 : 4;
+  c.warps = 4;
+  while (c.warps > 1 && jit_smem_bytes(pr, c, fp64) > 200 * 1024) c.warps /= 2;
   c.min_blocks = words * pr->P <= 42 ? 4 : words * pr->P <= 60 ? 3 : 2;
   const int64_t tiles = (N + 30) / 31;
   int64_t best = 0;
   for (int strip = 1; strip <= 4; ++strip) {
     const int64_t ctas = ((N - 1 + strip - 1) / strip * tiles + c.warps - 1) / c.warps * c.cgroups;
-    const int64_t at_once = fp64 ? 152 : 2 * 152;
-    const int64_t cost = (ctas + at_once - 1) / at_once * (2 * strip + 1);
+    const int64_t cost = (ctas + 2 * 152 - 1) / (2 * 152) * (2 * strip + 1);
     if (strip == 1 || cost < best) {
       best = cost;
       c.strip = strip;
