@@ -338,7 +338,11 @@ struct SolverCtx {
     return apply_op<T>(pr, true, X, ldc, nullptr, 0, Y, ldc, st);
   }
   // AMG V-cycle per mode on a coarse block
+  bool folded() const { return sizeof(T) == 4 && pc->amg.fold.ready; }
   sg_status amg(const T* B, T* X, cudaStream_t st) {
+    if constexpr (sizeof(T) == 4)
+      if (folded())
+        return amg_fold_apply(pc->amg, aw, pr->P, B, ldc, nullptr, 0, X, ldc, nullptr, nullptr, 0, st);
     const AmgLevel& L0 = pc->amg[0];
     SG_CUDA(cudaMemcpy2DAsync(aw.b[0], L0.ld * sizeof(T), B, ldc * sizeof(T), pc->co.nc * sizeof(T), pr->P,
                               cudaMemcpyDeviceToDevice, st));
@@ -347,7 +351,12 @@ struct SolverCtx {
   // coarse preconditioner on a block already in the AMG level-0 input:
   // V-cycle, copy out to `out` (coarse ld), Kronecker factor
   // (with Zs: the result also into slot dg.iv[0] of Zs, slot stride lenc)
+  // (folded V-cycle: the input is read from slot dg.iv[0] of V instead)
   sg_status coarse_pc_from_b0(T* out, cudaStream_t st, T* Zs = nullptr) {
+    if constexpr (sizeof(T) == 4)
+      if (folded())
+        return amg_fold_apply(pc->amg, aw, pr->P, dp<T>(coarse.V), ldc, dg.iv, lenc, out, ldc, dp<T>(pc->gkron32), Zs,
+                              lenc, st);
     SG_TRY(amg_vcycle<T>(pc->amg, aw, pr->P, st, out, ldc));
     return node_transform<T>(out, ldc, pc->co.nc, pr->P, dp_sel<T>(pc->gkron64, pc->gkron32), st, Zs, lenc,
                              Zs ? dg.iv : nullptr);

@@ -65,7 +65,10 @@ sg_status capture_coarse(SolverCtx<T>& c, cudaStream_t s1, cudaStream_t s2, cuda
       SG_TRY(dg_axpy_norm<T>(V, lenc, h2, w, lenc, W.s.scal, part, cnt, jdev, s3));
     }
     SG_TRY(dg_givens(c.dg, W.s, m, hin, s3));
-    SG_TRY(dg_scale_next<T>(w, V, lenc, lenc, c.dg, W.s.scal + 1, s3, c.aw.b[0], L0.ld, ldc, pc.co.nc));
+    if (c.folded())
+      SG_TRY(dg_scale_next<T>(w, V, lenc, lenc, c.dg, W.s.scal + 1, s3));
+    else
+      SG_TRY(dg_scale_next<T>(w, V, lenc, lenc, c.dg, W.s.scal + 1, s3, c.aw.b[0], L0.ld, ldc, pc.co.nc));
     SG_CUDA(cudaStreamEndCapture(s3, &body_in));
     return SG_OK;
   };
@@ -76,7 +79,8 @@ sg_status capture_coarse(SolverCtx<T>& c, cudaStream_t s1, cudaStream_t s2, cuda
     SG_CUDA(cudaGraphConditionalHandleCreate(&hin, gc, 0, 0));
     SG_TRY(dg_start(c.dg, W.s, m, W.s.scal + 3, hin, sc));
     SG_TRY(vec_scale_by<T>(V, V, lenc, W.s.scal + 3, true, sc));
-    SG_TRY(dg_copy_vj<T>(V, lenc, ldc, c.aw.b[0], L0.ld, pc.co.nc, c.pr->P, c.dg, sc));  // b_0 = V_0
+    if (!c.folded())
+      SG_TRY(dg_copy_vj<T>(V, lenc, ldc, c.aw.b[0], L0.ld, pc.co.nc, c.pr->P, c.dg, sc));  // b_0 = V_0
     cudaGraph_t body_in;
     SG_TRY(SolverCtx<T>::add_while(sc, hin, &body_in));
     const int64_t a = launch_count();

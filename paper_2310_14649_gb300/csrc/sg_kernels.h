@@ -34,7 +34,16 @@ sg_status ras_inverse_apply(const Precond& pc, int P, const float* R, int64_t ld
                             bool transform, int wait_limit, cudaStream_t st);
 sg_status ras_inverse_check(const Precond& pc, cudaStream_t st);
 template <typename T>
-sg_status amg_vcycle(const AmgHier& H, AmgWork<T>& w, int P, cudaStream_t st, T* out = nullptr, int64_t ldo = 0);
+// one V-cycle from a zero guess on w.b[l0], levels l0 and below
+sg_status amg_vcycle(const AmgHier& H, AmgWork<T>& w, int P, cudaStream_t st, T* out = nullptr, int64_t ldo = 0,
+                     int l0 = 0);
+// the folded FP32 V-cycle (H.fold.ready) of b (leading dimension ldb; with j
+// the block *j of an array of blocks, bstride apart) into out; with M, out <-
+// M out per node, and with Z2 also into slot *j of Z2 (slot stride stride2,
+// leading dimension ldo)
+sg_status amg_fold_apply(const AmgHier& H, AmgWork<float>& w, int P, const float* b, int64_t ldb, const int* j,
+                         int64_t bstride, float* out, int64_t ldo, const float* M, float* Z2, int64_t stride2,
+                         cudaStream_t st);
 sg_status frobenius_weights(sg_problem* pr, std::vector<double>& w);
 // sets the dynamic shared-memory limits of the library's kernels once per
 // process (before any graph capture)

@@ -613,6 +613,8 @@ struct AmgPhase {
   T* Y = nullptr;         // t (kDown, kResid), b_{l+1}, x (kProlong, +=), out (kFinal)
   int64_t ldy = 0;
   T* Y2 = nullptr;        // kDown: x = D^{-1} b (ld ldy)
+  const int* j = nullptr; // kRestrict: the gathered vector is block *j of X, xstride apart
+  int64_t xstride = 0;
 };
 
 // MB modes per thread group: the row's pattern and values are read once
@@ -625,6 +627,7 @@ __global__ void __launch_bounds__(128) k_amg_phase(const __grid_constant__ AmgPh
   const int64_t a0 = int64_t(blockIdx.y) * MB;
   const int nm = int(min(int64_t(MB), int64_t(p.P) - a0));
   const bool live = i < p.n;
+  const T* X0 = OP == kRestrict && p.j ? p.X + int64_t(*p.j) * p.xstride : p.X;
   T acc[MB];
 #pragma unroll
   for (int m = 0; m < MB; ++m) acc[m] = T(0);
@@ -638,7 +641,7 @@ __global__ void __launch_bounds__(128) k_amg_phase(const __grid_constant__ AmgPh
 #pragma unroll
       for (int m = 0; m < MB; ++m) {
         if (m < nm) {
-          const T* X = p.X + (a0 + m) * p.ldx;
+          const T* X = X0 + (a0 + m) * p.ldx;
           T g;
           if (OP == kDown)
             g = dj * X[j];
@@ -869,13 +872,13 @@ sg_status node_transform(T* Z, int64_t ld, int64_t n, int P, const T* M, cudaStr
 // Level buffers: b (rhs), x (solution), t (temporary), each [P][ld_l].
 // The result goes to `out` (ld `ldo`), or to x_0 when out is NULL.
 template <typename T>
-sg_status amg_vcycle(const AmgHier& H, AmgWork<T>& w, int P, cudaStream_t st, T* out, int64_t ldo) {
+sg_status amg_vcycle(const AmgHier& H, AmgWork<T>& w, int P, cudaStream_t st, T* out, int64_t ldo, int l0) {
   const int nl = int(H.size());
   if (!out) {
-    out = w.x[0];
-    ldo = H[0].ld;
+    out = w.x[l0];
+    ldo = H[l0].ld;
   }
-  if (H.fused && nl >= 2 && P > 0) {
+  if (H.fused && nl - l0 >= 2 && P > 0) {
     auto lanes = [P](const DevCsr& M) {
       // about two entries per lane on an average row, while rows x modes x
       // lanes stays within about two waves of resident threads (152 SMs x 2048)
@@ -894,7 +897,7 @@ sg_status amg_vcycle(const AmgHier& H, AmgWork<T>& w, int P, cudaStream_t st, T*
       p.v = dv<T>(M.v64, M.v32);
       return p;
     };
-    for (int l = 0; l < nl - 1; ++l) {
+    for (int l = l0; l < nl - 1; ++l) {
       const AmgLevel& L = H[l];
       AmgPhase<T> p = phase(L.A);
       p.X = w.b[l];
@@ -920,7 +923,7 @@ sg_status amg_vcycle(const AmgHier& H, AmgWork<T>& w, int P, cudaStream_t st, T*
                                                w.x[nl - 1], L.ld); note_launch();
       SG_CUDA(cudaGetLastError());
     }
-    for (int l = nl - 2; l >= 0; --l) {
+    for (int l = nl - 2; l >= l0; --l) {
       const AmgLevel& L = H[l];
       const AmgLevel& Ln = H[l + 1];
       AmgPhase<T> p = phase(L.Pm);
@@ -939,7 +942,7 @@ sg_status amg_vcycle(const AmgHier& H, AmgWork<T>& w, int P, cudaStream_t st, T*
       q.B = w.b[l];
       q.ldb = L.ld;
       q.d = dv<T>(L.dinv64, L.dinv32);
-      if (l > 0 || out == w.x[0]) {
+      if (l > l0 || out == w.x[l0]) {
         q.Y = w.t[l];
         q.ldy = L.ld;
         SG_CUDA((amg_phase_launch<T, kResid>(q, st)));
@@ -949,16 +952,16 @@ sg_status amg_vcycle(const AmgHier& H, AmgWork<T>& w, int P, cudaStream_t st, T*
         SG_CUDA((amg_phase_launch<T, kFinal>(q, st)));
       }
     }
-    if (out == w.x[0]) {
+    if (out == w.x[l0]) {
       // in place: the last smoothing step on its own
-      const AmgLevel& L0 = H[0];
+      const AmgLevel& L0 = H[l0];
       dim3 g(unsigned((L0.n + 127) / 128), unsigned(P));
-      k_diag<T><<<g, 128, 0, st>>>(L0.n, dv<T>(L0.dinv64, L0.dinv32), w.t[0], L0.ld, w.x[0], L0.ld, 1); note_launch();
+      k_diag<T><<<g, 128, 0, st>>>(L0.n, dv<T>(L0.dinv64, L0.dinv32), w.t[l0], L0.ld, w.x[l0], L0.ld, 1); note_launch();
       SG_CUDA(cudaGetLastError());
     }
     return SG_OK;
   }
-  for (int l = 0; l < nl - 1; ++l) {
+  for (int l = l0; l < nl - 1; ++l) {
     const AmgLevel& L = H[l];
     dim3 g(unsigned((L.n + 127) / 128), unsigned(P));
     k_diag<T><<<g, 128, 0, st>>>(L.n, dv<T>(L.dinv64, L.dinv32), w.b[l], L.ld, w.x[l], L.ld, 0); note_launch();
@@ -973,7 +976,7 @@ sg_status amg_vcycle(const AmgHier& H, AmgWork<T>& w, int P, cudaStream_t st, T*
                                         L.ld); note_launch();
     SG_CUDA(cudaGetLastError());
   }
-  for (int l = nl - 2; l >= 0; --l) {
+  for (int l = nl - 2; l >= l0; --l) {
     const AmgLevel& L = H[l];
     dim3 g(unsigned((L.n + 127) / 128), unsigned(P));
     SG_TRY(spmm<T>(L.Pm, w.x[l + 1], H[l + 1].ld, nullptr, 0, w.x[l], L.ld, P, 1, st));
@@ -981,9 +984,313 @@ sg_status amg_vcycle(const AmgHier& H, AmgWork<T>& w, int P, cudaStream_t st, T*
     k_diag<T><<<g, 128, 0, st>>>(L.n, dv<T>(L.dinv64, L.dinv32), w.t[l], L.ld, w.x[l], L.ld, 1); note_launch();
     SG_CUDA(cudaGetLastError());
   }
-  if (out != w.x[0])
-    SG_CUDA(cudaMemcpy2DAsync(out, ldo * sizeof(T), w.x[0], H[0].ld * sizeof(T), H[0].n * sizeof(T), P,
+  if (out != w.x[l0])
+    SG_CUDA(cudaMemcpy2DAsync(out, ldo * sizeof(T), w.x[l0], H[l0].ld * sizeof(T), H[l0].n * sizeof(T), P,
                               cudaMemcpyDeviceToDevice, st));
+  return SG_OK;
+}
+
+// ---------------------------------------------------------------------------
+// Folded FP32 V-cycle (AmgFold).  A cycle of four levels took 13 launches of
+// 4.5 to 14 us, bound by launch latency and short dependent loads; folded it
+// takes three (down, dense, up), and in the recorded coarse solves the copy of
+// the input and the Kronecker factor, two launches more, are part of the
+// first and the last.  256^2, P = 35 (16,129 coarse unknowns): 83 us of
+// kernels a cycle, now 34 (9.2 + 6.8 + 17.8); a coarse solve at tolerance
+// 1e-5 3.02 ms, now 2.58.
+// ---------------------------------------------------------------------------
+namespace {
+
+constexpr int kDenseRows = 64, kDenseSplit = 8, kDenseModes = 48, kDenseLd = 52;
+
+// X = B b for the dense part: a cluster of eight CTAs per 64 rows and 48
+// modes, each a slice of the sum (its matrix and vector slices brought to
+// shared memory in one round of 16-byte copies), the partial sums added over
+// the cluster in rank order through distributed shared memory.  At n = 1,849
+// the matrix is 13.7 MB, read once from L2.  b, x: mode-major.
+__global__ void __cluster_dims__(kDenseSplit, 1, 1) __launch_bounds__(128)
+    k_fold_dense(int n, int64_t ldd, const float* __restrict__ B, const float* __restrict__ b, int64_t ldb, int P,
+                 float* __restrict__ x, int64_t ldx, int slice) {
+  extern __shared__ __align__(16) float sm_fold[];
+  float* Bs = sm_fold;                       // [slice][64]
+  float* bs = Bs + slice * kDenseRows;       // [slice][52]: a mode's store along k meets 8 banks
+  const int rank = blockIdx.x, row0 = blockIdx.y * kDenseRows, a0 = blockIdx.z * kDenseModes;
+  const int k0 = rank * slice, kn = max(0, min(slice, n - k0)), nm = min(kDenseModes, P - a0);
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  for (int q = tid; q < kn * (kDenseRows / 4); q += 128) {
+    const int k = q / (kDenseRows / 4), c = q % (kDenseRows / 4);
+    // columns row0 .. row0 + 63 of row k (the matrix is symmetric; ldd covers whole tiles)
+    cp_async16(Bs + k * kDenseRows + 4 * c, B + int64_t(k0 + k) * ldd + row0 + 4 * c);
+  }
+  for (int k = tid; k < kn; k += 128)
+    for (int m = 0; m < kDenseModes; ++m) {
+      float* dst = bs + k * kDenseLd + m;
+      if (m < nm)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(
+                         static_cast<uint32_t>(__cvta_generic_to_shared(dst))),
+                     "l"(b + int64_t(a0 + m) * ldb + k0 + k)
+                     : "memory");
+      else
+        *dst = 0.f;
+    }
+  cp_async_commit();
+  cp_async_wait_all();
+  __syncthreads();
+  // thread: rows 2 lane, 2 lane + 1, modes 12 w .. 12 w + 11
+  float acc[2][12];
+#pragma unroll
+  for (int m = 0; m < 12; ++m) acc[0][m] = acc[1][m] = 0.f;
+#pragma unroll 4
+  for (int k = 0; k < kn; ++k) {
+    const float2 r = *reinterpret_cast<const float2*>(Bs + k * kDenseRows + 2 * lane);
+    const float4* v = reinterpret_cast<const float4*>(bs + k * kDenseLd + 12 * w);
+#pragma unroll
+    for (int u = 0; u < 3; ++u) {
+      const float4 t = v[u];
+      const float e[4] = {t.x, t.y, t.z, t.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        acc[0][4 * u + i] = fmaf(r.x, e[i], acc[0][4 * u + i]);
+        acc[1][4 * u + i] = fmaf(r.y, e[i], acc[1][4 * u + i]);
+      }
+    }
+  }
+  __syncthreads();
+  float* part = sm_fold;                     // [48][64]
+#pragma unroll
+  for (int m = 0; m < 12; ++m)
+    *reinterpret_cast<float2*>(part + (12 * w + m) * kDenseRows + 2 * lane) = make_float2(acc[0][m], acc[1][m]);
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+  // this CTA sums modes 6 rank .. 6 rank + 5 over the cluster
+  const uint32_t base = static_cast<uint32_t>(__cvta_generic_to_shared(part));
+  for (int q = tid; q < (kDenseModes / kDenseSplit) * kDenseRows; q += 128) {
+    const int m = rank * (kDenseModes / kDenseSplit) + q / kDenseRows, r = q % kDenseRows;
+    float s = 0.f;
+#pragma unroll
+    for (int c = 0; c < kDenseSplit; ++c) {
+      uint32_t addr;
+      float v;
+      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(addr) : "r"(base + 4u * (m * kDenseRows + r)), "r"(c));
+      asm volatile("ld.shared::cluster.f32 %0, [%1];\n" : "=f"(v) : "r"(addr) : "memory");
+      s += v;
+    }
+    if (m < nm && row0 + r < n) x[int64_t(a0 + m) * ldx + row0 + r] = s;
+  }
+  // no CTA leaves while another reads its partial sums
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+}
+
+struct FoldUp {
+  int n = 0, P = 0;
+  const int *rpS = nullptr, *ciS = nullptr, *rpP = nullptr, *ciP = nullptr;
+  const float *vS = nullptr, *vP = nullptr;
+  const float* b = nullptr;   // right-hand side of the level (block *j when j)
+  int64_t ldb = 0, bstride = 0;
+  const float* xc = nullptr;  // solution of the next level
+  int64_t ldc = 0;
+  const float* M = nullptr;   // P x P factor per node, or NULL
+  float* out = nullptr;
+  int64_t ldo = 0;
+  float* Z2 = nullptr;        // also into slot *j
+  int64_t stride2 = 0;
+  const int* j = nullptr;
+};
+
+// x = S b + P' x_c and, with M, x <- M x per node: lanes hold 32 rows, each of
+// up to four warps MW modes, so a row's pattern and values are read once per
+// warp for MW gathers; the 32 nodes' vectors meet in shared memory for the
+// factor
+template <int MW>
+__global__ void __launch_bounds__(128) k_fold_up(const __grid_constant__ FoldUp p) {
+  extern __shared__ __align__(16) float sm_up[];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, a0 = w * MW;
+  const int r = blockIdx.x * 32 + lane;
+  const bool live = r < p.n;
+  const int64_t j = p.j ? *p.j : 0;
+  const float* b = p.b + (p.bstride ? j * p.bstride : 0);
+  float* Ms = sm_up;                     // [P][4 MW]: column b of M, outputs along
+  float* zs = Ms + p.P * 4 * MW;         // [P][32]
+  if (p.M)
+    for (int e = threadIdx.x; e < p.P * 4 * MW; e += blockDim.x) {
+      const int c = e / (4 * MW), a = e - c * 4 * MW;
+      Ms[e] = a < p.P ? p.M[a * p.P + c] : 0.f;
+    }
+  float acc[MW];
+#pragma unroll
+  for (int m = 0; m < MW; ++m) acc[m] = 0.f;
+  if (live) {
+    const int e1 = p.rpS[r + 1];
+    for (int e = p.rpS[r]; e < e1; ++e) {
+      const int c = p.ciS[e];
+      const float v = p.vS[e];
+#pragma unroll
+      for (int m = 0; m < MW; ++m)
+        if (a0 + m < p.P) acc[m] = fmaf(v, b[int64_t(a0 + m) * p.ldb + c], acc[m]);
+    }
+    const int f1 = p.rpP[r + 1];
+    for (int e = p.rpP[r]; e < f1; ++e) {
+      const int c = p.ciP[e];
+      const float v = p.vP[e];
+#pragma unroll
+      for (int m = 0; m < MW; ++m)
+        if (a0 + m < p.P) acc[m] = fmaf(v, p.xc[int64_t(a0 + m) * p.ldc + c], acc[m]);
+    }
+  }
+  if (p.M) {
+#pragma unroll
+    for (int m = 0; m < MW; ++m)
+      if (a0 + m < p.P) zs[(a0 + m) * 32 + lane] = acc[m];
+    __syncthreads();
+#pragma unroll
+    for (int m = 0; m < MW; ++m) acc[m] = 0.f;
+    for (int c = 0; c < p.P; ++c) {
+      const float z = zs[c * 32 + lane];
+      const float4* row = reinterpret_cast<const float4*>(Ms + c * 4 * MW + a0);
+#pragma unroll
+      for (int u = 0; u < MW / 4; ++u) {
+        const float4 t = row[u];
+        acc[4 * u] = fmaf(t.x, z, acc[4 * u]);
+        acc[4 * u + 1] = fmaf(t.y, z, acc[4 * u + 1]);
+        acc[4 * u + 2] = fmaf(t.z, z, acc[4 * u + 2]);
+        acc[4 * u + 3] = fmaf(t.w, z, acc[4 * u + 3]);
+      }
+    }
+  }
+  if (!live) return;
+  float* z2 = p.Z2 ? p.Z2 + j * p.stride2 : nullptr;
+#pragma unroll
+  for (int m = 0; m < MW; ++m)
+    if (a0 + m < p.P) {
+      p.out[int64_t(a0 + m) * p.ldo + r] = acc[m];
+      if (z2) z2[int64_t(a0 + m) * p.ldo + r] = acc[m];
+    }
+}
+
+__global__ void k_fold_round(const double* __restrict__ x, int64_t ldx, int n, float* __restrict__ B, int64_t ldd) {
+  const int c = blockIdx.x * blockDim.x + threadIdx.x, r = blockIdx.y;
+  if (c < n) B[int64_t(r) * ldd + c] = float(x[int64_t(r) * ldx + c]);
+}
+__global__ void k_fold_units(double* __restrict__ b, int64_t ld, int n) {
+  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c < n) b[int64_t(c) * ld + c] = 1.0;
+}
+
+int fold_slice(int64_t n) { return int(round_up((n + kDenseSplit - 1) / kDenseSplit, 4)); }
+size_t fold_dense_smem(int64_t n) {
+  const size_t s = size_t(fold_slice(n)) * (kDenseRows + kDenseLd), part = size_t(kDenseModes) * kDenseRows;
+  return std::max(s, part) * sizeof(float);
+}
+
+template <int MW>
+sg_status fold_up_launch(const FoldUp& p, cudaStream_t st) {
+  const size_t smem = p.M ? (size_t(p.P) * 4 * MW + size_t(p.P) * 32) * sizeof(float) : 0;
+  k_fold_up<MW><<<unsigned((p.n + 31) / 32), unsigned(32 * ((p.P + MW - 1) / MW)), smem, st>>>(p);
+  note_launch();
+  SG_CUDA(cudaGetLastError());
+  return SG_OK;
+}
+
+}  // namespace
+
+sg_status fold_attrs_init() {
+  SG_CUDA(cudaFuncSetAttribute(k_fold_dense, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               int(fold_dense_smem(kFoldMax))));
+  SG_CUDA(cudaFuncSetAttribute(k_fold_up<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024));
+  return SG_OK;
+}
+
+sg_status amg_fold_dense(AmgHier& H) {
+  AmgFold& F = H.fold;
+  const int n = int(H[F.lf].n), nl = int(H.size());
+  // the FP64 cycle of levels lf and below on the n unit vectors
+  AmgWork<double> w;
+  std::vector<DevBuf> buf(3 * nl);
+  w.b.assign(nl, nullptr);
+  w.x.assign(nl, nullptr);
+  w.t.assign(nl, nullptr);
+  for (int l = F.lf; l < nl; ++l) {
+    for (int q = 0; q < 3; ++q) SG_TRY(buf[3 * l + q].alloc(size_t(n) * H[l].ld * 8));
+    w.b[l] = buf[3 * l].as<double>();
+    w.x[l] = buf[3 * l + 1].as<double>();
+    w.t[l] = buf[3 * l + 2].as<double>();
+  }
+  const int64_t ld = H[F.lf].ld;
+  k_fold_units<<<unsigned((n + 127) / 128), 128>>>(w.b[F.lf], ld, n);
+  note_launch();
+  SG_TRY(amg_vcycle<double>(H, w, n, nullptr, nullptr, 0, F.lf));
+  F.ldd = round_up(n, kDenseRows);
+  SG_TRY(F.dense.alloc(size_t(n) * F.ldd * 4));
+  k_fold_round<<<dim3(unsigned((n + 127) / 128), unsigned(n)), 128>>>(w.x[F.lf], ld, n, F.dense.as<float>(), F.ldd);
+  note_launch();
+  SG_CUDA(cudaGetLastError());
+  SG_CUDA(cudaDeviceSynchronize());
+  F.ready = true;
+  return SG_OK;
+}
+
+sg_status amg_fold_apply(const AmgHier& H, AmgWork<float>& w, int P, const float* b, int64_t ldb, const int* j,
+                         int64_t bstride, float* out, int64_t ldo, const float* M, float* Z2, int64_t stride2,
+                         cudaStream_t st) {
+  const AmgFold& F = H.fold;
+  for (int l = 0; l < F.lf; ++l) {
+    const DevCsr& R = F.Rp[l];
+    const int64_t avg = R.n > 0 ? (R.nnz + R.n - 1) / R.n : 1;
+    int G = 1;
+    while (G < 32 && 2 * G < avg && R.n * int64_t(P) * (2 * G) <= 2 * 152 * 2048) G <<= 1;
+    AmgPhase<float> p;
+    p.n = int(R.n);
+    p.P = P;
+    p.G = G;
+    p.rp = R.rowptr.as<int>();
+    p.ci = R.col.as<int>();
+    p.v = R.v32.as<float>();
+    p.X = l ? w.b[l] : b;
+    p.ldx = l ? H[l].ld : ldb;
+    p.j = l ? nullptr : j;
+    p.xstride = bstride;
+    p.Y = w.b[l + 1];
+    p.ldy = H[l + 1].ld;
+    SG_CUDA((amg_phase_launch<float, kRestrict>(p, st)));
+  }
+  {
+    const AmgLevel& L = H[F.lf];
+    const int n = int(L.n);
+    const dim3 grid(kDenseSplit, unsigned((n + kDenseRows - 1) / kDenseRows), unsigned((P + kDenseModes - 1) / kDenseModes));
+    k_fold_dense<<<grid, 128, fold_dense_smem(n), st>>>(n, F.ldd, F.dense.as<float>(), w.b[F.lf], L.ld, P, w.x[F.lf],
+                                                        L.ld, fold_slice(n));
+    note_launch();
+    SG_CUDA(cudaGetLastError());
+  }
+  for (int l = F.lf - 1; l >= 0; --l) {
+    FoldUp p;
+    p.n = int(H[l].n);
+    p.P = P;
+    p.rpS = F.S[l].rowptr.as<int>();
+    p.ciS = F.S[l].col.as<int>();
+    p.vS = F.S[l].v32.as<float>();
+    p.rpP = F.Pp[l].rowptr.as<int>();
+    p.ciP = F.Pp[l].col.as<int>();
+    p.vP = F.Pp[l].v32.as<float>();
+    p.b = l ? w.b[l] : b;
+    p.ldb = l ? H[l].ld : ldb;
+    p.xc = w.x[l + 1];
+    p.ldc = H[l + 1].ld;
+    p.out = l ? w.x[l] : out;
+    p.ldo = l ? H[l].ld : ldo;
+    if (l == 0) {
+      p.bstride = j ? bstride : 0;
+      p.j = j;
+      p.M = M;
+      p.Z2 = Z2;
+      p.stride2 = stride2;
+    }
+    if (P <= 16)
+      SG_TRY(fold_up_launch<4>(p, st));
+    else if (P <= 48)
+      SG_TRY(fold_up_launch<12>(p, st));
+    else
+      SG_TRY(fold_up_launch<32>(p, st));
+  }
   return SG_OK;
 }
 
@@ -1021,6 +1328,7 @@ sg_status kernel_attrs_init() {
   SG_CUDA(cudaFuncSetAttribute(k_node_transform<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
   SG_CUDA(cudaFuncSetAttribute(k_node_transform<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
   SG_TRY(apply_attrs_init());
+  SG_TRY(fold_attrs_init());
   done = true;
   return SG_OK;
 }
@@ -1042,7 +1350,7 @@ sg_status frobenius_weights(sg_problem* pr, std::vector<double>& w) {
   template sg_status ras_apply<T>(const Precond&, int64_t, int, const T*, int64_t, T*, cudaStream_t, bool,        \
                                   Profiler*);                                                                      \
   template sg_status node_transform<T>(T*, int64_t, int64_t, int, const T*, cudaStream_t, T*, int64_t, const int*);                \
-  template sg_status amg_vcycle<T>(const AmgHier&, AmgWork<T>&, int, cudaStream_t, T*, int64_t);
+  template sg_status amg_vcycle<T>(const AmgHier&, AmgWork<T>&, int, cudaStream_t, T*, int64_t, int);
 INST(float)
 INST(double)
 #undef INST

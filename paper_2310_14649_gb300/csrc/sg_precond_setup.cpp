@@ -472,8 +472,9 @@ static int32_t aggregate(const HCsr& A, std::vector<int32_t>& agg) {
   return na;
 }
 
-static sg_status setup_amg(AmgHier& H, const HCsr& A0c) {
+static sg_status setup_amg(AmgHier& H, const HCsr& A0c, bool fold) {
   H.lev.clear();
+  H.fold = AmgFold();
   HCsr A = A0c;
   std::vector<HCsr> As, Ps;
   std::vector<std::vector<int32_t>> aggs;
@@ -586,7 +587,44 @@ static sg_status setup_amg(AmgHier& H, const HCsr& A0c) {
     }
   SG_TRY(H.coarsest_inv64.alloc(inv.size() * 8));
   SG_CUDA(cudaMemcpy(H.coarsest_inv64.ptr, inv.data(), inv.size() * 8, cudaMemcpyHostToDevice));
-  return SG_OK;
+  if (!fold || As.size() < 2) return SG_OK;
+  AmgFold& F = H.fold;
+  F.lf = 1;
+  while (As[F.lf].n > kFoldMax && F.lf + 1 < int(As.size())) ++F.lf;
+  if (As[F.lf].n > kFoldMax) return SG_OK;  // the coarsening stalled: no dense part
+  F.Rp.resize(F.lf);
+  F.Pp.resize(F.lf);
+  F.S.resize(F.lf);
+  for (int l = 0; l < F.lf; ++l) {
+    const HCsr& A = As[l];
+    std::vector<double> di(A.n, 0.0);
+    for (int64_t i = 0; i < A.n; ++i) {
+      for (int32_t t = A.rp[i]; t < A.rp[i + 1]; ++t) di[i] += std::fabs(A.v[t]);
+      di[i] = 1.0 / di[i];
+    }
+    // P' = P - D^{-1} A P on the pattern of A P (it holds P's: the diagonal of A is nonzero)
+    HCsr Pf = matmul(A, Ps[l]);
+    for (int64_t i = 0; i < A.n; ++i) {
+      int32_t u = Ps[l].rp[i];
+      for (int32_t t = Pf.rp[i]; t < Pf.rp[i + 1]; ++t) {
+        Pf.v[t] *= -di[i];
+        if (u < Ps[l].rp[i + 1] && Ps[l].ci[u] == Pf.ci[t]) Pf.v[t] += Ps[l].v[u++];
+      }
+      if (u != Ps[l].rp[i + 1]) {
+        set_error("AMG setup: a prolongator entry outside A P");
+        return SG_ERR_ARG;
+      }
+    }
+    HCsr Sf = A;
+    for (int64_t i = 0; i < A.n; ++i)
+      for (int32_t t = A.rp[i]; t < A.rp[i + 1]; ++t)
+        Sf.v[t] = (A.ci[t] == i ? 2.0 * di[i] : 0.0) - di[i] * A.v[t] * di[A.ci[t]];
+    const HCsr Rf = transpose(Pf);
+    SG_TRY(F.Rp[l].upload(Rf.n, Rf.m, Rf.rp, Rf.ci, Rf.v));
+    SG_TRY(F.Pp[l].upload(Pf.n, Pf.m, Pf.rp, Pf.ci, Pf.v));
+    SG_TRY(F.S[l].upload(Sf.n, Sf.m, Sf.rp, Sf.ci, Sf.v));
+  }
+  return amg_fold_dense(H);
 }
 
 sg_status amg_setup_fine(const sg_problem* pr, AmgHier& h) {
@@ -596,7 +634,7 @@ sg_status amg_setup_fine(const sg_problem* pr, AmgHier& h) {
   A.rp = pr->rowptr;
   A.ci = pr->colidx;
   A.v = pr->a0;
-  return setup_amg(h, A);
+  return setup_amg(h, A, false);
 }
 
 sg_status precond_setup_host(sg_problem* pr, Precond& pc) {
@@ -604,7 +642,7 @@ sg_status precond_setup_host(sg_problem* pr, Precond& pc) {
   CoarsePlan plan;
   HCsr Ac0;
   SG_TRY(setup_coarse(pr, pc, plan, Ac0));
-  SG_TRY(setup_amg(pc.amg, Ac0));
+  SG_TRY(setup_amg(pc.amg, Ac0, pc.amg_fold));
   SG_TRY(precond_setup_coarse_plan(pr, pc, plan));
   return SG_OK;
 }

@@ -28,11 +28,29 @@ struct AmgLevel {
   std::vector<int32_t> agg;
 };
 
+// The FP32 V-cycle with its Jacobi steps multiplied into the transfers and
+// everything from level `lf` down as one dense matrix.  From a zero guess
+// the cycle of level l is the linear map
+//     b_{l+1} = R' b_l,  x_l = S b_l + P' x_{l+1},
+//     P' = (I - D^{-1} A) P,  R' = P'^T,  S = 2 D^{-1} - D^{-1} A D^{-1}
+// (A symmetric), so a level costs two launches instead of four and the
+// levels from the first with at most kFoldMax unknowns one dense product.
+constexpr int kFoldMax = 2048;
+constexpr int kFoldModes = 128;  // modes of the kernel with the Kronecker factor
+struct AmgFold {
+  bool ready = false;
+  int lf = 0;                       // first level of the dense part
+  std::vector<DevCsr> Rp, Pp, S;    // levels 0 .. lf - 1
+  DevBuf dense;                     // float n_lf x ldd, symmetric
+  int64_t ldd = 0;
+};
+
 // Smoothed-aggregation hierarchy: levels plus the explicit FP64 inverse of
 // the coarsest matrix.
 struct AmgHier {
   std::vector<AmgLevel> lev;
   DevBuf coarsest_inv64;
+  AmgFold fold;
   bool fused = true;  // V-cycle: lane groups per sparse row, Jacobi steps folded into the products
   size_t size() const { return lev.size(); }
   AmgLevel& operator[](size_t l) { return lev[l]; }
@@ -115,6 +133,7 @@ struct Precond {
   Harvest harvest;
   int inner_its_last = 0, inner_its_total = 0, inner_calls = 0;
   bool device_loops = true;                // coarse GMRES as one CUDA graph launch
+  bool amg_fold = false;                   // build the folded FP32 V-cycle
   int last_coarse_dtype = -1;              // 0 FP64, 1 FP32: context of the last graph solve
 };
 
@@ -127,6 +146,9 @@ struct CoarsePlan {
 };
 
 sg_status precond_setup_host(sg_problem* pr, Precond& pc);
+// the dense part of a folded hierarchy, from the FP64 V-cycle applied to the
+// unit vectors of level lf; synchronous
+sg_status amg_fold_dense(AmgHier& H);
 // smoothed-aggregation hierarchy of the fine mean matrix A_0 (training
 // targets of the learned smoother)
 sg_status amg_setup_fine(const sg_problem* pr, AmgHier& h);

@@ -376,3 +376,43 @@ def test_ras_explicit_inverses_wide_modes(gpu, L, p):
         assert np.max(np.abs(Y - Yr)) <= 1e-4 * np.max(np.abs(Yr))
     finally:
         prob.close()
+
+
+@pytest.mark.parametrize("N,L,p,flux", [
+    (34, 3, 1, False),    # 256 unknowns: one dense level, nothing to fold
+    (66, 5, 1, False),    # 1,024 unknowns; 6 modes
+    (96, 3, 3, False),    # 20 modes
+    (130, 4, 3, False),   # 35 modes, ragged last rows of the dense part
+    (66, 3, 5, False),    # 56 modes: the phase kernels
+    (66, 4, 4, True),     # 70 modes, the wide kernel and two mode tiles
+    (400, 1, 1, False),   # two sparse levels above the dense part
+])
+def test_amg_fold(gpu, N, L, p, flux):
+    """The folded FP32 V-cycle against the FP64 V-cycle.  Its longest sum has
+    n / 8 + 8 terms, n <= 2,048, with at most 56 more roundings around it, of
+    terms that the cycle of |b| bounds (the cycle of an M-matrix is a
+    nonnegative map up to its smoothed prolongator; factor 2)."""
+    import torch
+    import paper_2310_14649_gb300 as sg
+    prob = sg.sg_setup(N, L, p, min(2 * p, 8), sigma2=0.3, bx=0.5, by=0.5)
+    if flux:
+        sg.sg_apply_flux(prob, 1)
+    boxes = max(3, N // 24)
+    sg.sg_precond_setup(prob, boxes, boxes, 1, inner_rtol=0.1)
+    nc, P = (N // 2 - 1) ** 2, prob.P
+    B = random_block(nc, P, seed=36).astype(np.float32).astype(np.float64)
+    Y64, _ = run(prob, sg.PC_AMG, B, nc, torch.float64)
+    S64, _ = run(prob, sg.PC_AMG, np.abs(B), nc, torch.float64)
+    Y32, _ = run(prob, sg.PC_AMG, B, nc, torch.float32)
+    tol = 2 * (min(nc, 2048) / 8 + 64) * 2.0 ** -24
+    assert np.max(np.abs(Y32 - Y64)) <= tol * np.max(np.abs(S64))
+    # inside the coarse solver, with the factor per node: as many iterations
+    # and the same solution as with one kernel per level operation
+    X, it = {}, {}
+    for kernel in (0, 1):
+        sg.sg_precond_setup(prob, boxes, boxes, 1, inner_rtol=0.1, amg_kernel=kernel)
+        X[kernel] = torch.zeros((P, prob.n), dtype=torch.float64, device="cuda")
+        info = sg.sg_solve(prob, X[kernel], rtol=1e-8, mode=1)
+        it[kernel] = (info["outer_it"], info["inner_it"])
+    assert abs(it[0][0] - it[1][0]) <= 1 and abs(it[0][1] - it[1][1]) <= 2 + it[1][1] // 20, it
+    assert ((X[0] - X[1]).norm() / X[1].norm()).item() <= 1e-6
