@@ -88,53 +88,188 @@ __global__ void __launch_bounds__(256) k_apply_tile(ApplyArgs<T> p) {
 }
 
 // ---------------------------------------------------------------------------
-// Assembled FP64 apply.  The generated FP64 kernel spends two FP64
-// operations per triple and slot (2,395 triples at P = 35), and GB300's FP64
-// units (about 1.2 TFLOP/s) bound it; summing the K values of each stencil
-// edge into its symmetric P x P block once leaves P^2 FMAs per edge (3x
-// fewer FP64 operations) for (S P (P+1) / 2) doubles per row of memory.
-// Block build: thread per (row, packed pair), loop over the pair's (k, g)
-// list and the slots.  Apply: lane = row of a 32-row tile, warps over the
-// output modes; C_ab and C_ba are one stored value, read by two warps of
-// the same CTA (the second from L1).
+// Assembled FP64 apply.  GB300's FP64 units (2 FMAs per clock and SM) bound
+// FP64 applies: the generated kernel spends two FP64 operations per triple
+// and slot (2,395 triples at P = 35), one P x P block per edge P^2 FMAs, and
+// each edge's flux B^e (x_hi - x_lo) is formed once for both of its nodes, as
+// in the generated FP32 edge form: about 2.1 P^2 FMAs per row against 5 P^2
+// for a block per stencil slot.  An apply with cold caches, before and now:
+// 881 and 397 us at 256^2, P = 35 (the operations alone 255 us), 4.96 and 1.89
+// ms at 256^2, P = 84, 16.4 and 10.2 us at 32^2, P = 6.  Lane: a column of the tile (AsmBlocks): its
+// node's west edge from the lane itself, its east edge's flux from the next
+// lane; the CTA marches up its strip of rows and keeps the flux through a
+// row's upper edges for the next row; warps and CTA groups share the outputs,
+// a warp's outputs in registers.  The differences of up to 64 modes stand in
+// shared memory.  B_ab and B_ba are one stored value, read by two warps of
+// the CTA (the second from L1 or L2).
 // ---------------------------------------------------------------------------
-__global__ void k_asm_build(int64_t ldr, int S, int npair, const int* __restrict__ pptr, const int* __restrict__ pk,
-                            const double* __restrict__ pg, const double* __restrict__ V, double* __restrict__ C) {
-  const int64_t r = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-  const int p = blockIdx.y;
-  if (r >= ldr) return;
-  const int e0 = pptr[p], e1 = pptr[p + 1];
-  for (int s = 0; s < S; ++s) {
+
+// Blocks from the slot values: thread per edge (in the order of AsmBlocks) and
+// pairs p = blockIdx.y, blockIdx.y + gridDim.y, ...  The conductance of an
+// edge between two unknowns is minus their slot value.  A row's slot values
+// add up to the conductances of its edges to the Dirichlet boundary; those
+// edges act on the same difference, so the first of them (west, east, south,
+// north) takes the sum and the others zero.
+__global__ void k_edge_blocks64(int N, int strip, int64_t len, int S, int64_t ldr, const int* __restrict__ col,
+                                int npair, const int* __restrict__ pptr, const int* __restrict__ pk,
+                                const double* __restrict__ pg, const double* __restrict__ V, double* __restrict__ C) {
+  const int64_t q = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+  if (q >= len) return;
+  const int m = N - 1, lane = int(q & 31), visits = 2 * strip + 1;
+  const int64_t t = (q >> 5) / visits, column = 31 * t + lane;
+  const int visit = int((q >> 5) % visits), ver = visit % 2 == 0;
+  // the edge's nodes (i, j), (i2, j2); r: the row of one that is an unknown
+  const int64_t sn = column / N;
+  const int e = int(column - sn * N), j = int(std::min<int64_t>(N, sn * strip + (visit + 1) / 2));
+  const int i = e + ver, i2 = e + 1, j2 = j + ver;
+  const bool in = i >= 1 && i <= m && j >= 1 && j <= m, in2 = i2 >= 1 && i2 <= m && j2 >= 1 && j2 <= m;
+  const int64_t r = int64_t((in ? j : j2) - 1) * m + (in ? i : i2) - 1;
+  int s0 = 0, s1 = 0;  // the conductance is sign x the sum over slots s0 .. s1 - 1
+  double sign = 1.0;
+  if (in && in2) {
+    const int64_t r2 = int64_t(j2 - 1) * m + i2 - 1;
+    for (int s = 0; s < S; ++s)
+      if (col[s * ldr + r] == r2) {
+        s0 = s;
+        s1 = s + 1;
+      }
+    sign = -1.0;
+  } else if (in || in2) {
+    const int iu = in ? i : i2, ju = in ? j : j2;  // the unknown
+    const bool first = ver ? iu > 1 && iu < m && (j == 0 || ju > 1) : i == 0 || iu > 1;
+    if (first) s1 = S;
+  }
+  for (int p = blockIdx.y; p < npair; p += gridDim.y) {
     double c = 0.0;
-    for (int e = e0; e < e1; ++e) c += pg[e] * V[(int64_t(pk[e]) * S + s) * ldr + r];
-    C[(int64_t(s) * npair + p) * ldr + r] = c;
+    if (s1 > s0)
+      for (int u = pptr[p]; u < pptr[p + 1]; ++u) {
+        const double* v = V + int64_t(pk[u]) * S * ldr + r;
+        double x = v[s0 * ldr];
+        for (int s = s0 + 1; s < s1; ++s) x += v[s * ldr];
+        c = fma(pg[u], sign * x, c);
+      }
+    C[((q >> 5) * npair + p) * 32 + lane] = c;
   }
 }
 
-__global__ void __launch_bounds__(256) k_apply_asm64(int64_t n, int64_t ldr, int S, int P, int npair,
-                                                      const int* __restrict__ col, const double* __restrict__ C,
-                                                      const double* __restrict__ X, int64_t ldx,
-                                                      const double* __restrict__ F, int64_t ldf,
-                                                      double* __restrict__ Y, int64_t ldy) {
-  const int64_t r = int64_t(blockIdx.x) * 32 + threadIdx.x;
-  if (r >= n) return;
-  for (int a = threadIdx.y; a < P; a += blockDim.y) {
-    // packed index of (lo, hi), lo <= hi: off(lo) + hi with
-    // off(b) = b P - b (b - 1) / 2 - b
-    const int off_a = a * P - a * (a - 1) / 2 - a;
-    double acc = 0.0;
-    for (int s = 0; s < S; ++s) {
-      const int c = col[int64_t(s) * ldr + r];
-      const double* Cs = C + int64_t(s) * npair * ldr + r;
-      const double* xc = X + c;
-      int off_b = 0;
-      for (int b = 0; b < P; ++b) {
-        const int pidx = b < a ? off_b + a : off_a + b;
-        acc = fma(Cs[int64_t(pidx) * ldr], xc[int64_t(b) * ldx], acc);
-        off_b += P - b - 1;
+constexpr int kAsmModes = 64;  // modes whose differences are in shared memory at a time
+constexpr int kAsmWarps = 16;
+
+struct AsmArgs {
+  int N, P, npair, strip, W, G;
+  const double* C;
+  const double* X;
+  int64_t ldx;
+  const double* F;
+  int64_t ldf;
+  double* Y;
+  int64_t ldy;
+};
+
+// packed index of (a, b): the pair's row starts at lo P - lo (lo + 1) / 2
+__device__ __forceinline__ int pair_index(int P, int a, int b) {
+  const int lo = min(a, b), hi = max(a, b);
+  return lo * P - lo * (lo + 1) / 2 + hi;
+}
+
+// f += sum_b B_ab d_b over modes b0 .. b0 + nb - 1 (d: [64][32], lane's column)
+__device__ __forceinline__ double asm_dot(const double* __restrict__ C, int P, int a, int b0, int nb, const double* d,
+                                          double f) {
+  int b = 0;
+  for (; b + 8 <= nb; b += 8) {
+    double c[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) c[u] = C[int64_t(pair_index(P, a, b0 + b + u)) * 32];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) f = fma(c[u], d[(b + u) * 32], f);
+  }
+  for (; b < nb; ++b) f = fma(C[int64_t(pair_index(P, a, b0 + b)) * 32], d[b * 32], f);
+  return f;
+}
+
+// the same over two edges: f += sum_b C_ab d_b, f2 += sum_b C2_ab d2_b
+__device__ __forceinline__ void asm_dot2(const double* __restrict__ C, const double* __restrict__ C2, int P, int a,
+                                         int b0, int nb, const double* d, const double* d2, double& f, double& f2) {
+  constexpr int U = 4;
+  int b = 0;
+  for (; b + U <= nb; b += U) {
+    double c[U], c2[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int64_t o = int64_t(pair_index(P, a, b0 + b + u)) * 32;
+      c[u] = C[o];
+      c2[u] = C2[o];
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      f = fma(c[u], d[(b + u) * 32], f);
+      f2 = fma(c2[u], d2[(b + u) * 32], f2);
+    }
+  }
+  for (; b < nb; ++b) {
+    const int64_t o = int64_t(pair_index(P, a, b0 + b)) * 32;
+    f = fma(C[o], d[b * 32], f);
+    f2 = fma(C2[o], d2[b * 32], f2);
+  }
+}
+
+template <int MO>
+__global__ void __launch_bounds__(32 * kAsmWarps, 2) k_apply_edge64(const __grid_constant__ AsmArgs p) {
+  extern __shared__ double ds[];  // [3][min(P, 64)][32]: west, upper, lower edge
+  const int P = p.P, N = p.N, m = N - 1, lane = threadIdx.x, w = threadIdx.y;
+  const int g = blockIdx.x % p.G;
+  const int bc = min(P, kAsmModes);
+  double* dh = ds + lane;
+  double* dv = dh + bc * 32;
+  double* dl = dv + bc * 32;
+  const int64_t t = blockIdx.x / p.G, column = 31 * t + lane, sn = column / N;
+  const int i = int(column - sn * N);  // node column to the west; the lane's own node is i + 1
+  const int j0 = 1 + int(sn) * p.strip;
+  const double* C = p.C + t * (2 * p.strip + 1) * p.npair * 32 + lane;
+  double lower[MO];
+#pragma unroll
+  for (int o = 0; o < MO; ++o) lower[o] = 0.0;
+  for (int k = 0; k < p.strip; ++k) {
+    const int j = j0 + k;
+    const bool in0 = i >= 1 && j <= m, in1 = i + 1 <= m && j <= m;
+    const double* Ch = C + int64_t(2 * k + 1) * p.npair * 32;
+    const double* Cv = Ch + int64_t(p.npair) * 32;
+    const int64_t r = int64_t(j - 1) * m + i;  // the lane's own node
+    double fh[MO], fv[MO];
+#pragma unroll
+    for (int o = 0; o < MO; ++o) fh[o] = fv[o] = 0.0;
+    for (int b0 = 0; b0 < P; b0 += kAsmModes) {
+      const int nb = min(kAsmModes, P - b0);
+      __syncthreads();
+#pragma unroll 4
+      for (int b = w; b < nb; b += p.W) {
+        const double* x = p.X + int64_t(b0 + b) * p.ldx + r;
+        const double x1 = in1 ? x[0] : 0.0;
+        const double x0 = in0 ? x[-1] : 0.0;
+        const double x2 = in1 && j < m ? x[m] : 0.0;
+        dh[b * 32] = x1 - x0;
+        dv[b * 32] = x2 - x1;
+        if (k == 0) dl[b * 32] = x1 - (in1 && j > 1 ? x[-m] : 0.0);
+      }
+      __syncthreads();
+#pragma unroll
+      for (int o = 0; o < MO; ++o) {
+        const int a = g + p.G * (w + p.W * o);
+        if (a < P) {
+          if (k == 0) lower[o] = asm_dot(C, P, a, b0, nb, dl, lower[o]);
+          asm_dot2(Ch, Cv, P, a, b0, nb, dh, dv, fh[o], fv[o]);
+        }
       }
     }
-    Y[int64_t(a) * ldy + r] = F ? F[int64_t(a) * ldf + r] - acc : acc;
+#pragma unroll
+    for (int o = 0; o < MO; ++o) {
+      const int a = g + p.G * (w + p.W * o);
+      const double east = __shfl_down_sync(0xffffffffu, fh[o], 1);
+      const double y = (fh[o] - east) + (lower[o] - fv[o]);
+      lower[o] = fv[o];
+      if (a < P && lane < 31 && in1)
+        p.Y[int64_t(a) * p.ldy + r] = p.F ? p.F[int64_t(a) * p.ldf + r] - y : y;
+    }
   }
 }
 
@@ -256,15 +391,39 @@ void pair_lists(const sg_problem* pr, std::vector<int>& pptr, std::vector<int>& 
   }
 }
 
-sg_status asm_prepare(sg_problem* pr, const Ell& A, AsmBlocks& B, cudaStream_t st) {
+sg_status asm_prepare(sg_problem* pr, bool coarse, cudaStream_t st) {
+  AsmBlocks& B = coarse ? coarse_asm(pr) : pr->asm_fine;
   if (B.tried || pr->asm_mode == 1) return SG_OK;
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   SG_CUDA(cudaStreamIsCapturing(st, &cs));
   if (cs != cudaStreamCaptureStatusNone) return SG_OK;
   B.tried = true;
-  const int P = pr->P, S = A.S;
+  const int P = pr->P, N = coarse ? pr->N / 2 : pr->N, m = N - 1;
   const int npair = P * (P + 1) / 2;
-  const size_t bytes = size_t(S) * npair * A.ldr * sizeof(double);
+  if (m <= 0) return SG_OK;
+  // An SM's CTAs share its FP64 units: the strip and the split of the outputs
+  // over groups of CTAs with the fewest CTAs per SM x visits x work of a
+  // visit (its outputs, and the differences, worth about two); one CTA alone
+  // on an SM leaves a quarter of its time to latencies.  Measured at 256^2, P =
+  // 35, us by strip and groups: (4, 1) 416, (8, 1) 400, (16, 1) 494, (4, 4)
+  // 399, (16, 4) 510; 200^2, P = 56: (3, 1) 582, (8, 1) 909, (3, 4) 594, (16,
+  // 1) 961.
+  auto tiles_of = [&](int strip) { return (int64_t((m + strip - 1) / strip) * N + 30) / 31; };
+  int strip = 1, groups = 1;
+  int64_t best = 0;
+  for (int s = 1; s <= 16; ++s)
+    for (int outs = std::min(P, kAsmModes); outs >= std::min(P, 4); --outs) {
+      const int g = (P + outs - 1) / outs;
+      const int64_t per_sm = (tiles_of(s) * g + 151) / 152;
+      const int64_t cost = (per_sm == 1 ? 5 : 4 * per_sm) * (2 * s + 1) * (outs + 2);
+      if (best == 0 || cost < best) {
+        best = cost;
+        strip = s;
+        groups = g;
+      }
+    }
+  const int64_t tiles = tiles_of(strip);
+  const size_t bytes = size_t(tiles) * (2 * strip + 1) * 32 * npair * sizeof(double);
   if (pr->asm_mode == 0) {
     // automatic: only while the blocks take at most a quarter of free memory
     size_t fr = 0, tot = 0;
@@ -274,6 +433,7 @@ sg_status asm_prepare(sg_problem* pr, const Ell& A, AsmBlocks& B, cudaStream_t s
   std::vector<int> pptr, pk;
   std::vector<double> pg;
   pair_lists(pr, pptr, pk, pg);
+  const Ell& A = coarse ? coarse_ell(pr) : pr->fine;
   DevBuf dptr, dk, dg, c;
   SG_TRY(c.alloc(bytes));
   SG_TRY(dptr.alloc(pptr.size() * 4));
@@ -284,25 +444,57 @@ sg_status asm_prepare(sg_problem* pr, const Ell& A, AsmBlocks& B, cudaStream_t s
     SG_CUDA(cudaMemcpy(dk.ptr, pk.data(), pk.size() * 4, cudaMemcpyHostToDevice));
     SG_CUDA(cudaMemcpy(dg.ptr, pg.data(), pg.size() * 8, cudaMemcpyHostToDevice));
   }
-  k_asm_build<<<dim3(unsigned((A.ldr + 127) / 128), unsigned(npair)), 128, 0, st>>>(
-      A.ldr, S, npair, dptr.as<int>(), dk.as<int>(), dg.as<double>(), A.v64.as<double>(), c.as<double>());
+  const int64_t len = int64_t(bytes / sizeof(double)) / npair;
+  const int64_t nb = (len + 127) / 128;
+  k_edge_blocks64<<<dim3(unsigned(nb), unsigned(std::min<int64_t>({npair, 65535, std::max<int64_t>(1, 152 * 64 / nb)}))),
+                    128, 0, st>>>(N, strip, len, A.S, A.ldr, A.col.as<int>(), npair, dptr.as<int>(), dk.as<int>(),
+                                  dg.as<double>(), A.v64.as<double>(), c.as<double>());
   note_launch();
   SG_CUDA(cudaGetLastError());
   SG_CUDA(cudaStreamSynchronize(st));
+  B.N = N;
+  B.strip = strip;
+  B.groups = groups;
   B.npair = npair;
   B.c = std::move(c);
   return SG_OK;
 }
 
-sg_status apply_asm64(const sg_problem* pr, const Ell& A, const AsmBlocks& B, const double* X, int64_t ldx,
-                      const double* F, int64_t ldf, double* Y, int64_t ldy, cudaStream_t st) {
-  if (A.n == 0) return SG_OK;
-  const dim3 block(32, 8);
-  k_apply_asm64<<<unsigned((A.n + 31) / 32), block, 0, st>>>(A.n, A.ldr, A.S, pr->P, B.npair, A.col.as<int>(),
-                                                              B.c.as<double>(), X, ldx, F, ldf, Y, ldy);
+template <int MO>
+static sg_status asm_launch(const AsmArgs& a, dim3 grid, size_t smem, cudaStream_t st) {
+  k_apply_edge64<MO><<<grid, dim3(32, a.W), smem, st>>>(a);
   note_launch();
   SG_CUDA(cudaGetLastError());
   return SG_OK;
+}
+
+sg_status apply_asm64(const sg_problem* pr, const AsmBlocks& B, const double* X, int64_t ldx, const double* F,
+                      int64_t ldf, double* Y, int64_t ldy, cudaStream_t st) {
+  const int N = B.N, m = N - 1, P = pr->P;
+  AsmArgs a;
+  a.N = N;
+  a.P = P;
+  a.npair = B.npair;
+  a.strip = B.strip;
+  a.G = B.groups;
+  a.W = std::min(kAsmWarps, (P + a.G - 1) / a.G);
+  a.C = B.c.as<double>();
+  a.X = X;
+  a.ldx = ldx;
+  a.F = F;
+  a.ldf = ldf;
+  a.Y = Y;
+  a.ldy = ldy;
+  const int64_t tiles = (int64_t((m + a.strip - 1) / a.strip) * N + 30) / 31;
+  const dim3 grid(unsigned(tiles * a.G));
+  const size_t smem = size_t(3) * std::min(P, kAsmModes) * 32 * sizeof(double);
+  const int mo = (P + a.G * a.W - 1) / (a.G * a.W);
+  switch (mo) {
+    case 1: return asm_launch<1>(a, grid, smem, st);
+    case 2: return asm_launch<2>(a, grid, smem, st);
+    case 3: return asm_launch<3>(a, grid, smem, st);
+    default: return asm_launch<4>(a, grid, smem, st);
+  }
 }
 
 bool solver_edge(const sg_problem* pr) {
@@ -323,7 +515,7 @@ sg_status apply_any(sg_problem* pr, bool coarse, const T* X, int64_t ldx, const 
   if (sizeof(T) == 8) {
     const AsmBlocks& B = coarse ? coarse_asm(pr) : pr->asm_fine;
     if (B.c.ptr)
-      return apply_asm64(pr, A, B, reinterpret_cast<const double*>(X), ldx, reinterpret_cast<const double*>(F),
+      return apply_asm64(pr, B, reinterpret_cast<const double*>(X), ldx, reinterpret_cast<const double*>(F),
                          ldf, reinterpret_cast<double*>(Y), ldy, st);
   }
   if (pr->apply_mode != 1 && jit_eligible(pr)) {
@@ -354,7 +546,7 @@ template sg_status apply_any<float>(sg_problem*, bool, const float*, int64_t, co
 template <typename T>
 sg_status apply_op(sg_problem* pr, bool coarse, const T* X, int64_t ldx, const T* F, int64_t ldf, T* Y,
                    int64_t ldy, cudaStream_t st, bool solver) {
-  if (sizeof(T) == 8) SG_TRY(asm_prepare(pr, coarse ? coarse_ell(pr) : pr->fine, coarse ? coarse_asm(pr) : pr->asm_fine, st));
+  if (sizeof(T) == 8) SG_TRY(asm_prepare(pr, coarse, st));
   size_t slot = 0;
   const bool on = pr->prof.on;
   if (on) SG_TRY(pr->prof.begin((coarse ? 2 : 0) + (sizeof(T) == 8 ? 1 : 0), st, slot));

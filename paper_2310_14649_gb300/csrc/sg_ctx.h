@@ -444,8 +444,8 @@ struct SolverCtx {
   // specialised kernels, kernel attributes, network buffers
   sg_status capture_prepare() {
     if (sizeof(T) == 8) {
-      SG_TRY(asm_prepare(pr, pr->fine, pr->asm_fine, nullptr));
-      SG_TRY(asm_prepare(pr, pc->co.ell, pc->co.asm_c, nullptr));
+      SG_TRY(asm_prepare(pr, false, nullptr));
+      SG_TRY(asm_prepare(pr, true, nullptr));
       SG_TRY(resid_prepare(pr, nullptr));
     }
     if (sizeof(T) == 4) {

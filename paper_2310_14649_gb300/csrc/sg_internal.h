@@ -105,11 +105,20 @@ struct EdgeTerms {
   DevBuf scale;           // double K: factor of the stored conductances
 };
 
-// The Galerkin operator summed per stencil edge into its P x P block (FP64),
-//   C_ab^{r,s} = sum_k g_kab v_k^{r,s}   (symmetric: a <= b stored, packed
-//   row by row), layout [S][npair][ldr]; built on demand for FP64 applies.
+// The Galerkin operator of an N x N mesh with each edge's P x P block summed
+// once (FP64), B_ab^e = sum_k g_kab w_k(e) (symmetric: a <= b stored, packed
+// row by row), in the order the apply reads them: the node rows are cut into
+// strips of `strip` rows, the strips' N edge columns laid side by side, and
+// tile t holds columns 31 t + lane (the last one again in the next tile);
+// visit 0 of a tile is the vertical edges below the strip's first row, visits
+// 2 k + 1 and 2 k + 2 the horizontal edges of its row k and the vertical ones
+// above,
+//     c[((t (2 strip + 1) + visit) npair + pair) 32 + lane],
+// one contiguous run per tile.  Column e of a strip: the horizontal edge
+// (e, j)-(e + 1, j), the vertical edges of node column e + 1.  Built on demand
+// for FP64 applies.
 struct AsmBlocks {
-  int npair = 0;
+  int N = 0, npair = 0, strip = 1, groups = 1;
   bool tried = false;  // the policy was applied (built or declined)
   DevBuf c;
 };
@@ -332,7 +341,7 @@ bool solver_edge(const sg_problem* pr);
 sg_status apply_prepare32(sg_problem* pr, bool coarse, cudaStream_t st);
 // assembled FP64 blocks (sg_apply.cu): build per the problem's policy (no-op
 // once tried; never while `st` is capturing), and the apply over them
-sg_status asm_prepare(sg_problem* pr, const Ell& A, AsmBlocks& B, cudaStream_t st);
+sg_status asm_prepare(sg_problem* pr, bool coarse, cudaStream_t st);
 // (k, g_kab) list of every packed pair a <= b (pair index a P - a (a - 1) / 2
 // + b - a): pair q owns entries [pptr[q], pptr[q + 1]) of pk, pg
 void pair_lists(const sg_problem* pr, std::vector<int>& pptr, std::vector<int>& pk, std::vector<double>& pg);
@@ -345,8 +354,8 @@ sg_status resid_df(sg_problem* pr, const double* F, int64_t ldf, const double* X
                    int64_t ldr, cudaStream_t st);
 sg_status refine_residual(sg_problem* pr, const double* F, int64_t ldf, const double* X, int64_t ldx, double* R,
                           int64_t ldr, cudaStream_t st);
-sg_status apply_asm64(const sg_problem* pr, const Ell& A, const AsmBlocks& B, const double* X, int64_t ldx,
-                      const double* F, int64_t ldf, double* Y, int64_t ldy, cudaStream_t st);
+sg_status apply_asm64(const sg_problem* pr, const AsmBlocks& B, const double* X, int64_t ldx, const double* F,
+                      int64_t ldf, double* Y, int64_t ldy, cudaStream_t st);
 // (solver: the form FP32 solves use, solver_edge)
 // the operator apply without timing: assembled blocks (FP64, when built),
 // else the specialised kernel, else the shared-memory kernel

@@ -332,8 +332,8 @@ sg_status sg_set_apply_fp64(sg_problem* pr, int mode) {
   pr->asm_fine = AsmBlocks();
   if (pr->solver) pr->solver->pc.co.asm_c = AsmBlocks();
   if (mode == 2) {
-    SG_TRY(asm_prepare(pr, pr->fine, pr->asm_fine, nullptr));
-    if (pr->solver && pr->solver->pc.ready) SG_TRY(asm_prepare(pr, coarse_ell(pr), coarse_asm(pr), nullptr));
+    SG_TRY(asm_prepare(pr, false, nullptr));
+    if (pr->solver && pr->solver->pc.ready) SG_TRY(asm_prepare(pr, true, nullptr));
   }
   return SG_OK;
 }

@@ -115,6 +115,17 @@ def test_apply_vs_oracle(gpu, dt, N, L, p, q):
     check_apply(prob, ref, random_block(ref.n, ref.P, seed=4), dtype, ld=ref.n + 37, kernel=kernel, fp64=fp64)
 
 
+@pytest.mark.parametrize("N,L,p", [(2, 1, 1), (3, 2, 1), (31, 1, 2), (32, 15, 1), (33, 16, 1), (63, 3, 1),
+                                   (125, 2, 2), (18, 3, 5), (19, 4, 4), (160, 3, 2)])
+def test_fp64_blocks_tiles(gpu, N, L, p):
+    """The FP64 apply over edge blocks at the edges of its tiles: one unknown,
+    strips that share a tile, a last strip cut short, 16 and 17 outputs, more
+    modes than one shared-memory block of differences (70)."""
+    import torch
+    prob, ref = setup_pair(N, L, p, min(2 * p, 8 if L > 1 else 16))
+    check_apply(prob, ref, random_block(ref.n, ref.P, seed=15), torch.float64, ld=ref.n + 3, fp64=2)
+
+
 @pytest.mark.parametrize("fp64", [1, 2])
 def test_residual_in_place(gpu, fp64):
     import torch
