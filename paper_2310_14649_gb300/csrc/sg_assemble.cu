@@ -145,6 +145,60 @@ __global__ void k_edge_values(const Tc* __restrict__ cb, int N, int KT, const in
   }
 }
 
+// All terms at once: CTA per (node row, tile, direction), warp per four
+// consecutive positions, which a lane writes as one 16- or 32-byte piece (a
+// thread per term writes single words 16 bytes apart: 80 us at 128^2, K = 210
+// for 55 MB in and out)
+// FP32 coefficients: scale = hi + lo in FP32 (the conversions and products of
+// FP64 run at 1/64 of the FP32 rate: 65 us; now 21).
+template <typename Tc>
+__global__ void __launch_bounds__(256) k_edge_values_all(const Tc* __restrict__ cb, int N, int KT,
+                                                         const int* __restrict__ term,
+                                                         const double* __restrict__ scale,
+                                                         const float2* __restrict__ scale2, float* __restrict__ v32,
+                                                         double* __restrict__ v64) {
+  const int m = N - 1, ntile = (N + 30) / 31, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  const int64_t E = 2LL * N * N, q = blockIdx.x;
+  const int ver = int(q & 1), tile = int((q >> 1) % ntile), j = int((q >> 1) / ntile), e = 31 * tile + lane;
+  // the edge's two triangles (edge_conductance), or none
+  int64_t t0 = -1, t1 = -1;
+  if (ver) {
+    if (lane < 31 && e + 1 <= m) {
+      t0 = 2 * (int64_t(j) * N + e + 1) + 1;
+      t1 = 2 * (int64_t(j) * N + e);
+    }
+  } else if (j >= 1 && e < N) {
+    t0 = 2 * (int64_t(j) * N + e);
+    t1 = 2 * (int64_t(j - 1) * N + e) + 1;
+  }
+#pragma unroll 2
+  for (int g = threadIdx.x >> 5; g < KT / 4; g += nw) {
+    const int4 k4 = reinterpret_cast<const int4*>(term)[g];
+    const int k[4] = {k4.x, k4.y, k4.z, k4.w};
+    Tc w[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      w[u] = k[u] >= 0 && t0 >= 0 ? Tc(0.5) * (cb[k[u] * E + t0] + cb[k[u] * E + t1]) : Tc(0);
+    const int64_t at = (q * (KT / 4) + g) * 32 + lane;
+    if constexpr (sizeof(Tc) == 4) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const float2 s = scale2[k[u] >= 0 ? k[u] : 0];
+        w[u] = fmaf(w[u], s.x, w[u] * s.y);
+      }
+      if (v32) reinterpret_cast<float4*>(v32)[at] = make_float4(w[0], w[1], w[2], w[3]);
+    } else {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) w[u] *= scale[k[u] >= 0 ? k[u] : 0];
+      if (v32) reinterpret_cast<float4*>(v32)[at] = make_float4(float(w[0]), float(w[1]), float(w[2]), float(w[3]));
+    }
+    if (v64) {
+      reinterpret_cast<double2*>(v64)[2 * at] = make_double2(w[0], w[1]);
+      reinterpret_cast<double2*>(v64)[2 * at + 1] = make_double2(w[2], w[3]);
+    }
+  }
+}
+
 __global__ void k_round_values(const double* __restrict__ v64, float* __restrict__ v32, int64_t len) {
   for (int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; t < len; t += int64_t(gridDim.x) * blockDim.x)
     v32[t] = float(v64[t]);
@@ -213,6 +267,19 @@ sg_status edge_values(const sg_problem* pr, const Tc* coef, int k0, int kn, Edge
 template sg_status edge_values<float>(const sg_problem*, const float*, int, int, EdgeVals&, cudaStream_t);
 template sg_status edge_values<double>(const sg_problem*, const double*, int, int, EdgeVals&, cudaStream_t);
 
+template <typename Tc>
+sg_status edge_values_all(const sg_problem* pr, const Tc* coef, EdgeVals& out, cudaStream_t st) {
+  const EdgeTerms& T = pr->edge_terms;
+  const int64_t blocks = 2 * int64_t(out.N) * ((out.N + 30) / 31);
+  k_edge_values_all<Tc><<<unsigned(blocks), 256, 0, st>>>(coef, out.N, T.KT, T.term.as<int>(), T.scale.as<double>(),
+                                                          T.scale2.as<float2>(), out.v32.as<float>(), out.v64.as<double>());
+  note_launch();
+  SG_CUDA(cudaGetLastError());
+  return SG_OK;
+}
+template sg_status edge_values_all<float>(const sg_problem*, const float*, EdgeVals&, cudaStream_t);
+template sg_status edge_values_all<double>(const sg_problem*, const double*, EdgeVals&, cudaStream_t);
+
 static sg_status edge_terms_build(sg_problem* pr) {
   const std::vector<int> term = jit_edge_terms(pr);
   std::vector<int> off(pr->K + 1, 0), pos(term.size());
@@ -228,9 +295,18 @@ static sg_status edge_terms_build(sg_problem* pr) {
   SG_TRY(T.off.alloc(off.size() * 4));
   SG_TRY(T.pos.alloc(pos.size() * 4));
   SG_CUDA(cudaMemcpy(T.off.ptr, off.data(), off.size() * 4, cudaMemcpyHostToDevice));
+  SG_TRY(T.term.alloc(term.size() * 4));
+  SG_CUDA(cudaMemcpy(T.term.ptr, term.data(), term.size() * 4, cudaMemcpyHostToDevice));
   const std::vector<double> scale = jit_edge_scale(pr);
   SG_TRY(T.scale.alloc(scale.size() * 8));
   SG_CUDA(cudaMemcpy(T.scale.ptr, scale.data(), scale.size() * 8, cudaMemcpyHostToDevice));
+  std::vector<float2> scale2(scale.size());
+  for (size_t k = 0; k < scale.size(); ++k) {
+    const float hi = float(scale[k]);
+    scale2[k] = make_float2(hi, float(scale[k] - double(hi)));
+  }
+  SG_TRY(T.scale2.alloc(scale2.size() * 8));
+  SG_CUDA(cudaMemcpy(T.scale2.ptr, scale2.data(), scale2.size() * 8, cudaMemcpyHostToDevice));
   SG_CUDA(cudaMemcpy(T.pos.ptr, pos.data(), pos.size() * 4, cudaMemcpyHostToDevice));
   return SG_OK;
 }

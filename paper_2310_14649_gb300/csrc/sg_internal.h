@@ -102,7 +102,9 @@ struct EdgeVals {
 struct EdgeTerms {
   int KT = 0, R = 1;  // positions; turns of the kernel's loop over orbits (KT / R positions each)
   DevBuf off, pos;        // int32 K + 1, KT
+  DevBuf term;            // int32 KT: the term at a position, -1 for padding
   DevBuf scale;           // double K: factor of the stored conductances
+  DevBuf scale2;          // float2 K: the same as hi + lo
 };
 
 // The Galerkin operator of an N x N mesh with each edge's P x P block summed
@@ -295,6 +297,9 @@ sg_status coarse_edge_build(sg_problem* pr, EdgeVals& out);
 sg_status edge_alloc(const sg_problem* pr, int N, bool f32, bool f64, EdgeVals& out);
 template <typename Tc>
 sg_status edge_values(const sg_problem* pr, const Tc* coef, int k0, int kn, EdgeVals& out, cudaStream_t st);
+// the same for all terms at once
+template <typename Tc>
+sg_status edge_values_all(const sg_problem* pr, const Tc* coef, EdgeVals& out, cudaStream_t st);
 // the FP32 five- or seven-slot values of an ELL family (rounded from the
 // FP64 ones on first use; synchronous then, never while `st` is capturing)
 sg_status ell_f32(const Ell& A, int K, cudaStream_t st);

@@ -25,6 +25,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <map>
 
 #include "sg_ctx.h"
 #include "sg_stencil.h"
@@ -39,8 +40,12 @@ struct NewtonWork {
   Ell op;                            // A(U): values of sum_j A(ctil_j) (FP64 and FP32)
   Ell dop;                           // A(dctil), the Jacobian's derivative part
   EdgeVals eop, edop;                // the same in the edge form (where the specialised kernel runs)
-  DevBuf ppp_off, ppp_ab, ppp_m64, ppp_m32;  // <psi_a psi_b psi_f> by rows f
-  DevBuf kfj_off, kfj_kf, kfj_m64, kfj_m32;  // <psi_k psi_f psi_j> by rows j (k | f << 16)
+  struct RowLists {
+    DevBuf row, ptr, at, m64, m32;         // groups of equal coefficients
+    DevBuf qrow, qat, qm32;                // the same in quads
+  };
+  RowLists ppp, kfj;                 // <He_a He_b He_f> / f! by rows f, <He_k He_f He_j> / j! by rows j
+  DevBuf scale64, scale32;           // K: 1 / sqrt(k!)
   DevBuf u64, u32, f64, r64, r32, d32, d64, tmp32, tmp64, one, scal;
   double* host = nullptr;            // pinned scalars
   ~NewtonWork() {
@@ -55,76 +60,162 @@ void newton_free(sg_problem* pr) {
 
 namespace {
 
-constexpr int kNlElems = 32;   // elements per CTA, one per lane
-constexpr int kNlWarps = 8;
-
 // interior index of grid node (x, y), -1 on the boundary
 __device__ inline int64_t node_index(int x, int y, int N) {
   return (x >= 1 && x <= N - 1 && y >= 1 && y <= N - 1) ? int64_t(y - 1) * (N - 1) + (x - 1) : -1;
 }
 
+// Rows of sums over triples in the unnormalised chaos (He, not psi), where
+// the projection coefficients are integers of few distinct values: row f owns
+// groups [row[f], row[f + 1]), group g entries [4 ptr[g].x, ptr[g].y) of `at`
+// (first mode | second << 16) and adds mult[g] times the sum of their
+// products.  Quads: group g is the four entries at[g].
+template <typename T>
+struct Rows {
+  const int* row = nullptr;
+  const int2* ptr = nullptr;
+  const T* mult = nullptr;
+  const int4* at = nullptr;
+};
+
+// a lane's values: one element's in FP64, its cell's two elements' in FP32
+template <typename T> struct Lane;
+template <> struct Lane<double> { using V = double; };
+template <> struct Lane<float> { using V = float2; };
+__device__ __forceinline__ double vfma(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c) {
+  return make_float2(fmaf(a.x, b.x, c.x), fmaf(a.y, b.y, c.y));
+}
+__device__ __forceinline__ float2 vfma(float a, float2 b, float2 c) {
+  return make_float2(fmaf(a, b.x, c.x), fmaf(a, b.y, c.y));
+}
+
+// sum over the groups of a row of mult x sum first[k] second[f] (both
+// [modes][32], lane's column)
+template <typename T, typename V = typename Lane<T>::V>
+__device__ __forceinline__ V row_sum(const Rows<T>& R, int f, const V* first, const V* second) {
+  V acc = V();
+  const int g1 = R.row[f + 1];
+  for (int g = R.row[f]; g < g1; ++g) {
+    const int2 pe = R.ptr[g];
+    V s = V();
+    int t = 4 * pe.x;
+    for (; t + 4 <= pe.y; t += 4) {
+      const int4 q = R.at[t >> 2];
+      const int e[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+      for (int u = 0; u < 4; ++u) s = vfma(first[(e[u] & 0xffff) * 32], second[(e[u] >> 16) * 32], s);
+    }
+    if (t < pe.y) {
+      const int4 q = R.at[t >> 2];
+      const int e[3] = {q.x, q.y, q.z};
+#pragma unroll
+      for (int u = 0; u < 3; ++u)
+        if (t + u < pe.y) s = vfma(first[(e[u] & 0xffff) * 32], second[(e[u] >> 16) * 32], s);
+    }
+    acc = vfma(R.mult[g], s, acc);
+  }
+  return acc;
+}
+// the same over quads: no load of the lists waits for another
+template <typename T, typename V = typename Lane<T>::V>
+__device__ __forceinline__ V quad_sum(const Rows<T>& R, int f, const V* first, const V* second) {
+  V acc = V();
+  const int g1 = R.row[f + 1];
+#pragma unroll 4
+  for (int g = R.row[f]; g < g1; ++g) {
+    const int4 q = R.at[g];
+    const T m = R.mult[g];
+    const int e[4] = {q.x, q.y, q.z, q.w};
+    V s = V();
+#pragma unroll
+    for (int u = 0; u < 4; ++u) s = vfma(first[(e[u] & 0xffff) * 32], second[(e[u] >> 16) * 32], s);
+    acc = vfma(m, s, acc);
+  }
+  return acc;
+}
+
 // Per element block: the element averages of U (and dU), the projected
 // square w = Pi_p[ubar^2] (or its derivative dw = 2 Pi_p[ubar dubar]), and
 // out_j = base_j + sum_{(i,f)} <psi_i psi_f psi_j> cbar_i w_f for j < K.
-// Lane = element, warps stride over modes and output rows.
+// Warps stride over modes and output rows; the modes are scaled to the
+// unnormalised chaos (scale[k] = 1 / sqrt(k!), out[j] sqrt(j!)) so that one
+// FMA per triple remains and its coefficient is read once per group.  FP64,
+// lane = element: bound by the FP64 units.  FP32, lane = cell: bound by the
+// two shared-memory loads of a triple; the list's loads and address
+// arithmetic serve a cell's two triangles, and the groups are cut into quads
+// (the last one filled up with products of a zero row).  128^2, P = 35, K =
+// 210 (11,634 triples in 1,431 groups): FP64 1.76 ms with a coefficient per
+// triple, now 1.06 (the operations alone 0.75); FP32 234 us, now 185 (the
+// shared-memory loads alone 97; one element a lane 242, and 293 without the
+// quads).
 template <typename T>
-__global__ void __launch_bounds__(kNlElems* kNlWarps)
+__global__ void __launch_bounds__(32 * (sizeof(T) == 8 ? 8 : 16))
     k_nl_coef(int N, int64_t E, int P, int K, const T* __restrict__ U, int64_t ldu, const T* __restrict__ dU,
-              int64_t lddu, const T* __restrict__ cbar, const T* __restrict__ base, const int* __restrict__ ppp_off,
-              const int2* __restrict__ ppp_ab, const T* __restrict__ ppp_m, const int* __restrict__ kfj_off,
-              const int* __restrict__ kfj_kf, const T* __restrict__ kfj_m, T* __restrict__ out) {
+              int64_t lddu, const T* __restrict__ cbar, const T* __restrict__ base, const T* __restrict__ scale,
+              const __grid_constant__ Rows<T> ppp, const __grid_constant__ Rows<T> kfj, T* __restrict__ out) {
+  using V = typename Lane<T>::V;
+  constexpr int PER = sizeof(V) / sizeof(T);  // elements of a lane
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* sU = reinterpret_cast<T*>(smem_raw);   // [P][32]
-  T* sD = sU + P * kNlElems;                // [P][32]
-  T* sW = sD + P * kNlElems;                // [P][32]
-  T* sC = sW + P * kNlElems;                // [K][32]
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t e = int64_t(blockIdx.x) * kNlElems + lane;
+  V* sC = reinterpret_cast<V*>(smem_raw);  // [K][32]
+  V* sW = sC + K * 32;                     // [P][32]
+  V* sD = sW + P * 32;                     // [P][32]
+  V* sU = sD + P * 32;                     // [P][32]; row 0 is the zero row (mode K + 2 P of sC) after w
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int64_t e = (int64_t(blockIdx.x) * 32 + lane) * PER;
   const bool valid = e < E;
-  int64_t v[3] = {-1, -1, -1};
+  // nodes of the cell: (i,j), (i+1,j), (i+1,j+1), (i,j+1); the lower triangle
+  // holds the first three, the upper one all but the second
+  int64_t v[4] = {-1, -1, -1, -1};
   if (valid) {
     const int64_t cell = e >> 1;
     const int i = int(cell % N), j = int(cell / N);
-    if ((e & 1) == 0) {  // lower triangle (i,j), (i+1,j), (i+1,j+1)
-      v[0] = node_index(i, j, N);
-      v[1] = node_index(i + 1, j, N);
-      v[2] = node_index(i + 1, j + 1, N);
-    } else {             // upper triangle (i,j), (i+1,j+1), (i,j+1)
-      v[0] = node_index(i, j, N);
-      v[1] = node_index(i + 1, j + 1, N);
-      v[2] = node_index(i, j + 1, N);
-    }
+    v[0] = node_index(i, j, N);
+    if (PER == 2 || (e & 1) == 0) v[1] = node_index(i + 1, j, N);
+    v[2] = node_index(i + 1, j + 1, N);
+    if (PER == 2 || (e & 1)) v[3] = node_index(i, j + 1, N);
   }
   const T third = T(1) / T(3);
-  for (int a = warp; a < P; a += kNlWarps) {
-    T s = 0, sd = 0;
-    for (int q = 0; q < 3; ++q) {
-      if (v[q] < 0) continue;
-      s += U[int64_t(a) * ldu + v[q]];
-      if (dU) sd += dU[int64_t(a) * lddu + v[q]];
-    }
-    sU[a * kNlElems + lane] = s * third;
-    sD[a * kNlElems + lane] = sd * third;
+  auto average = [&](const T* x, T f) {
+    T u[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) u[q] = v[q] >= 0 ? x[v[q]] : T(0);
+    if constexpr (PER == 2)
+      return make_float2((u[0] + u[1] + u[2]) * f, (u[0] + u[2] + u[3]) * f);
+    else
+      return (u[0] + u[1] + u[2] + u[3]) * f;
+  };
+  for (int a = warp; a < P; a += nw) {
+    const T f = third * scale[a];
+    sU[a * 32 + lane] = average(U + int64_t(a) * ldu, f);
+    if (dU) sD[a * 32 + lane] = average(dU + int64_t(a) * lddu, f);
   }
-  for (int k = warp; k < K; k += kNlWarps) sC[k * kNlElems + lane] = valid ? cbar[int64_t(k) * E + e] : T(0);
-  __syncthreads();
-  const T* sB = dU ? sD : sU;
-  for (int f = warp; f < P; f += kNlWarps) {
-    T acc = 0;
-    for (int t = ppp_off[f]; t < ppp_off[f + 1]; ++t) {
-      const int2 ab = ppp_ab[t];
-      acc += ppp_m[t] * sU[ab.x * kNlElems + lane] * sB[ab.y * kNlElems + lane];
-    }
-    sW[f * kNlElems + lane] = dU ? T(2) * acc : acc;
+  auto global = [&](auto* x, int k) { return reinterpret_cast<decltype(x)>(x + int64_t(k) * E + e); };
+#pragma unroll 4
+  for (int k = warp; k < K; k += nw) {
+    const V c = valid ? *reinterpret_cast<const V*>(global(cbar, k)) : V();
+    sC[k * 32 + lane] = vfma(scale[k], c, V());
   }
   __syncthreads();
-  for (int j = warp; j < K; j += kNlWarps) {
-    T acc = (base && valid) ? base[int64_t(j) * E + e] : T(0);
-    for (int t = kfj_off[j]; t < kfj_off[j + 1]; ++t) {
-      const int kf = kfj_kf[t];
-      acc += kfj_m[t] * sC[(kf & 0xffff) * kNlElems + lane] * sW[(kf >> 16) * kNlElems + lane];
-    }
-    if (valid) out[int64_t(j) * E + e] = acc;
+  const V* sB = dU ? sD : sU;
+  for (int f = warp; f < P; f += nw) {
+    const V acc = row_sum<T>(ppp, f, sU + lane, sB + lane);
+    sW[f * 32 + lane] = vfma(dU ? T(2) : T(1), acc, V());
+  }
+  __syncthreads();
+  if constexpr (PER == 2) {
+    if (warp == 0) sU[lane] = V();
+    __syncthreads();
+  }
+  for (int j = warp; j < K; j += nw) {
+    const V b = (base && valid) ? *reinterpret_cast<const V*>(global(base, j)) : V();
+    V acc;
+    if constexpr (PER == 2)
+      acc = quad_sum<T>(kfj, j, sC + lane, sW + lane);
+    else
+      acc = row_sum<T>(kfj, j, sC + lane, sW + lane);
+    // <psi_i psi_f psi_j> = (integer) sqrt(j!) / (sqrt(i!) sqrt(f!))
+    if (valid) *reinterpret_cast<V*>(global(out, j)) = vfma(T(1) / scale[j], acc, b);
   }
 }
 
@@ -157,7 +248,8 @@ __global__ void k_to_f32(const double* __restrict__ x, float* __restrict__ y, in
 
 unsigned grid_len(int64_t len) { return unsigned(std::min<int64_t>((len + 255) / 256, 152 * 16)); }
 
-size_t coef_smem(int P, int K, size_t elem) { return size_t(3 * P + K) * kNlElems * elem; }
+// 32 values of 8 bytes (a double, two floats) per mode
+size_t coef_smem(int P, int K) { return size_t(3 * P + K) * 32 * 8; }
 
 sg_status attrs_once() {
   static bool done = false;
@@ -195,7 +287,7 @@ sg_status newton_prepare(sg_problem* pr) {
   SG_ARG(pr->q >= 2 * pr->p,
          "the nonlinear problem needs an input order q_in >= 2 p_out (the fourfold products go through the input set)");
   SG_ARG(K < 65536 && P < 32768, "the nonlinear problem supports K < 65536 and P < 32768");
-  if (coef_smem(P, K, 8) > 227 * 1024) {
+  if (coef_smem(P, K) > 227 * 1024) {
     set_error("the nonlinear problem's coefficient kernel needs (3 P + K) x 256 bytes of shared memory <= 227 KB");
     return SG_ERR_UNSUPPORTED;
   }
@@ -204,65 +296,66 @@ sg_status newton_prepare(sg_problem* pr) {
   w->P = P;
   w->K = K;
   w->E = pr->E;
-  // <psi_a psi_b psi_f>, a, b, f < P: the triples (k, a, b) with k < P (the
-  // output set is the leading part of the input set), rows by f = k
-  std::vector<int> poff(P + 1, 0);
-  std::vector<int2> pab;
-  std::vector<double> pm;
-  for (int64_t t = 0; t < pr->T; ++t) {
-    const int k = pr->kab[3 * t];
-    if (k >= P) break;
-    pab.push_back(make_int2(pr->kab[3 * t + 1], pr->kab[3 * t + 2]));
-    pm.push_back(pr->g[t]);
-    poff[k + 1] = int(pab.size());
-  }
-  for (int f = 1; f <= P; ++f) poff[f] = std::max(poff[f], poff[f - 1]);
-  // <psi_k psi_f psi_j>, k, j < K, f < P, by rows j (ascending k, f)
-  std::vector<int> koff(K + 1, 0), kkf;
-  std::vector<double> km;
-  std::vector<double> isf(K);
-  for (int k = 0; k < K; ++k) {
-    double fct = 1.0;
-    for (int i = 0; i < L; ++i)
-      for (int v = 2; v <= pr->mi_in[size_t(k) * L + i]; ++v) fct *= v;
-    isf[k] = 1.0 / std::sqrt(fct);
-  }
-  // 1D integers <He_a He_b He_c>, a, c <= q, b <= p
+  // 1D integers <He_a He_b He_c> / c! and, over the L variables, the factor
+  // of He_j in He_k He_f (1 / sqrt(k!) scales a mode to the He's)
   const int q = pr->q, p = pr->p;
-  std::vector<double> t1(size_t(q + 1) * (p + 1) * (q + 1));
+  std::vector<double> t1(size_t(q + 1) * (p + 1) * (q + 1)), isf(K), fact(q + 1, 1.0);
+  for (int c = 1; c <= q; ++c) fact[c] = fact[c - 1] * c;
   for (int a = 0; a <= q; ++a)
     for (int b = 0; b <= p; ++b)
-      for (int c = 0; c <= q; ++c) t1[(size_t(a) * (p + 1) + b) * (q + 1) + c] = double(he_triple_1d(a, b, c));
-  for (int j = 0; j < K; ++j) {
-    const int32_t* aj = &pr->mi_in[size_t(j) * L];
-    for (int k = 0; k < K; ++k) {
-      const int32_t* ak = &pr->mi_in[size_t(k) * L];
-      for (int f = 0; f < P; ++f) {
-        const int32_t* af = &pr->mi_in[size_t(f) * L];
-        double num = 1.0;
-        for (int i = 0; i < L && num != 0.0; ++i) num *= t1[(size_t(ak[i]) * (p + 1) + af[i]) * (q + 1) + aj[i]];
-        if (num == 0.0) continue;
-        kkf.push_back(k | (f << 16));
-        km.push_back(num * isf[k] * isf[f] * isf[j]);
-      }
-    }
-    koff[j + 1] = int(kkf.size());
+      for (int c = 0; c <= q; ++c)
+        t1[(size_t(a) * (p + 1) + b) * (q + 1) + c] = double(he_triple_1d(a, b, c)) / fact[c];
+  for (int k = 0; k < K; ++k) {
+    double fct = 1.0;
+    for (int i = 0; i < L; ++i) fct *= fact[pr->mi_in[size_t(k) * L + i]];
+    isf[k] = 1.0 / std::sqrt(fct);
   }
-  auto f32 = [](const std::vector<double>& v) {
-    std::vector<float> o(v.size());
-    for (size_t i = 0; i < v.size(); ++i) o[i] = float(v[i]);
-    return o;
+  // rows j < nrow over first modes k < nfirst and second modes f < P (the
+  // output set is the leading part of the input set), by value, k and f
+  auto build = [&](int nrow, int nfirst, NewtonWork::RowLists& out) -> sg_status {
+    std::vector<int> row(1, 0), at, qrow(1, 0), qat;
+    std::vector<int2> ptr;
+    std::vector<double> mult;
+    std::vector<float> qmult;
+    for (int j = 0; j < nrow; ++j) {
+      const int32_t* aj = &pr->mi_in[size_t(j) * L];
+      std::map<double, std::vector<int>> by;
+      for (int k = 0; k < nfirst; ++k) {
+        const int32_t* ak = &pr->mi_in[size_t(k) * L];
+        for (int f = 0; f < P; ++f) {
+          const int32_t* af = &pr->mi_in[size_t(f) * L];
+          double num = 1.0;
+          for (int i = 0; i < L && num != 0.0; ++i) num *= t1[(size_t(ak[i]) * (p + 1) + af[i]) * (q + 1) + aj[i]];
+          if (num != 0.0) by[num].push_back(k | (f << 16));
+        }
+      }
+      for (const auto& g : by) {
+        mult.push_back(g.first);
+        ptr.push_back(make_int2(int(at.size() / 4), int(at.size() + g.second.size())));
+        at.insert(at.end(), g.second.begin(), g.second.end());
+        qat.insert(qat.end(), g.second.begin(), g.second.end());
+        at.resize(round_up(at.size(), 4), 0);
+        qat.resize(at.size(), K + 2 * P);
+        qmult.resize(qat.size() / 4, float(g.first));
+      }
+      row.push_back(int(ptr.size()));
+      qrow.push_back(int(qmult.size()));
+    }
+    SG_TRY(upload(out.row, row.data(), row.size() * 4));
+    SG_TRY(upload(out.ptr, ptr.data(), ptr.size() * sizeof(int2)));
+    SG_TRY(upload(out.at, at.data(), at.size() * 4));
+    SG_TRY(upload(out.m64, mult.data(), mult.size() * 8));
+    const std::vector<float> m32(mult.begin(), mult.end());
+    SG_TRY(upload(out.m32, m32.data(), m32.size() * 4));
+    SG_TRY(upload(out.qrow, qrow.data(), qrow.size() * 4));
+    SG_TRY(upload(out.qat, qat.data(), qat.size() * 4));
+    return upload(out.qm32, qmult.data(), qmult.size() * 4);
   };
-  SG_TRY(upload(w->ppp_off, poff.data(), poff.size() * 4));
-  SG_TRY(upload(w->ppp_ab, pab.data(), pab.size() * sizeof(int2)));
-  SG_TRY(upload(w->ppp_m64, pm.data(), pm.size() * 8));
-  std::vector<float> pm32 = f32(pm);
-  SG_TRY(upload(w->ppp_m32, pm32.data(), pm32.size() * 4));
-  SG_TRY(upload(w->kfj_off, koff.data(), koff.size() * 4));
-  SG_TRY(upload(w->kfj_kf, kkf.data(), kkf.size() * 4));
-  SG_TRY(upload(w->kfj_m64, km.data(), km.size() * 8));
-  std::vector<float> km32 = f32(km);
-  SG_TRY(upload(w->kfj_m32, km32.data(), km32.size() * 4));
+  SG_TRY(build(P, P, w->ppp));
+  SG_TRY(build(K, K, w->kfj));
+  SG_TRY(upload(w->scale64, isf.data(), isf.size() * 8));
+  const std::vector<float> isf32(isf.begin(), isf.end());
+  SG_TRY(upload(w->scale32, isf32.data(), isf32.size() * 4));
   // lognormal coefficients of every input term at every element
   const int64_t E = pr->E, KE = int64_t(K) * E;
   SG_TRY(w->cbar64.alloc(size_t(KE) * 8));
@@ -295,11 +388,20 @@ sg_status newton_prepare(sg_problem* pr) {
 template <typename T>
 sg_status nl_coef(sg_problem* pr, const T* U, const T* dU, const T* base, T* out, cudaStream_t st) {
   NewtonWork& w = *pr->nl;
-  const unsigned grid = unsigned((w.E + kNlElems - 1) / kNlElems);
-  k_nl_coef<T><<<grid, kNlElems * kNlWarps, coef_smem(w.P, w.K, sizeof(T)), st>>>(
-      pr->N, w.E, w.P, w.K, U, pr->ld, dU, pr->ld, sel<T>(w.cbar64, w.cbar32), base, dp<int>(w.ppp_off),
-      dp<int2>(w.ppp_ab), sel<T>(w.ppp_m64, w.ppp_m32), dp<int>(w.kfj_off), dp<int>(w.kfj_kf),
-      sel<T>(w.kfj_m64, w.kfj_m32), out);
+  constexpr int per = sizeof(T) == 8 ? 1 : 2;
+  const unsigned grid = unsigned((w.E + 32 * per - 1) / (32 * per));
+  auto rows = [](const NewtonWork::RowLists& l) {
+    return Rows<T>{dp<int>(l.row), dp<int2>(l.ptr), sel<T>(l.m64, l.m32), dp<int4>(l.at)};
+  };
+  Rows<T> kfj = rows(w.kfj);
+  if (sizeof(T) == 4) {
+    kfj.row = dp<int>(w.kfj.qrow);
+    kfj.at = dp<int4>(w.kfj.qat);
+    kfj.mult = dp<T>(w.kfj.qm32);
+  }
+  k_nl_coef<T><<<grid, 32 * (sizeof(T) == 8 ? 8 : 16), coef_smem(w.P, w.K), st>>>(
+      pr->N, w.E, w.P, w.K, U, pr->ld, dU, pr->ld, sel<T>(w.cbar64, w.cbar32), base, sel<T>(w.scale64, w.scale32),
+      rows(w.ppp), kfj, out);
   note_launch();
   SG_CUDA(cudaGetLastError());
   return SG_OK;
@@ -316,7 +418,7 @@ template <typename Tc>
 sg_status nl_values(sg_problem* pr, const Tc* coef, Ell& A, EdgeVals& E, bool f32, bool f64, cudaStream_t st) {
   if (nl_edge(pr)) {
     SG_TRY(edge_alloc(pr, pr->N, f32, f64, E));
-    return edge_values<Tc>(pr, coef, 0, pr->K, E, st);
+    return edge_values_all<Tc>(pr, coef, E, st);
   }
   const size_t len = size_t(pr->K) * A.S * A.ldr;
   if (f64 && !A.v64.ptr) SG_TRY(A.v64.alloc(len * 8));

@@ -148,3 +148,27 @@ def test_newton_full_384(gpu):
     sg.sg_newton(prob, Y, tol_update=1e-8, mode=0)
     assert ((X - Y).norm() / Y.norm()).item() <= 1e-7
     prob.close()
+
+
+@pytest.mark.parametrize("N,L,p,q", [(4, 1, 1, 2), (17, 1, 2, 4), (18, 4, 1, 3), (33, 2, 3, 7)])
+def test_coefficient_rows_at_ragged_sizes(gpu, N, L, p, q):
+    """Residual and Jacobian where the coefficient kernel's blocks of elements
+    are cut short, rows have few triples, and the input order exceeds 2 p;
+    the bounds of the tests above."""
+    import torch
+    import paper_2310_14649_gb300 as sg
+    prob = sg.sg_setup(N, L, p, q, sigma2=0.3, bx=0.5, by=0.5)
+    ref = galerkin.build(N, L, p, q, 0.3, 0.5, 0.5)
+    nl = newton.Problem(ref)
+    U, X = 0.8 * random_block(ref.n, ref.P, seed=97), random_block(ref.n, ref.P, seed=98)
+    Ud = dev(U, torch.float64)
+    Rd = torch.full_like(Ud, float("nan"))
+    sg.sg_nonlinear_residual(prob, Ud, Rd)
+    Rr = nl.residual(U)
+    assert np.max(np.abs(host(Rd, ref.n) - Rr)) <= 1e-12 * np.max(np.abs(Rr))
+    for dtype, tol in ((torch.float64, 1e-12), (torch.float32, 2e-5)):
+        Uq, Xq = (host(dev(B, dtype), ref.n) for B in (U, X))
+        Yd = torch.full_like(dev(X, dtype), float("nan"))
+        sg.sg_nonlinear_jacobian_apply(prob, dev(U, dtype), dev(X, dtype), Yd)
+        Yr = galerkin.from_vec(nl.jacobian(Uq) @ galerkin.to_vec(Xq), ref.n, ref.P)
+        assert np.max(np.abs(host(Yd, ref.n) - Yr)) <= tol * np.max(np.abs(Yr))
