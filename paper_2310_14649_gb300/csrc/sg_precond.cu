@@ -276,6 +276,112 @@ __global__ void k_ras_local(const T* __restrict__ R, int64_t ld, T* __restrict__
 }
 
 // ---------------------------------------------------------------------------
+// FP64 local solve.  With D_l the Schur complement of line l and A_l the
+// (diagonal) coupling of its nodes with the line below,
+//   forward   z_l = r_l - A_l v_{l-1},  v_l = D_l^{-1} z_l,
+//   backward  x_l = v_l - D_l^{-1} A_{l+1} x_{l+1}:
+// one dense W x W product a line and sweep instead of the two (one of them
+// triangular) of the Cholesky factors, and the FP64 units (2 FMAs per clock
+// and SM) bound it: every other instruction is free, so a thread owns one
+// (slot, mode) and loads both factors of each FMA from shared memory.  Slots
+// are aligned over a box's lines, so z_l takes only the thread's own v_{l-1}
+// and a line needs one barrier.  The line matrices come through a ring of
+// cp.async copies.  Q lanes share a slot's sum where there is too little work
+// to cover the latency of the chain.  256^2, 64 boxes of 36 x 36 nodes, P =
+// 35: 1.42 ms with the Cholesky factors, now 0.57 (the operations alone
+// 0.36).
+// ---------------------------------------------------------------------------
+template <int Q>
+__global__ void k_ras_lines64(const double* __restrict__ R, int64_t ld, double* __restrict__ Z, int P, int MC, int W,
+                              int Lm, const int* __restrict__ nlines, const int* __restrict__ gidx,
+                              const double* __restrict__ sinv, const double* __restrict__ aoff, int stages) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int WW = W * W, VS = MC * W;
+  double* ring = reinterpret_cast<double*>(smem_raw);  // [stages][W][W]
+  double* v = ring + stages * WW;                      // [Lm][MC][W]
+  double* zb = v + Lm * VS;                            // [2][MC][W]
+  const int box = blockIdx.x, nl = nlines[box];
+  const int q = threadIdx.x % Q, item = threadIdx.x / Q;
+  const bool act = item < VS;
+  const int m = act ? item / W : 0, t = act ? item - m * W : 0, a = blockIdx.y * MC + m;
+  const bool mode = act && a < P;
+  const int* gi = gidx + size_t(box) * Lm * W + t;
+  const double* ao = aoff + size_t(box) * Lm * W + t;
+  const double* S = sinv + size_t(box) * Lm * WW;
+  const int steps = 2 * nl - 1;
+  auto line_of = [&](int st) { return st < nl ? st : 2 * nl - 2 - st; };
+  auto stage = [&](int st) {
+    if (st < steps) {
+      const double* src = S + size_t(line_of(st)) * WW;
+      double* dst = ring + (st % stages) * WW;
+      for (int c = threadIdx.x; c < WW / 2; c += blockDim.x) cp_async16(dst + 2 * c, src + 2 * c);
+    }
+    cp_async_commit();
+  };
+  // the residual of line l (and the node's index), the coupling below it
+  auto load_r = [&](int g) { return mode && g >= 0 ? R[int64_t(a) * ld + (g & kIdxMask)] : 0.0; };
+  for (int st = 0; st < stages - 1; ++st) stage(st);
+  double in = load_r(gi[0]), own = 0.0;
+  int g1 = nl > 1 ? gi[W] : -1;
+  for (int st = 0; st < steps; ++st) {
+    const int l = line_of(st);
+    const bool fwd = st < nl;
+    // the next line's values travel during this line's product
+    double r1 = 0.0, a1 = 0.0;
+    if (st + 1 < nl) {
+      r1 = load_r(g1);
+      a1 = ao[(st + 1) * W];
+      g1 = st + 2 < nl ? gi[(st + 2) * W] : -1;
+    } else if (st + 1 < steps) {
+      a1 = ao[(line_of(st + 1) + 1) * W];
+    }
+    double* z = zb + (st & 1) * VS;
+    if (act && q == 0) z[item] = in;
+    cp_async_wait_dyn(stages - 2);
+    __syncthreads();
+    stage(st + stages - 1);  // into the buffer of the step before
+    if (act) {
+      const double* M = ring + (st % stages) * WW + t;
+      const double* zm = z + m * W;
+      double c0 = 0.0, c1 = 0.0;
+      int u = q;
+      for (; u + 3 * Q < W; u += 4 * Q) {
+        c0 = fma(M[u * W], zm[u], c0);
+        c1 = fma(M[(u + Q) * W], zm[u + Q], c1);
+        c0 = fma(M[(u + 2 * Q) * W], zm[u + 2 * Q], c0);
+        c1 = fma(M[(u + 3 * Q) * W], zm[u + 3 * Q], c1);
+      }
+      for (; u < W; u += Q) c0 = fma(M[u * W], zm[u], c0);
+      own = c0 + c1;
+    }
+#pragma unroll
+    for (int off = 1; off < Q; off <<= 1) own += __shfl_xor_sync(0xffffffffu, own, off);
+    if (act) {
+      if (!fwd) own = v[l * VS + item] - own;
+      if (q == 0 && fwd) v[l * VS + item] = own;
+      if (q == 0 && mode && st >= nl - 1) {
+        const int g = gi[l * W];
+        if (g >= 0 && (g & kOwnedBit)) Z[int64_t(a) * ld + (g & kIdxMask)] = own;
+      }
+    }
+    in = st + 1 < nl ? r1 - a1 * own : a1 * own;
+  }
+}
+
+__global__ void k_line_inverses(int W, const int2* __restrict__ line, const double* __restrict__ linv,
+                                double* __restrict__ S) {
+  const int2 dl = line[blockIdx.x];
+  const double* L = linv + size_t(blockIdx.x) * W * W;
+  for (int e = threadIdx.x; e < W * W; e += blockDim.x) {
+    const int t = e / W - dl.x, u = e % W - dl.x;
+    double s = 0.0;
+    if (t >= 0 && t < dl.y && u >= 0 && u < dl.y)
+      for (int k = max(t, u); k < dl.y; ++k) s = fma(L[k * W + t], L[k * W + u], s);
+    S[size_t(blockIdx.x) * W * W + e] = s;
+  }
+}
+
+// ---------------------------------------------------------------------------
 // RAS local solve on the tensor cores (FP32 data).  Each line step is two
 // small dense products, (W x W)(W x MC): the off-diagonal coupling and the
 // triangular inverse (zero above its diagonal, so the full tile product is
@@ -737,6 +843,58 @@ sg_status spmm(const DevCsr& A, const T* X, int64_t ldx, const T* B, int64_t ldb
   return SG_OK;
 }
 
+sg_status ras_line_inverses(RasData& R, const std::vector<int2>& line) {
+  DevBuf dl;
+  SG_TRY(dl.alloc(line.size() * sizeof(int2)));
+  SG_CUDA(cudaMemcpy(dl.ptr, line.data(), line.size() * sizeof(int2), cudaMemcpyHostToDevice));
+  SG_TRY(R.sinv64.alloc(line.size() * R.wmax * R.wmax * 8));
+  k_line_inverses<<<unsigned(line.size()), 256>>>(R.wmax, dl.as<int2>(), R.linv64.as<double>(), R.sinv64.as<double>());
+  note_launch();
+  SG_CUDA(cudaGetLastError());
+  SG_CUDA(cudaDeviceSynchronize());
+  return SG_OK;
+}
+
+// FP64 local solves over the lines' inverses; false when a box's lines do not
+// fit in shared memory with one mode (the kernel over the Cholesky factors
+// keeps what it takes)
+static bool ras_lines64(const Precond& pc, int P, const double* R, int64_t ld, double* Z, cudaStream_t st) {
+  const RasData& D = pc.ras;
+  if (!D.sinv64.ptr) return false;
+  const int W = D.wmax, Lm = D.lmax;
+  const int stages = pc.ras_stages > 0 ? std::max(2, std::min(pc.ras_stages, kRasMaxStages)) : kRasStages;
+  const size_t per_mode = (size_t(Lm) + 2) * W * 8, fixed = size_t(stages) * W * W * 8;
+  if (fixed + per_mode > 227 * 1024 || W > 1024) return false;
+  int most = std::min<int64_t>({P, 1024 / W, int64_t((227 * 1024 - fixed) / per_mode)});
+  if (pc.ras_modes > 0) most = std::min(most, pc.ras_modes);
+  // an SM's CTAs share its FP64 units: the split of the modes with the fewest
+  // CTAs per SM x modes (64 boxes, 35 modes: 7 CTAs of 5, three an SM)
+  int MC = most;
+  int64_t best = 0;
+  for (int mc = most; mc >= 1; --mc) {
+    const int64_t cost = (int64_t(D.nbox) * ((P + mc - 1) / mc) + 151) / 152 * mc;
+    if (best == 0 || cost < best) {
+      best = cost;
+      MC = mc;
+    }
+  }
+  const int nchunk = (P + MC - 1) / MC;
+  const size_t smem = fixed + MC * per_mode;
+  // fewer than eight warps an SM: four lanes share a slot
+  const int64_t warps = int64_t(D.nbox) * nchunk * ((W * MC + 31) / 32);
+  const dim3 grid(unsigned(D.nbox), unsigned(nchunk));
+  const int Q = warps < 8 * 152 && 4 * W * MC <= 1024 ? 4 : 1;
+  const unsigned threads = unsigned((Q * W * MC + 31) & ~31);
+  if (Q == 4)
+    k_ras_lines64<4><<<grid, threads, smem, st>>>(R, ld, Z, P, MC, W, Lm, D.d_nlines.as<int>(), D.d_gidx64.as<int>(),
+                                                  D.sinv64.as<double>(), D.aoff64.as<double>(), stages);
+  else
+    k_ras_lines64<1><<<grid, threads, smem, st>>>(R, ld, Z, P, MC, W, Lm, D.d_nlines.as<int>(), D.d_gidx64.as<int>(),
+                                                  D.sinv64.as<double>(), D.aoff64.as<double>(), stages);
+  note_launch();
+  return true;
+}
+
 template <typename T>
 sg_status ras_apply(const Precond& pc, int64_t n, int P, const T* R, int64_t ld, T* Z, cudaStream_t st,
                     bool transform, Profiler* prof) {
@@ -823,9 +981,14 @@ sg_status ras_apply(const Precond& pc, int64_t n, int P, const T* R, int64_t ld,
   size_t slot = 0;
   const bool timed = prof && prof->on;
   if (timed) SG_TRY(prof->begin(sizeof(T) == 8 ? 5 : 4, st, slot));
-  k_ras_local<T><<<grid, threads, smem, st>>>(R, ld, Z, P, MC, D.wmax, D.lmax, D.d_nlines.as<int>(),
-                                              D.d_gidx.as<int>(), dv<T>(D.linv64, D.linv32),
-                                              dv<T>(D.loff64, D.loff32), stages); note_launch();
+  bool done = false;
+  if constexpr (sizeof(T) == 8) done = ras_lines64(pc, P, R, ld, Z, st);
+  if (!done) {
+    k_ras_local<T><<<grid, threads, smem, st>>>(R, ld, Z, P, MC, D.wmax, D.lmax, D.d_nlines.as<int>(),
+                                                D.d_gidx.as<int>(), dv<T>(D.linv64, D.linv32),
+                                                dv<T>(D.loff64, D.loff32), stages);
+    note_launch();
+  }
   SG_CUDA(cudaGetLastError());
   if (timed) SG_TRY(prof->end(slot, st));
   if (transform) SG_TRY(node_transform<T>(Z, ld, n, P, dv<T>(pc.gtinv64, pc.gtinv32), st));
@@ -1325,6 +1488,8 @@ sg_status kernel_attrs_init() {
   if (done) return SG_OK;
   SG_CUDA(cudaFuncSetAttribute(k_ras_local<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
   SG_CUDA(cudaFuncSetAttribute(k_ras_local<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+  SG_CUDA(cudaFuncSetAttribute(k_ras_lines64<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+  SG_CUDA(cudaFuncSetAttribute(k_ras_lines64<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
   SG_CUDA(cudaFuncSetAttribute(k_node_transform<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
   SG_CUDA(cudaFuncSetAttribute(k_node_transform<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
   SG_TRY(apply_attrs_init());

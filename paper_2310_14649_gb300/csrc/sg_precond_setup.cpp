@@ -269,7 +269,37 @@ static sg_status setup_ras(sg_problem* pr, Precond& pc) {
   SG_CUDA(cudaMemcpy(R.loff32.ptr, loff32.data(), loff32.size() * 4, cudaMemcpyHostToDevice));
   SG_CUDA(cudaMemcpy(R.d_gidx.ptr, gidx.data(), gidx.size() * 4, cudaMemcpyHostToDevice));
   SG_CUDA(cudaMemcpy(R.d_nlines.ptr, R.nlines.data(), R.nlines.size() * 4, cudaMemcpyHostToDevice));
-  return SG_OK;
+  // aligned slots of the FP64 solve
+  std::vector<int2> line(size_t(R.nbox) * Lm, make_int2(0, 0));
+  std::vector<int32_t> gidx64(size_t(R.nbox) * Lm * W, -1);
+  std::vector<double> aoff(gidx64.size(), 0.0);
+  bool fits = true;
+  for (int b = 0; b < R.nbox; ++b) {
+    int32_t x = m, xe = 0;
+    for (auto [j, x0, len] : lines[b]) {
+      x = std::min(x, x0);
+      xe = std::max(xe, x0 + len);
+    }
+    fits = fits && xe - x <= W;
+    for (int l = 0; fits && l < R.nlines[b]; ++l) {
+      auto [j, x0, len] = lines[b][l];
+      line[size_t(b) * Lm + l] = make_int2(x0 - x, len);
+      for (int t = 0; t < len; ++t) {
+        const int64_t r = int64_t(j) * m + x0 + t;
+        const size_t at = (size_t(b) * Lm + l) * W + (x0 - x) + t;
+        gidx64[at] = gidx[(size_t(b) * Lm + l) * W + t];
+        if (l > 0 && x0 + t >= lines[b][l - 1][1] && x0 + t < lines[b][l - 1][1] + lines[b][l - 1][2])
+          aoff[at] = a0(r, r - m);
+      }
+    }
+  }
+  R.sinv64.free_();
+  if (!fits) return SG_OK;
+  SG_TRY(R.aoff64.alloc(aoff.size() * 8));
+  SG_TRY(R.d_gidx64.alloc(gidx64.size() * 4));
+  SG_CUDA(cudaMemcpy(R.aoff64.ptr, aoff.data(), aoff.size() * 8, cudaMemcpyHostToDevice));
+  SG_CUDA(cudaMemcpy(R.d_gidx64.ptr, gidx64.data(), gidx64.size() * 4, cudaMemcpyHostToDevice));
+  return ras_line_inverses(R, line);
 }
 
 // --------------------------------------------------------------------------

@@ -69,6 +69,10 @@ struct RasData {
   DevBuf d_nlines;                         // int32 nbox
   DevBuf d_gidx;                           // int32 nbox x lmax x wmax (-1 pad, owned | 1<<30)
   DevBuf linv64, loff64, linv32, loff32;   // nbox x lmax x wmax x wmax
+  // the FP64 solve's form (k_ras_lines64), slots aligned over a box's lines
+  // (slot = column - leftmost column of the box): inverses D_l^{-1} of the
+  // lines' Schur complements, couplings with the line below, node indices
+  DevBuf sinv64, aoff64, d_gidx64;         // nbox x lmax x wmax x wmax, nbox x lmax x wmax (twice)
   // explicit local inverses (ras_kernel 2): the owned rows of A_{0,i}^{-1}
   // in FP32 as chunks of 128 rows x 32 overlapped nodes in the tensor-core
   // operand layout (tiles of 128 owned rows in box order, chunks in node
@@ -146,6 +150,8 @@ struct CoarsePlan {
 };
 
 sg_status precond_setup_host(sg_problem* pr, Precond& pc);
+// sinv64 from linv64; `line`: first slot and length of every line (nbox x lmax)
+sg_status ras_line_inverses(RasData& R, const std::vector<int2>& line);
 // the dense part of a folded hierarchy, from the FP64 V-cycle applied to the
 // unit vectors of level lf; synchronous
 sg_status amg_fold_dense(AmgHier& H);

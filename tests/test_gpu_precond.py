@@ -416,3 +416,28 @@ def test_amg_fold(gpu, N, L, p, flux):
         it[kernel] = (info["outer_it"], info["inner_it"])
     assert abs(it[0][0] - it[1][0]) <= 1 and abs(it[0][1] - it[1][1]) <= 2 + it[1][1] // 20, it
     assert ((X[0] - X[1]).norm() / X[1].norm()).item() <= 1e-6
+
+
+@pytest.mark.parametrize("N,L,p,sx,sy,overlap,modes", [
+    (32, 1, 1, 2, 2, 1, 0),     # four lanes a slot
+    (26, 2, 3, 3, 1, 3, 0),     # lines longer than the box has, a ragged row of boxes
+    (64, 3, 2, 9, 7, 2, 0),     # many small boxes, uneven
+    (64, 3, 4, 3, 3, 2, 0),     # one lane a slot, several modes a CTA
+    (64, 3, 4, 3, 3, 2, 4),     # the last CTA of a box cut short
+    (8, 2, 2, 7, 7, 2, 0),      # boxes clipped on all sides
+])
+def test_ras_fp64_lines(gpu, N, L, p, sx, sy, overlap, modes):
+    """The FP64 local solves over the lines' inverses at the shapes that
+    select its variants, against the oracle's local solves; bound of the FP64
+    test above."""
+    import torch
+    import paper_2310_14649_gb300 as sg
+    prob = sg.sg_setup(N, L, p, 2 * p, sigma2=0.3, bx=0.5, by=0.5)
+    sg.sg_precond_setup(prob, sx, sy, overlap, ras_modes=modes)
+    ref = galerkin.build(N, L, p, 2 * p, sigma2=0.3, bx=0.5, by=0.5)
+    parts = ras.partitions(ref.A(0), ref.N, sx, sy, overlap)
+    solvers = ras.local_solvers(ref.A(0), parts)
+    X = random_block(ref.n, ref.P, seed=41)
+    Y, Xq = run(prob, sg.PC_RAS_LOCAL, X, ref.n, torch.float64)
+    Yr = ras.apply_ras(parts, solvers, Xq)
+    assert np.max(np.abs(Y - Yr)) <= 1e-11 * np.max(np.abs(Yr))
