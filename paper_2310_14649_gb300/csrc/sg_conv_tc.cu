@@ -240,27 +240,34 @@ __global__ void __launch_bounds__(128) k_conv_tc(const bf16* __restrict__ X, con
 //     db[co] = sum_pixels G[y][x][co],
 // as one implicit GEMM per tap row dy: D_dy[(dx, ci)][co] = sum_x A[(dx, ci)][x]
 // B[co][x], M = 3 C_in shifted input channels (+ a row of ones that yields
-// the bias gradient, the rest zero) padded to 128, N = C_out, K = the 128
+// the bias gradient, the rest unused) padded to 128, N = C_out, K = the 128
 // pixels of one image-row segment.  A CTA walks down a strip of rows of one
-// 128-pixel column segment: input row y + 1 is transposed into one of three
-// rolling shared-memory slots (pixels along K, three copies shifted by dx),
-// so the rows y - 1, y and y + 1 that output row y needs are resident, and
-// the output-gradient row y is transposed into B.  The three accumulators
-// (one per dy) stay in tensor memory over the whole strip; the epilogue adds
-// them to the FP32 gradient with atomics.  Shared-memory operands are
-// K-major in the canonical layout (8-row x 16-byte core matrices; planes of
-// 8 pixels, rows 16 bytes apart).
-constexpr int kWgRows = 128;       // M rows of the A operand (padded)
+// 128-pixel column segment with input rows y - 1, y and y + 1 resident in
+// three rolling shared-memory slots.  The three accumulators (one per dy)
+// stay in tensor memory over the whole strip; the epilogue adds them to the
+// FP32 gradient with atomics.  Both operands are MN-major (pixels along K,
+// the eight channels of a 16-byte piece contiguous, planes of eight channels
+// PLANE bytes apart), which is how the images lie in memory: a row is staged
+// as 16-byte pieces, three copies shifted by one pixel for the taps dx, from
+// registers that were loaded while the MMAs of the row before ran.  K-major
+// operands took a transpose of 2-byte stores (2.7 of a training
+// step's 4.2 ms on 32 images of 255 x 255, the tensor pipe 8 % active; now
+// 0.81 ms).  PLANE is 128
+// pixels and 32 bytes: the four pieces of a pixel and its neighbour's land in
+// distinct banks.
 constexpr int kWgPix = 128;        // pixels per chunk (K)
 
 template <int CI, int CO>
 struct WgShape {
-  static constexpr int PLANE_A = kWgRows * 16;            // bytes per 8-pixel plane of A
-  static constexpr int SLOT = (kWgPix / 8) * PLANE_A;     // bytes per rolling input slot
-  static constexpr int PLANE_B = CO * 16;
-  static constexpr int SB = (kWgPix / 8) * PLANE_B;
+  static constexpr int PLANE = kWgPix * 16 + 32;          // bytes per plane of 8 channels
   static constexpr int ONES = 3 * CI;                     // the row of ones (bias gradient)
-  static constexpr int SMEM = 3 * SLOT + SB + 16;
+  static constexpr int NPA = ONES / 8 + 1;                // planes of a slot: the shifted copies, the ones
+  static constexpr int SLOT = NPA * PLANE;                // bytes per rolling input slot
+  static constexpr int SB = CO / 8 * PLANE;
+  // rows past ONES (planes NPA .. 15) read what follows the slot: their
+  // results are not used, their addresses stay inside the allocation
+  static constexpr int TAIL = (16 - NPA) * PLANE > SB ? (16 - NPA) * PLANE : SB;
+  static constexpr int SMEM = 3 * SLOT + TAIL + 16;
 };
 
 template <int CI, int CO>
@@ -271,50 +278,58 @@ __global__ void __launch_bounds__(128) k_wgrad_tc(const bf16* __restrict__ X, co
   extern __shared__ __align__(128) uint8_t sm[];
   uint8_t* sA = sm;
   uint8_t* sB = sm + 3 * S::SLOT;
-  uint64_t* mbar = reinterpret_cast<uint64_t*>(sB + S::SB);
+  uint64_t* mbar = reinterpret_cast<uint64_t*>(sB + S::TAIL);
   uint32_t* tslot = reinterpret_cast<uint32_t*>(mbar + 1);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int x0 = blockIdx.x * kWgPix, img = blockIdx.z;
   const int ya = blockIdx.y * rows_per_cta, yb = min(H, ya + rows_per_cta);
   const bf16* Ximg = X + size_t(img) * H * W * CI;
   const bf16* Gimg = G + size_t(img) * H * W * CO;
-  // element (row m, pixel k) of slot s / of B (row co, pixel k)
-  auto a_off = [&](int s, int m, int k) { return s * S::SLOT + (k >> 3) * S::PLANE_A + (m >> 3) * 128 + (m & 7) * 16 + (k & 7) * 2; };
-  auto b_off = [&](int co, int k) { return (k >> 3) * S::PLANE_B + (co >> 3) * 128 + (co & 7) * 16 + (k & 7) * 2; };
-  // zero every slot, then the row of ones
-  for (int e = tid; e < 3 * S::SLOT / 16; e += 128) reinterpret_cast<uint4*>(sA)[e] = make_uint4(0, 0, 0, 0);
-  __syncthreads();
-  const bf16 one = __float2bfloat16(1.0f);
+  // the planes of ones: channel 0 of every pixel
   for (int e = tid; e < 3 * kWgPix; e += 128)
-    *reinterpret_cast<bf16*>(sA + a_off(e / kWgPix, S::ONES, e % kWgPix)) = one;
-  // input row r (zero outside the image) into slot (r + 3) % 3: position q
-  // (x = x0 + q - 1) feeds copies dx with pixel k = q - dx
-  auto stage_x = [&](int r) {
-    const int s = (r + 3) % 3;
-    for (int e = tid; e < (kWgPix + 2) * (CI / 8); e += 128) {
-      const int q = e / (CI / 8), c8 = e % (CI / 8);
-      const int x = x0 + q - 1;
-      uint4 v = make_uint4(0, 0, 0, 0);
-      if (r >= 0 && r < H && x >= 0 && x < W) v = *reinterpret_cast<const uint4*>(Ximg + (size_t(r) * W + x) * CI + 8 * c8);
-      const bf16* hv = reinterpret_cast<const bf16*>(&v);
+    *reinterpret_cast<uint4*>(sA + (e / kWgPix) * S::SLOT + (S::ONES / 8) * S::PLANE + (e % kWgPix) * 16) =
+        make_uint4(uint32_t(__bfloat16_as_ushort(__float2bfloat16(1.0f))), 0, 0, 0);
+  // 16-byte pieces of a row: piece e = (position q, channels 8 c8 ..); input
+  // position q is x = x0 + q - 1 and feeds the copies dx with pixel k = q - dx
+  constexpr int CX = CI / 8, CG = CO / 8;
+  constexpr int EX = (kWgPix + 2) * CX, EG = kWgPix * CG;
+  constexpr int LX = (EX + 127) / 128, LG = EG / 128;
+  uint4 vx[LX], vg[LG];
+  auto load_x = [&](int r) {  // zero outside the image
+#pragma unroll
+    for (int u = 0; u < LX; ++u) {
+      const int e = tid + 128 * u, x = x0 + e / CX - 1;
+      vx[u] = make_uint4(0, 0, 0, 0);
+      if (e < EX && r >= 0 && r < H && x >= 0 && x < W)
+        vx[u] = *reinterpret_cast<const uint4*>(Ximg + (size_t(r) * W + x) * CI + 8 * (e % CX));
+    }
+  };
+  auto load_g = [&](int y) {
+#pragma unroll
+    for (int u = 0; u < LG; ++u) {
+      const int e = tid + 128 * u, x = x0 + e / CG;
+      vg[u] = make_uint4(0, 0, 0, 0);
+      if (x < W) vg[u] = *reinterpret_cast<const uint4*>(Gimg + (size_t(y) * W + x) * CO + 8 * (e % CG));
+    }
+  };
+  auto store_x = [&](int r) {
+    uint8_t* slot = sA + ((r + 3) % 3) * S::SLOT;
+#pragma unroll
+    for (int u = 0; u < LX; ++u) {
+      const int e = tid + 128 * u, q = e / CX, c8 = e % CX;
 #pragma unroll
       for (int dx = 0; dx < 3; ++dx) {
         const int k = q - dx;
-        if (k < 0 || k >= kWgPix) continue;
-#pragma unroll
-        for (int c = 0; c < 8; ++c) *reinterpret_cast<bf16*>(sA + a_off(s, dx * CI + 8 * c8 + c, k)) = hv[c];
+        if (e < EX && k >= 0 && k < kWgPix)
+          *reinterpret_cast<uint4*>(slot + (dx * CX + c8) * S::PLANE + k * 16) = vx[u];
       }
     }
   };
-  auto stage_g = [&](int y) {
-    for (int e = tid; e < kWgPix * (CO / 8); e += 128) {
-      const int k = e / (CO / 8), c8 = e % (CO / 8);
-      const int x = x0 + k;
-      uint4 v = make_uint4(0, 0, 0, 0);
-      if (x < W) v = *reinterpret_cast<const uint4*>(Gimg + (size_t(y) * W + x) * CO + 8 * c8);
-      const bf16* hv = reinterpret_cast<const bf16*>(&v);
+  auto store_g = [&]() {
 #pragma unroll
-      for (int c = 0; c < 8; ++c) *reinterpret_cast<bf16*>(sB + b_off(8 * c8 + c, k)) = hv[c];
+    for (int u = 0; u < LG; ++u) {
+      const int e = tid + 128 * u;
+      *reinterpret_cast<uint4*>(sB + (e % CG) * S::PLANE + (e / CG) * 16) = vg[u];
     }
   };
   if (warp == 0) {
@@ -328,15 +343,19 @@ __global__ void __launch_bounds__(128) k_wgrad_tc(const bf16* __restrict__ X, co
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
   if (ya < yb) {
-    stage_x(ya - 1);
-    stage_x(ya);
+    load_x(ya - 1);
+    store_x(ya - 1);
+    load_x(ya);
+    store_x(ya);
+    load_x(ya + 1);
+    load_g(ya);
   }
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
   const uint32_t tmem = *tslot;
   const uint32_t a0 = smem_u32(sA), b0 = smem_u32(sB);
-  constexpr uint32_t idesc = inst_desc(128, CO);
+  constexpr uint32_t idesc = inst_desc(128, CO) | (1u << 15) | (1u << 16);  // A and B MN-major
   auto poll = [&](int limit, uint32_t parity) {
     uint32_t done = 0;
     for (int it = 0; it < limit && !done; ++it)
@@ -350,8 +369,8 @@ __global__ void __launch_bounds__(128) k_wgrad_tc(const bf16* __restrict__ X, co
   bool ok = true;
   uint32_t phase = 0;
   for (int y = ya; y < yb; ++y) {
-    stage_x(y + 1);
-    stage_g(y);
+    store_x(y + 1);
+    store_g();
     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
@@ -362,8 +381,9 @@ __global__ void __launch_bounds__(128) k_wgrad_tc(const bf16* __restrict__ X, co
         const int s = (y + dy - 1 + 3) % 3;
 #pragma unroll
         for (int kc = 0; kc < kWgPix / 16; ++kc) {
-          const uint64_t ad = mat_desc(a0 + uint32_t(s * S::SLOT + 2 * kc * S::PLANE_A), S::PLANE_A, 128);
-          const uint64_t bd = mat_desc(b0 + uint32_t(2 * kc * S::PLANE_B), S::PLANE_B, 128);
+          // eight pixels of eight channels are 128 bytes; next pixels LBO, next channels SBO
+          const uint64_t ad = mat_desc(a0 + uint32_t(s * S::SLOT + 256 * kc), 128, S::PLANE);
+          const uint64_t bd = mat_desc(b0 + uint32_t(256 * kc), 128, S::PLANE);
           const uint32_t acc = (y > ya || kc > 0) ? 1u : 0u;
           asm volatile(
               "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
@@ -375,6 +395,10 @@ __global__ void __launch_bounds__(128) k_wgrad_tc(const bf16* __restrict__ X, co
       asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
                        smem_u32(mbar))
                    : "memory");
+    }
+    if (y + 1 < yb) {
+      load_x(y + 2);
+      load_g(y + 1);
     }
     // the MMAs read the slots and B: wait before the next staging
     const uint32_t done = poll(wait_limit, phase);

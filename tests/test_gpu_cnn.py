@@ -286,3 +286,26 @@ def test_network_operators_in_precond_apply(pair):
     Zlr = 0.75 * np.linalg.solve(Gt, Zn)
     assert np.max(np.abs(Zl - Zlr)) <= 1e-5 * np.max(np.abs(Zlr))
     sg.sg_precond_set_smoother(prob, 0)
+
+
+@pytest.mark.parametrize("N,images", [(4, 1), (18, 5), (128, 2), (129, 2), (130, 2), (258, 1)])
+def test_weight_gradient_segments(gpu, N, images):
+    """Weight and bias gradients where a row of pixels fills its last
+    128-pixel segment, misses it by one or starts a new one, and where strips
+    are a few rows: tcgen05 and mma.sync form the same sums of BF16 products
+    from activations that differ by BF16 rounding (2^-8; bound of the test of
+    the forward kernels)."""
+    import torch
+    import paper_2310_14649_gb300 as sg
+    prob = sg.sg_setup(N, 1, images - 1, 2 * images, sigma2=0.3, bx=0.5, by=0.5)
+    sg.sg_cnn_set_weights(prob, params_for(14))
+    R, Z = (torch.from_numpy(random_block(prob.n, images, seed=s).T.copy()).float().cuda() for s in (79, 80))
+    out = []
+    for kernel in (1, 0):
+        sg.sg_cnn_set_kernel(prob, kernel)
+        sg.sg_cnn_train_step(prob, R, Z, update=False)
+        out.append(sg.cnn_unflatten(sg.sg_cnn_get_weights(prob, gradient=True)))
+    for (gW, gb), (hW, hb) in zip(*out):
+        assert np.linalg.norm(gW - hW) <= 1e-2 * np.linalg.norm(hW)
+        assert np.linalg.norm(gb - hb) <= 1e-2 * np.linalg.norm(hb)
+    prob.close()
