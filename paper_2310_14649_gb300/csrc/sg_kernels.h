@@ -30,8 +30,10 @@ sg_status node_transform(T* Z, int64_t ld, int64_t n, int P, const T* M, cudaStr
 // Kronecker factor M fused when transform
 bool ras_inverse_supported(int P);
 sg_status ras_inverse_build(sg_problem* pr, Precond& pc, cudaStream_t st);
-sg_status ras_inverse_apply(const Precond& pc, int P, const float* R, int64_t ld, float* Z, const float* M,
-                            bool transform, int wait_limit, cudaStream_t st);
+sg_status ras_inverse_apply(const Precond& pc, int P, const float* R, int64_t ldr, float* Z, int64_t ldz,
+                            const float* M, bool transform, int wait_limit, cudaStream_t st);
+// whether the blocks R and Z (P rows each) share no memory, as the apply needs
+bool ras_inverse_disjoint(int P, const float* R, int64_t ldr, const float* Z, int64_t ldz);
 sg_status ras_inverse_check(const Precond& pc, cudaStream_t st);
 template <typename T>
 // one V-cycle from a zero guess on w.b[l0], levels l0 and below

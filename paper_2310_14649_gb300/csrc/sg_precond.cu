@@ -904,7 +904,7 @@ sg_status ras_apply(const Precond& pc, int64_t n, int P, const T* R, int64_t ld,
     size_t slot = 0;
     const bool timed = prof && prof->on;
     if (timed) SG_TRY(prof->begin(4, st, slot));
-    SG_TRY(ras_inverse_apply(pc, P, reinterpret_cast<const float*>(R), ld, reinterpret_cast<float*>(Z),
+    SG_TRY(ras_inverse_apply(pc, P, reinterpret_cast<const float*>(R), ld, reinterpret_cast<float*>(Z), ld,
                              reinterpret_cast<const float*>(pc.gtinv32.ptr), transform, pc.wait_limit, st));
     if (timed) SG_TRY(prof->end(slot, st));
     return SG_OK;

@@ -536,7 +536,7 @@ __global__ void __launch_bounds__(kPackThreads) k_ras_inv_pack(const float* __re
     const int c = int(e % P);
     const int64_t r = e / P;
     const int g = tile_owned[int64_t(split_tile[r / 128]) * 128 + int(r % 128)];
-    if (g >= 0) a.Z[int64_t(c) * ld + g] = 0.f;
+    if (g >= 0) a.Z[int64_t(c) * a.ld + g] = 0.f;
   }
 }
 
@@ -751,8 +751,12 @@ sg_status ras_inverse_build(sg_problem* pr, Precond& pc, cudaStream_t st) {
   return SG_OK;
 }
 
-sg_status ras_inverse_apply(const Precond& pc, int P, const float* R, int64_t ld, float* Z, const float* M,
-                            bool transform, int wait_limit, cudaStream_t st) {
+bool ras_inverse_disjoint(int P, const float* R, int64_t ldr, const float* Z, int64_t ldz) {
+  return R >= Z + int64_t(P) * ldz || Z >= R + int64_t(P) * ldr;
+}
+
+sg_status ras_inverse_apply(const Precond& pc, int P, const float* R, int64_t ldr, float* Z, int64_t ldz,
+                            const float* M, bool transform, int wait_limit, cudaStream_t st) {
   const RasData& D = pc.ras;
   if (transform && !M) {
     set_error("ras_inverse_apply: the Kronecker factor is not on the device yet");
@@ -763,15 +767,14 @@ sg_status ras_inverse_apply(const Precond& pc, int P, const float* R, int64_t ld
     return SG_ERR_ARG;
   }
   // the pack kernel reads R while it zeroes rows of Z
-  const float *r0 = R, *r1 = R + int64_t(P) * ld, *z0 = Z, *z1 = Z + int64_t(P) * ld;
-  if (r0 < z1 && z0 < r1) {
+  if (!ras_inverse_disjoint(P, R, ldr, Z, ldz)) {
     set_error("ras_inverse_apply: input and output overlap");
     return SG_ERR_ARG;
   }
   const int N = D.inv_n;
   InvArgs a = inv_args(D);
   a.Z = Z;
-  a.ld = ld;
+  a.ld = ldz;
   a.ainv = dp<float>(D.d_inv);
   a.bpack = dp<float>(D.d_inv_bpack);
   a.M = M;
@@ -805,7 +808,7 @@ sg_status ras_inverse_apply(const Precond& pc, int P, const float* R, int64_t ld
   a.wait_limit = wait_limit;
   // one block per packed chunk (every chunk's loads in flight at once)
   const int pgrid = int(std::max<int64_t>(1, std::min<int64_t>(D.inv_bchunks, 1 << 30)));
-  k_ras_inv_pack<<<unsigned(pgrid), kPackThreads, 0, st>>>(R, ld, P, N, D.inv_bchunks, a, dp<float>(D.d_inv_bpack),
+  k_ras_inv_pack<<<unsigned(pgrid), kPackThreads, 0, st>>>(R, ldr, P, N, D.inv_bchunks, a, dp<float>(D.d_inv_bpack),
                                                            D.inv_nsplit);
   note_launch();
   SG_CUDA(cudaGetLastError());

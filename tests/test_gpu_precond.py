@@ -441,3 +441,31 @@ def test_ras_fp64_lines(gpu, N, L, p, sx, sy, overlap, modes):
     Y, Xq = run(prob, sg.PC_RAS_LOCAL, X, ref.n, torch.float64)
     Yr = ras.apply_ras(parts, solvers, Xq)
     assert np.max(np.abs(Y - Yr)) <= 1e-11 * np.max(np.abs(Yr))
+
+
+@pytest.mark.parametrize("which", ["PC_SMOOTH", "PC_RAS_LOCAL"])
+def test_smoother_on_callers_blocks(gpu, which):
+    """The explicit local inverses read and write the caller's blocks: any
+    two leading dimensions and alignments, nothing outside the n values of a
+    row, and in place (where the blocks overlap they go through a copy), all
+    with the same bits."""
+    import torch
+    import paper_2310_14649_gb300 as sg
+    prob = sg.sg_setup(32, 2, 2, 4, sigma2=0.3, bx=0.5, by=0.5)
+    sg.sg_precond_setup(prob, 2, 2, 1, ras_kernel=2)
+    op, n, P = getattr(sg, which), prob.n, prob.P
+    X = torch.from_numpy(random_block(n, P, seed=42).T.copy()).float().cuda()
+    Z = torch.zeros_like(X)
+    sg.sg_precond_apply(prob, op, X, Z)
+    pool = torch.full((P, 2 * n + 9), 7.0, dtype=torch.float32, device="cuda")
+    for Rv, Zv in ((pool[:, 1:n + 1], torch.full((P, n + 3), 7.0, device="cuda")), (X, pool[:, :n + 5])):
+        pool.fill_(7.0)
+        Rv[:, :n] = X
+        sg.sg_precond_apply(prob, op, Rv, Zv)
+        assert torch.equal(Zv[:, :n], Z) and bool((Zv[:, n:] == 7.0).all())
+    both = X.clone()
+    sg.sg_precond_apply(prob, op, both, both)
+    assert torch.equal(both, Z)
+    pool[:, :n] = X                     # rows of input and output side by side
+    sg.sg_precond_apply(prob, op, pool[:, :n], pool[:, n:2 * n])
+    assert torch.equal(pool[:, n:2 * n], Z) and torch.equal(pool[:, :n], X)
