@@ -1160,7 +1160,8 @@ sg_status amg_vcycle(const AmgHier& H, AmgWork<T>& w, int P, cudaStream_t st, T*
 // the input and the Kronecker factor, two launches more, are part of the
 // first and the last.  256^2, P = 35 (16,129 coarse unknowns): 83 us of
 // kernels a cycle, now 34 (9.2 + 6.8 + 17.8); a coarse solve at tolerance
-// 1e-5 3.02 ms, now 2.58.
+// 1e-5 3.02 ms, now 2.58.  A hierarchy of one level is the dense product alone
+// (32^2, 225 unknowns: 35 us, now 6).
 // ---------------------------------------------------------------------------
 namespace {
 
@@ -1173,13 +1174,14 @@ constexpr int kDenseRows = 64, kDenseSplit = 8, kDenseModes = 48, kDenseLd = 52;
 // the matrix is 13.7 MB, read once from L2.  b, x: mode-major.
 __global__ void __cluster_dims__(kDenseSplit, 1, 1) __launch_bounds__(128)
     k_fold_dense(int n, int64_t ldd, const float* __restrict__ B, const float* __restrict__ b, int64_t ldb, int P,
-                 float* __restrict__ x, int64_t ldx, int slice) {
+                 float* __restrict__ x, int64_t ldx, int slice, const int* __restrict__ j, int64_t bstride) {
   extern __shared__ __align__(16) float sm_fold[];
   float* Bs = sm_fold;                       // [slice][64]
   float* bs = Bs + slice * kDenseRows;       // [slice][52]: a mode's store along k meets 8 banks
   const int rank = blockIdx.x, row0 = blockIdx.y * kDenseRows, a0 = blockIdx.z * kDenseModes;
   const int k0 = rank * slice, kn = max(0, min(slice, n - k0)), nm = min(kDenseModes, P - a0);
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  if (j) b += int64_t(*j) * bstride;
   for (int q = tid; q < kn * (kDenseRows / 4); q += 128) {
     const int k = q / (kDenseRows / 4), c = q % (kDenseRows / 4);
     // columns row0 .. row0 + 63 of row k (the matrix is symmetric; ldd covers whole tiles)
@@ -1419,10 +1421,13 @@ sg_status amg_fold_apply(const AmgHier& H, AmgWork<float>& w, int P, const float
     const AmgLevel& L = H[F.lf];
     const int n = int(L.n);
     const dim3 grid(kDenseSplit, unsigned((n + kDenseRows - 1) / kDenseRows), unsigned((P + kDenseModes - 1) / kDenseModes));
-    k_fold_dense<<<grid, 128, fold_dense_smem(n), st>>>(n, F.ldd, F.dense.as<float>(), w.b[F.lf], L.ld, P, w.x[F.lf],
-                                                        L.ld, fold_slice(n));
+    const bool all = F.lf == 0;  // the whole cycle
+    k_fold_dense<<<grid, 128, fold_dense_smem(n), st>>>(n, F.ldd, F.dense.as<float>(), all ? b : w.b[F.lf],
+                                                        all ? ldb : L.ld, P, all ? out : w.x[F.lf], all ? ldo : L.ld,
+                                                        fold_slice(n), all ? j : nullptr, bstride);
     note_launch();
     SG_CUDA(cudaGetLastError());
+    if (all) return M ? node_transform<float>(out, ldo, n, P, M, st, Z2, stride2, Z2 ? j : nullptr) : SG_OK;
   }
   for (int l = F.lf - 1; l >= 0; --l) {
     FoldUp p;

@@ -617,9 +617,9 @@ static sg_status setup_amg(AmgHier& H, const HCsr& A0c, bool fold) {
     }
   SG_TRY(H.coarsest_inv64.alloc(inv.size() * 8));
   SG_CUDA(cudaMemcpy(H.coarsest_inv64.ptr, inv.data(), inv.size() * 8, cudaMemcpyHostToDevice));
-  if (!fold || As.size() < 2) return SG_OK;
+  if (!fold || As.size() < 1) return SG_OK;
   AmgFold& F = H.fold;
-  F.lf = 1;
+  F.lf = As.size() > 1 ? 1 : 0;
   while (As[F.lf].n > kFoldMax && F.lf + 1 < int(As.size())) ++F.lf;
   if (As[F.lf].n > kFoldMax) return SG_OK;  // the coarsening stalled: no dense part
   F.Rp.resize(F.lf);

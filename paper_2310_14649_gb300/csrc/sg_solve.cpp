@@ -240,7 +240,7 @@ static sg_status precond_apply_t(sg_problem* pr, int which, const T* Rin, int64_
     ~Restore() { pc.use_cnn = v; }
   } restore{S.pc, prev_cnn};
   // the explicit inverses read and write blocks of any leading dimension: the
-  // four passes over a block below were 50 of 181 us at 256^2, P = 35
+  // four passes over a block below were 35 of 181 us at 256^2, P = 35
   if constexpr (sizeof(T) == 4)
     if ((which == 7 || (which == 1 && !S.pc.use_cnn && !S.pc.harvest.on)) && S.pc.ras_kernel == 2 &&
         S.pc.ras.d_inv.ptr && ras_inverse_disjoint(P, Rin, ldr, Zout, ldz)) {
