@@ -309,3 +309,20 @@ def test_weight_gradient_segments(gpu, N, images):
         assert np.linalg.norm(gW - hW) <= 1e-2 * np.linalg.norm(hW)
         assert np.linalg.norm(gb - hb) <= 1e-2 * np.linalg.norm(hb)
     prob.close()
+
+
+def test_image_scales(gpu):
+    """The network sees r / rms(r), so scaling a residual by a power of two
+    scales the output by it, bit for bit; 2^-100 takes the factor out of the
+    range in which FP32 pairs hold it."""
+    import torch
+    import paper_2310_14649_gb300 as sg
+    prob = sg.sg_setup(34, 2, 1, 2, sigma2=0.3, bx=0.5, by=0.5)
+    sg.sg_cnn_set_weights(prob, params_for(15))
+    R = torch.from_numpy(random_block(prob.n, 3, seed=81).T.copy()).float().cuda()
+    Z, Zs = torch.zeros_like(R), torch.zeros_like(R)
+    sg.sg_cnn_apply(prob, R, Z)
+    for e in (-100, -60, 40, 90):
+        sg.sg_cnn_apply(prob, R * 2.0 ** e, Zs)
+        assert torch.equal(Zs, Z * 2.0 ** e), e
+    prob.close()
