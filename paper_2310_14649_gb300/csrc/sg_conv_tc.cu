@@ -97,13 +97,22 @@ __global__ void __launch_bounds__(128) k_conv_tc(const bf16* __restrict__ X, con
   // image the source size is 0 and the destination is zero-filled)
   for (int e = tid; e < S::SB / 16; e += 128) cp_async16(sB + 16 * e, Wp + 8 * e, 16);
   const bf16* Ximg = X + size_t(img) * H * W * CI;
-  for (int e = tid; e < (kRows + 2) * kHalo * S::NPA; e += 128) {
-    const int c8 = e % S::NPA, pos = e / S::NPA;
-    const int hr = pos / kHalo, hc = pos - hr * kHalo;
-    const int gy = y0 + hr - 1, gx = x0 + hc - 1;
-    const bool in = gy >= 0 && gy < H && gx >= 0 && gx < W;
-    const bf16* src = in ? Ximg + (size_t(gy) * W + gx) * CI + c8 * 8 : Ximg;
-    cp_async16(sA + c8 * S::PLA + pos * 16, src, in ? 16 : 0);
+  // a thread's pieces of a halo row, then the rows: a few instructions a copy
+  // (with each copy's row and column divided out of its index half of the
+  // kernel's instructions were address arithmetic)
+#pragma unroll
+  for (int u = 0; u < (kHalo * S::NPA + 127) / 128; ++u) {
+    const int e = tid + 128 * u, c8 = e % S::NPA, hc = e / S::NPA, gx = x0 + hc - 1;
+    if (e >= kHalo * S::NPA) break;
+    const bool inx = gx >= 0 && gx < W;
+    const bf16* col = Ximg + (inx ? size_t(gx) * CI + c8 * 8 : 0);
+    uint8_t* dst = sA + c8 * S::PLA + hc * 16;
+#pragma unroll
+    for (int hr = 0; hr < kRows + 2; ++hr) {
+      const int gy = y0 + hr - 1;
+      const bool in = inx && gy >= 0 && gy < H;
+      cp_async16(dst + hr * kHalo * 16, in ? col + size_t(gy) * W * CI : Ximg, in ? 16 : 0);
+    }
   }
   asm volatile("cp.async.commit_group;\n" ::: "memory");
   asm volatile("cp.async.wait_group 0;\n" ::: "memory");
@@ -126,14 +135,16 @@ __global__ void __launch_bounds__(128) k_conv_tc(const bf16* __restrict__ X, con
   if (tid == 0) {
     const uint32_t a0 = smem_u32(sA), b0 = smem_u32(sB);
     constexpr uint32_t idesc = inst_desc(128, CO);
+    // back-to-back MMAs into one accumulator wait for each other, so the rows'
+    // accumulators take turns (each still sums its taps in order)
 #pragma unroll 1
-    for (int r = 0; r < kRows; ++r) {
-      uint32_t acc = 0;
-#pragma unroll 1
-      for (int t = 0; t < 9; ++t) {
-        const int p0 = (r + t / 3) * kHalo + (t % 3);
+    for (int t = 0; t < 9; ++t) {
 #pragma unroll
-        for (int kc = 0; kc < CI / 16; ++kc) {
+      for (int kc = 0; kc < CI / 16; ++kc) {
+#pragma unroll
+        for (int r = 0; r < kRows; ++r) {
+          const int p0 = (r + t / 3) * kHalo + (t % 3);
+          const uint32_t acc = t > 0 || kc > 0;
           const uint64_t ad = mat_desc(a0 + uint32_t(2 * kc * S::PLA + p0 * 16), S::PLA, 128);
           const uint64_t bd = mat_desc(b0 + uint32_t((t * S::NPB + 2 * kc) * S::PLB), S::PLB, 128);
           asm volatile(
@@ -141,13 +152,17 @@ __global__ void __launch_bounds__(128) k_conv_tc(const bf16* __restrict__ X, con
               "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem + uint32_t(32 * r)),
               "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
               : "memory");
-          acc = 1;
         }
       }
     }
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
                      smem_u32(mbar))
                  : "memory");
+  }
+  float bs[EPI == 0 ? CO : 1];
+  if (EPI == 0) {
+#pragma unroll
+    for (int c = 0; c < CO; ++c) bs[EPI == 0 ? c : 0] = bias[c];
   }
   // accumulator complete (bounded wait of wait_limit polls; on a timeout
   // the error flag is set and nothing is stored, and a second bounded wait
@@ -193,8 +208,8 @@ __global__ void __launch_bounds__(128) k_conv_tc(const bf16* __restrict__ X, con
           if (EPI == 0) {
 #pragma unroll
             for (int c = 0; c < 16; ++c)
-              o[c] = pack_bf2(relu_nan(__uint_as_float(r[2 * c]) + bias[2 * c]),
-                              relu_nan(__uint_as_float(r[2 * c + 1]) + bias[2 * c + 1]));
+              o[c] = pack_bf2(relu_nan(__uint_as_float(r[2 * c]) + bs[EPI == 0 ? 2 * c : 0]),
+                              relu_nan(__uint_as_float(r[2 * c + 1]) + bs[EPI == 0 ? 2 * c + 1 : 0]));
           } else {
             const uint4* mk = reinterpret_cast<const uint4*>(mask + pix * 32);
 #pragma unroll
@@ -249,10 +264,10 @@ __global__ void __launch_bounds__(128) k_conv_tc(const bf16* __restrict__ X, con
 // the eight channels of a 16-byte piece contiguous, planes of eight channels
 // PLANE bytes apart), which is how the images lie in memory: a row is staged
 // as 16-byte pieces, three copies shifted by one pixel for the taps dx, from
-// registers that were loaded while the MMAs of the row before ran.  K-major
+// registers that were loaded two rows ahead of the MMAs.  K-major
 // operands took a transpose of 2-byte stores (2.7 of a training
 // step's 4.2 ms on 32 images of 255 x 255, the tensor pipe 8 % active; now
-// 0.81 ms).  PLANE is 128
+// 0.72 ms).  PLANE is 128
 // pixels and 32 bytes: the four pieces of a pixel and its neighbour's land in
 // distinct banks.
 constexpr int kWgPix = 128;        // pixels per chunk (K)
@@ -294,25 +309,27 @@ __global__ void __launch_bounds__(128) k_wgrad_tc(const bf16* __restrict__ X, co
   constexpr int CX = CI / 8, CG = CO / 8;
   constexpr int EX = (kWgPix + 2) * CX, EG = kWgPix * CG;
   constexpr int LX = (EX + 127) / 128, LG = EG / 128;
-  uint4 vx[LX], vg[LG];
-  auto load_x = [&](int r) {  // zero outside the image
+  struct Row {
+    uint4 x[LX], g[LG];
+  };
+  auto load_x = [&](Row& v, int r) {  // zero outside the image
 #pragma unroll
     for (int u = 0; u < LX; ++u) {
       const int e = tid + 128 * u, x = x0 + e / CX - 1;
-      vx[u] = make_uint4(0, 0, 0, 0);
+      v.x[u] = make_uint4(0, 0, 0, 0);
       if (e < EX && r >= 0 && r < H && x >= 0 && x < W)
-        vx[u] = *reinterpret_cast<const uint4*>(Ximg + (size_t(r) * W + x) * CI + 8 * (e % CX));
+        v.x[u] = *reinterpret_cast<const uint4*>(Ximg + (size_t(r) * W + x) * CI + 8 * (e % CX));
     }
   };
-  auto load_g = [&](int y) {
+  auto load_g = [&](Row& v, int y) {
 #pragma unroll
     for (int u = 0; u < LG; ++u) {
       const int e = tid + 128 * u, x = x0 + e / CG;
-      vg[u] = make_uint4(0, 0, 0, 0);
-      if (x < W) vg[u] = *reinterpret_cast<const uint4*>(Gimg + (size_t(y) * W + x) * CO + 8 * (e % CG));
+      v.g[u] = make_uint4(0, 0, 0, 0);
+      if (x < W) v.g[u] = *reinterpret_cast<const uint4*>(Gimg + (size_t(y) * W + x) * CO + 8 * (e % CG));
     }
   };
-  auto store_x = [&](int r) {
+  auto store_x = [&](const Row& v, int r) {
     uint8_t* slot = sA + ((r + 3) % 3) * S::SLOT;
 #pragma unroll
     for (int u = 0; u < LX; ++u) {
@@ -321,15 +338,15 @@ __global__ void __launch_bounds__(128) k_wgrad_tc(const bf16* __restrict__ X, co
       for (int dx = 0; dx < 3; ++dx) {
         const int k = q - dx;
         if (e < EX && k >= 0 && k < kWgPix)
-          *reinterpret_cast<uint4*>(slot + (dx * CX + c8) * S::PLANE + k * 16) = vx[u];
+          *reinterpret_cast<uint4*>(slot + (dx * CX + c8) * S::PLANE + k * 16) = v.x[u];
       }
     }
   };
-  auto store_g = [&]() {
+  auto store_g = [&](const Row& v) {
 #pragma unroll
     for (int u = 0; u < LG; ++u) {
       const int e = tid + 128 * u;
-      *reinterpret_cast<uint4*>(sB + (e % CG) * S::PLANE + (e / CG) * 16) = vg[u];
+      *reinterpret_cast<uint4*>(sB + (e % CG) * S::PLANE + (e / CG) * 16) = v.g[u];
     }
   };
   if (warp == 0) {
@@ -342,13 +359,20 @@ __global__ void __launch_bounds__(128) k_wgrad_tc(const bf16* __restrict__ X, co
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(mbar)) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
+  // rows y and y + 1 of the strip in registers (output gradient of the row,
+  // input row after it), two rows ahead of the MMAs
+  Row even, odd;
   if (ya < yb) {
-    load_x(ya - 1);
-    store_x(ya - 1);
-    load_x(ya);
-    store_x(ya);
-    load_x(ya + 1);
-    load_g(ya);
+    load_x(even, ya - 1);
+    load_x(odd, ya);
+    store_x(even, ya - 1);
+    store_x(odd, ya);
+    load_x(even, ya + 1);
+    load_g(even, ya);
+    if (ya + 1 < yb) {
+      load_x(odd, ya + 2);
+      load_g(odd, ya + 1);
+    }
   }
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
   __syncthreads();
@@ -368,19 +392,21 @@ __global__ void __launch_bounds__(128) k_wgrad_tc(const bf16* __restrict__ X, co
   };
   bool ok = true;
   uint32_t phase = 0;
-  for (int y = ya; y < yb; ++y) {
-    store_x(y + 1);
-    store_g();
+  auto row_step = [&](int y, Row& v) {
+    store_x(v, y + 1);
+    store_g(v);
     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     if (tid == 0) {
-#pragma unroll 1
-      for (int dy = 0; dy < 3; ++dy) {
-        const int s = (y + dy - 1 + 3) % 3;
+      // the three accumulators take turns (k_conv_tc)
+      const int s0 = (y + 2) % 3;
 #pragma unroll
-        for (int kc = 0; kc < kWgPix / 16; ++kc) {
+      for (int kc = 0; kc < kWgPix / 16; ++kc) {
+#pragma unroll
+        for (int dy = 0; dy < 3; ++dy) {
+          const int s = s0 + dy < 3 ? s0 + dy : s0 + dy - 3;
           // eight pixels of eight channels are 128 bytes; next pixels LBO, next channels SBO
           const uint64_t ad = mat_desc(a0 + uint32_t(s * S::SLOT + 256 * kc), 128, S::PLANE);
           const uint64_t bd = mat_desc(b0 + uint32_t(256 * kc), 128, S::PLANE);
@@ -396,9 +422,9 @@ __global__ void __launch_bounds__(128) k_wgrad_tc(const bf16* __restrict__ X, co
                        smem_u32(mbar))
                    : "memory");
     }
-    if (y + 1 < yb) {
-      load_x(y + 2);
-      load_g(y + 1);
+    if (y + 2 < yb) {
+      load_x(v, y + 3);
+      load_g(v, y + 2);
     }
     // the MMAs read the slots and B: wait before the next staging
     const uint32_t done = poll(wait_limit, phase);
@@ -407,8 +433,11 @@ __global__ void __launch_bounds__(128) k_wgrad_tc(const bf16* __restrict__ X, co
     if (!ok) {
       if (tid == 0) atomicExch(err, 1);
       poll(kDrainLimit, phase ^ 1u);   // the MMAs of this chunk, before tensor memory is freed
-      break;
     }
+  };
+  for (int y = ya; ok && y < yb; y += 2) {
+    row_step(y, even);
+    if (ok && y + 1 < yb) row_step(y + 1, odd);
   }
   asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
   if (ok && ya < yb) {
