@@ -501,6 +501,10 @@ bool solver_edge(const sg_problem* pr) {
   return jit_eligible(pr) && (pr->jit_cfg_user[0] ? pr->jit_cfg[0].flux != 0 : pr->flux_allowed && pr->P <= 48);
 }
 
+bool coarse_edge_form(const sg_problem* pr) {
+  return solver_edge(pr) && (pr->jit_cfg_user[0] || pr->N * pr->p <= 800);
+}
+
 // generated family of an FP32 apply: a solve on the slot form while the fine
 // family's own (untuned) form is the edge form has a family for it
 static int fp32_family(const sg_problem* pr, bool coarse, bool solver) {

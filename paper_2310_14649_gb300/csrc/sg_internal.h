@@ -342,6 +342,14 @@ sg_status jit_edge_launch(sg_problem* pr, int which, const EdgeVals& A, const T*
 // several times faster (345 us against 2.1 ms an apply): sg_apply_flux(prob,
 // 1) selects it.
 bool solver_edge(const sg_problem* pr);
+// whether coarse solves use the coarse edge form and the folded V-cycle: in
+// solves that use the edge form, and (untuned) while N p <= 800.  A coarse
+// solve to the default tolerance (1e-5) in FP32 returns the rounding error of
+// its operator amplified by the condition of the coarse matrix: the two
+// forms' corrections differ by 1.2e-5 at 256^2, p = 3, 1.5e-5 at 320^2, p = 3
+// and 1.6e-5 at 256^2, p = 4 (1.0e-5 at 200^2, p = 3, 5e-6 at 256^2, p = 2),
+// and beyond the line by more than FP32 results may move.
+bool coarse_edge_form(const sg_problem* pr);
 // FP32 values the applies of a solve need, built before any capture
 sg_status apply_prepare32(sg_problem* pr, bool coarse, cudaStream_t st);
 // assembled FP64 blocks (sg_apply.cu): build per the problem's policy (no-op

@@ -878,7 +878,7 @@ static JitConfig edge_default(const sg_problem* pr, int N, bool fp64) {
 
 JitConfig jit_default_config(const sg_problem* pr, int which) {
   if ((which == 0 && pr->flux_allowed) || which == 4) return edge_default(pr, pr->N, false);
-  if (which == 1 && solver_edge(pr)) return edge_default(pr, pr->N / 2, false);
+  if (which == 1 && coarse_edge_form(pr)) return edge_default(pr, pr->N / 2, false);
   if (which == 5) return edge_default(pr, pr->N, true);
   const bool fp64 = which == 2 || which == 3;
   JitConfig c;

@@ -314,8 +314,8 @@ sg_status sg_precond_setup(sg_problem* pr, const sg_precond_opts* o, void* strea
   pc.ras_kernel = o->ras_kernel;
   pc.inner_passes = o->inner_orth_passes > 0 ? o->inner_orth_passes : 1;
   SG_TRY(kernel_attrs_init());
-  // the FP32 V-cycle keeps its phase kernels where a solve keeps the slot form
-  pc.amg_fold = o->amg_kernel == 0 && solver_edge(pr) && pr->P <= kFoldModes;
+  // the FP32 V-cycle keeps its phase kernels where coarse solves keep the slot form
+  pc.amg_fold = o->amg_kernel == 0 && coarse_edge_form(pr) && pr->P <= kFoldModes;
   sg_status s = precond_setup_host(pr, pc);
   pc.amg.fused = o->amg_kernel == 0;
   pc.wait_limit = pr->wait_limit;

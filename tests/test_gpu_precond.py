@@ -469,3 +469,23 @@ def test_smoother_on_callers_blocks(gpu, which):
     pool[:, :n] = X                     # rows of input and output side by side
     sg.sg_precond_apply(prob, op, pool[:, :n], pool[:, n:2 * n])
     assert torch.equal(pool[:, n:2 * n], Z) and torch.equal(pool[:, :n], X)
+
+
+@pytest.mark.parametrize("N,p,slot", [(200, 4, False), (202, 4, True)])
+def test_coarse_solves_keep_the_slot_form_beyond_the_line(gpu, N, p, slot):
+    """Untuned coarse corrections with N p > 800 return the bits of the slot
+    operator and the unfolded V-cycle; up to the line they use the edge form
+    (equal to the tolerance of the coarse solve, 1e-5, times ten)."""
+    import torch
+    import paper_2310_14649_gb300 as sg
+    Z = []
+    for form in (2, 0):
+        prob = sg.sg_setup(N, 1, p, 2 * p, sigma2=0.3, bx=0.5, by=0.5)
+        sg.sg_apply_flux(prob, form)
+        sg.sg_precond_setup(prob, 8, 8, 1)
+        R = torch.from_numpy(random_block(prob.n, prob.P, seed=43).T.copy()).float().cuda()
+        Z.append(torch.zeros_like(R))
+        sg.sg_precond_apply(prob, sg.PC_COARSE, R, Z[-1])
+        prob.close()
+    assert torch.equal(Z[0], Z[1]) == slot
+    assert (Z[0] - Z[1]).norm() <= 1e-4 * Z[1].norm()
