@@ -684,13 +684,13 @@ def main():
     sg.sg_profile(prob, False)
 
     # roofline of the fine FP32 operator apply: algorithmic bytes per launch
-    # (five-slot form: values, pattern and blocks read once; edge-flux form:
-    # one conductance per edge and term, two indices per edge slot of a row)
+    # (five-slot form: values, pattern and blocks read once; edge form: one
+    # conductance per edge and term)
     K, nnz = prob.K, prob.nnzA
     flux_on = sg.sg_apply_flux(prob, -1)
     N_ = c["N"]
     bytes_slot = K * nnz * 4 + nnz * 4 + (n + 1) * 4 + 2 * n * P * 4
-    bytes_flux = K * 2 * N_ * (N_ - 1) * 4 + 4 * 2 * 4 * n + 2 * n * P * 4
+    bytes_flux = K * 2 * N_ * (N_ - 1) * 4 + 2 * n * P * 4
     bytes_f32 = bytes_flux if flux_on else bytes_slot
     cnt, kms = kinds["apply_fine_f32"]
     avg_ms = kms / max(cnt, 1)
