@@ -205,7 +205,7 @@ struct ProfScope {
 constexpr int kJitFamilies = 4;
 constexpr int kJitAllFamilies = 7;
 constexpr int kJitMaxP = 128;
-constexpr int kJitGeneratorVersion = 11;  // bump when the generated code changes
+constexpr int kJitGeneratorVersion = 12;  // bump when the generated code changes
 constexpr int64_t kJitMaxT = 40000;
 struct JitConfig {
   int rows = 1;        // rows per thread (2: paired FP32 FMA)

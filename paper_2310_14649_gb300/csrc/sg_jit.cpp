@@ -766,9 +766,20 @@ std::string jit_edge_source(const sg_problem* pr, const JitConfig& c, bool fp64)
     os << "      } else {\n"
           "        if (v && own) {\n"
           "          const long long r = (long long)((up ? j : j + 1) - 1) * m + c - 1;\n";
-    for (size_t u = 0; u < outs.size(); ++u)
-      os << "          { const T o = " << fma << "(-sg, f" << outs[u] << ", y[" << 32 * u << "]); Y[" << outs[u]
-         << "ll * ldy + r] = F ? F[" << outs[u] << "ll * ldf + r] - o : o; }\n";
+    // eight outputs at a time, their loads of F together (F may be Y: a load
+    // behind a store waits for nothing but is not moved before it; 62 us an
+    // apply with F at 256^2, P = 35 one by one, 34 without F)
+    for (size_t u0 = 0; u0 < outs.size(); u0 += 8) {
+      const size_t u1 = std::min(outs.size(), u0 + 8);
+      os << "          {";
+      for (size_t u = u0; u < u1; ++u)
+        os << " const T g" << u << " = F ? F[" << outs[u] << "ll * ldf + r] : T(0);";
+      os << "\n";
+      for (size_t u = u0; u < u1; ++u)
+        os << "            { const T o = " << fma << "(-sg, f" << outs[u] << ", y[" << 32 * u << "]); Y[" << outs[u]
+           << "ll * ldy + r] = F ? g" << u << " - o : o; }\n";
+      os << "          }\n";
+    }
     os << "        }\n";
     for (size_t u = 0; u < outs.size(); ++u) os << "        y[" << 32 * u << "] = sg * f" << outs[u] << ";\n";
     os << "      }\n"
