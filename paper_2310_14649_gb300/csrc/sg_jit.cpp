@@ -768,7 +768,7 @@ std::string jit_edge_source(const sg_problem* pr, const JitConfig& c, bool fp64)
           "          const long long r = (long long)((up ? j : j + 1) - 1) * m + c - 1;\n";
     // eight outputs at a time, their loads of F together (F may be Y: a load
     // behind a store waits for nothing but is not moved before it; 62 us an
-    // apply with F at 256^2, P = 35 one by one, 34 without F)
+    // apply with F at 256^2, P = 35 one by one, now 44; 37 without F)
     for (size_t u0 = 0; u0 < outs.size(); u0 += 8) {
       const size_t u1 = std::min(outs.size(), u0 + 8);
       os << "          {";
