@@ -550,8 +550,9 @@ static EdgeOrder edge_order(const sg_problem* pr) {
 }
 
 // terms per staged chunk (a multiple of 4): at most `prefetch`, and a turn has at least
-// stages - 1 chunks (the copies run that far ahead, into the next turn at most)
-static int edge_stages(const JitConfig& c, int Kr) { return std::min(c.stages, Kr / 4 + 1); }
+// stages - 1 chunks (the copies run that far ahead, into the next turn at most); Kr > 0, so
+// at least two stages
+static int edge_stages(const JitConfig& c, int Kr) { return std::max(2, std::min(c.stages, Kr / 4 + 1)); }
 static int edge_chunk(const JitConfig& c, int Kr) {
   return 4 * std::max(1, std::min(c.prefetch / 4, Kr / 4 / (edge_stages(c, Kr) - 1)));
 }
@@ -888,9 +889,13 @@ static JitConfig edge_default(const sg_problem* pr, int N, bool fp64) {
 }
 
 JitConfig jit_default_config(const sg_problem* pr, int which) {
-  if ((which == 0 && pr->flux_allowed) || which == 4) return edge_default(pr, pr->N, false);
-  if (which == 1 && coarse_edge_form(pr)) return edge_default(pr, pr->N / 2, false);
-  if (which == 5) return edge_default(pr, pr->N, true);
+  // a handle beyond the specialised kernel's limits has no edge form (its
+  // applies run on the shared-memory kernel): it reports the slot shape
+  if (jit_eligible(pr)) {
+    if ((which == 0 && pr->flux_allowed) || which == 4) return edge_default(pr, pr->N, false);
+    if (which == 1 && coarse_edge_form(pr)) return edge_default(pr, pr->N / 2, false);
+    if (which == 5) return edge_default(pr, pr->N, true);
+  }
   const bool fp64 = which == 2 || which == 3;
   JitConfig c;
   c.rows = 1;

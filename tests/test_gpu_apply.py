@@ -464,3 +464,27 @@ def test_solves_above_48_modes_keep_the_slot_form(gpu):
     assert torch.equal(X[0], X[1])
     assert not torch.equal(X[0], X[2]) and (X[0] - X[2]).norm() <= 1e-7 * X[0].norm()
     prob.close()
+
+
+@pytest.mark.parametrize("L,p,q", [(4, 5, 10), (9, 3, 2)])
+def test_settings_beyond_the_specialised_kernel(gpu, L, p, q):
+    """T = 53,157 and P = 220: no generated kernel, hence no edge form.  The
+    entry points that describe or choose tile shapes still answer, with the
+    slot form's shape, and the apply agrees with the oracle after each."""
+    import torch
+    import paper_2310_14649_gb300 as sg
+    prob, ref = setup_pair(6, L, p, q)
+    assert prob.P > 128 or prob.T > 40000
+    X = random_block(ref.n, ref.P, seed=93)
+    for which in range(4):
+        assert sg.sg_apply_info(prob, which=which)["stages"] == 0
+    for mode in (-1, 0, 2):
+        assert sg.sg_apply_flux(prob, mode) == 0
+        assert sg.sg_apply_info(prob)["stages"] == 0
+        check_apply(prob, ref, X, torch.float32)
+    with pytest.raises(sg.SgError):
+        sg.sg_apply_flux(prob, 1)
+    sg.sg_apply_config(prob, 1, 1, 1, 1, 16, 1)
+    assert sg.sg_apply_info(prob)["prefetch"] == 16
+    check_apply(prob, ref, X, torch.float32)
+    prob.close()
