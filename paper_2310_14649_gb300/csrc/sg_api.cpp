@@ -121,7 +121,10 @@ sg_status sg_apply_flux(sg_problem* pr, int mode, int* on) {
   if (mode >= 0) {
     const JitConfig was = jit_config(pr, 0);
     pr->flux_allowed = mode != 0;
-    if ((mode == 0 || mode == 1) && was.flux != mode) SG_TRY(jit_configure(pr, 0, jit_default_config(pr, 0)));
+    if (mode < 2 && was.flux != mode)
+      SG_TRY(jit_configure(pr, 0, jit_default_config(pr, 0)));
+    else if (mode < 2 && !pr->jit_cfg_user[0])
+      SG_TRY(jit_keep(pr, 0));
   }
   if (on) *on = jit_eligible(pr) && jit_config(pr, 0).flux;
   return SG_OK;

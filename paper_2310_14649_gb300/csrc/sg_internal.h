@@ -323,6 +323,8 @@ sg_status jit_autotune(sg_problem* pr, int which, int force, double* best_ms);
 sg_status jit_apply_build(sg_problem* pr, int which);
 void jit_free(sg_problem* pr, int which);
 sg_status jit_configure(sg_problem* pr, int which, const JitConfig& c);
+// the form a family runs on untuned becomes the program's own choice (solver_edge)
+sg_status jit_keep(sg_problem* pr, int which);
 bool jit_eligible(const sg_problem* pr);
 sg_status jit_apply_launch(sg_problem* pr, int which, const Ell& A, const double* X, int64_t ldx, const double* F,
                            int64_t ldf, double* Y, int64_t ldy, cudaStream_t st);

@@ -976,6 +976,16 @@ sg_status jit_configure(sg_problem* pr, int which, const JitConfig& c) {
   return jit_apply_build(pr, which);
 }
 
+sg_status jit_keep(sg_problem* pr, int which) {
+  const bool edge = solver_edge(pr);
+  pr->jit_cfg[which] = jit_config(pr, which);
+  pr->jit_cfg_set[which] = true;
+  pr->jit_cfg_user[which] = true;
+  // recorded coarse-solve graphs run the form solves used until now
+  if (solver_edge(pr) != edge) drop_recorded(pr);
+  return jit_eligible(pr) ? jit_apply_build(pr, which) : SG_OK;
+}
+
 void jit_free(sg_problem* pr, int which) {
   if (!pr->jit[which]) return;
   if (pr->jit[which]->lib) cudaLibraryUnload(pr->jit[which]->lib);

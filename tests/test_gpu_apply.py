@@ -488,3 +488,31 @@ def test_settings_beyond_the_specialised_kernel(gpu, L, p, q):
     assert sg.sg_apply_info(prob)["prefetch"] == 16
     check_apply(prob, ref, X, torch.float32)
     prob.close()
+
+
+@pytest.mark.parametrize("solved_before", [False, True])
+def test_edge_form_chosen_on_a_fresh_handle(gpu, solved_before):
+    """sg_apply_flux(1) as the first choice made on a handle moves mixed
+    solves at P > 48 to the edge form, as it does after mode 0, and also once
+    a solve has run (and recorded its coarse solves) on the slot form."""
+    import torch
+    import paper_2310_14649_gb300 as sg
+
+    def solve(modes, before=False):
+        prob = sg.sg_setup(24, 5, 3, 6)
+        sg.sg_apply_config(prob, 1, 1, 1, 2, 16, 1, which=1)     # one coarse operator for all
+        sg.sg_precond_setup(prob, 2, 2, 1, inner_rtol=0.5)
+        x = torch.zeros((prob.P, prob.n), dtype=torch.float64, device="cuda")
+        if before:
+            sg.sg_solve(prob, x, rtol=1e-9, mode=1)
+        for mode in modes:
+            assert sg.sg_apply_flux(prob, mode) == mode
+        x.zero_()
+        sg.sg_solve(prob, x, rtol=1e-9, mode=1)
+        prob.close()
+        return x
+
+    slot, edge = solve([]), solve([0, 1])
+    fresh = solve([1], solved_before)
+    assert not torch.equal(slot, edge)
+    assert torch.equal(fresh, edge)
