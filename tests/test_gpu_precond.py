@@ -489,3 +489,31 @@ def test_coarse_solves_keep_the_slot_form_beyond_the_line(gpu, N, p, slot):
         prob.close()
     assert torch.equal(Z[0], Z[1]) == slot
     assert (Z[0] - Z[1]).norm() <= 1e-4 * Z[1].norm()
+
+
+@pytest.mark.parametrize("N,L,p,q,launches", [
+    (34, 3, 1, 2, 1),      # one level: the dense product alone
+    (66, 4, 4, 8, 3),      # 70 modes: the wide kernel, two mode tiles
+    (40, 5, 4, 4, 3),      # 126 modes: three mode tiles, the last cut short
+    (400, 1, 1, 2, 5),     # two sparse levels
+])
+def test_amg_fold_is_the_cycle_that_runs(gpu, N, L, p, q, launches):
+    """With the edge form chosen the FP32 V-cycle is the folded one at every
+    P: a launch down and one up per sparse level and the dense product.
+    Bound as in test_amg_fold."""
+    import torch
+    import paper_2310_14649_gb300 as sg
+    prob = sg.sg_setup(N, L, p, q, sigma2=0.3, bx=0.5, by=0.5)
+    sg.sg_apply_flux(prob, 1)
+    sg.sg_precond_setup(prob, 3, 3, 1, omega=0.3)
+    nc, P = (N // 2 - 1) ** 2, prob.P
+    B = random_block(nc, P, seed=37).astype(np.float32).astype(np.float64)
+    Y64, _ = run(prob, sg.PC_AMG, B, nc, torch.float64)
+    S64, _ = run(prob, sg.PC_AMG, np.abs(B), nc, torch.float64)
+    run(prob, sg.PC_AMG, B, nc, torch.float32)
+    before = sg.sg_launch_count()
+    Y32, _ = run(prob, sg.PC_AMG, B, nc, torch.float32)
+    assert sg.sg_launch_count() - before == launches
+    tol = 2 * (min(nc, 2048) / 8 + 64) * 2.0 ** -24
+    assert np.max(np.abs(Y32 - Y64)) <= tol * np.max(np.abs(S64))
+    prob.close()
