@@ -57,6 +57,7 @@ sg_status sg_setup(const sg_mesh_desc* mesh, const sg_kl_desc* kl, int p_out, in
   sg_status st = build_host(pr, kl);
   if (st == SG_OK) st = assemble_fine(pr);
   if (st == SG_OK) st = build_triple_tables(pr, pr->tri, pr->fine.S);
+  if (st == SG_OK) st = fp32_values(pr);
   if (st != SG_OK) {
     sg_destroy(pr);
     return st;
@@ -94,6 +95,7 @@ sg_status sg_set_apply_kernel(sg_problem* pr, int mode) {
   }
   drop_recorded(pr);
   pr->apply_mode = mode;
+  SG_TRY(fp32_values(pr));
   if (mode != 1 && jit_eligible(pr)) return jit_apply_build(pr, 0);
   return SG_OK;
 }

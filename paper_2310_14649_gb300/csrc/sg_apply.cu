@@ -533,6 +533,14 @@ sg_status apply_any(sg_problem* pr, bool coarse, const T* X, int64_t ldx, const 
   return apply_ell<T>(A, coarse ? coarse_tri(pr) : pr->tri, pr->P, pr->K, X, ldx, F, ldf, Y, ldy, st);
 }
 
+sg_status fp32_values(sg_problem* pr) {
+  const bool generated = pr->apply_mode != 1 && jit_eligible(pr);
+  if (!generated || !jit_config(pr, 0).flux || (pr->solver && !solver_edge(pr)))
+    SG_TRY(ell_f32(pr->fine, pr->K, nullptr));
+  if (pr->solver && (!generated || !jit_config(pr, 1).flux)) SG_TRY(ell_f32(coarse_ell(pr), pr->K, nullptr));
+  return SG_OK;
+}
+
 sg_status apply_prepare32(sg_problem* pr, bool coarse, cudaStream_t st) {
   if (pr->apply_mode != 1 && jit_eligible(pr)) {
     const int which = fp32_family(pr, coarse, true);

@@ -82,7 +82,7 @@ struct Ell {
   int64_t n = 0, ldr = 0;
   DevBuf col;      // int32 S x ldr
   DevBuf v64;      // double K x S x ldr
-  mutable DevBuf v32;  // float  K x S x ldr, rounded from v64 on first use (ell_f32)
+  mutable DevBuf v32;  // float  K x S x ldr, rounded from v64 where the slot form runs (ell_f32)
 };
 
 // The same family in the edge form: one conductance per edge of a mesh of
@@ -301,7 +301,8 @@ sg_status edge_values(const sg_problem* pr, const Tc* coef, int k0, int kn, Edge
 template <typename Tc>
 sg_status edge_values_all(const sg_problem* pr, const Tc* coef, EdgeVals& out, cudaStream_t st);
 // the FP32 five- or seven-slot values of an ELL family (rounded from the
-// FP64 ones on first use; synchronous then, never while `st` is capturing)
+// FP64 ones when they are not there yet, see fp32_values; synchronous then,
+// never while `st` is capturing)
 sg_status ell_f32(const Ell& A, int K, cudaStream_t st);
 sg_status build_triple_tables(sg_problem* pr, TripleTables& t, int S);
 // apply (sg_apply.cu)
@@ -352,6 +353,10 @@ bool solver_edge(const sg_problem* pr);
 // and 1.6e-5 at 256^2, p = 4 (1.0e-5 at 200^2, p = 3, 5e-6 at 256^2, p = 2),
 // and beyond the line by more than FP32 results may move.
 bool coarse_edge_form(const sg_problem* pr);
+// the FP32 slot values of the operators that run on the slot form, with the
+// handle, its preconditioner or the choice of the form: a first apply may be
+// captured and neither allocates nor waits.  Synchronous.
+sg_status fp32_values(sg_problem* pr);
 // FP32 values the applies of a solve need, built before any capture
 sg_status apply_prepare32(sg_problem* pr, bool coarse, cudaStream_t st);
 // assembled FP64 blocks (sg_apply.cu): build per the problem's policy (no-op

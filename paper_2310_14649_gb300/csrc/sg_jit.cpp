@@ -972,6 +972,7 @@ sg_status jit_configure(sg_problem* pr, int which, const JitConfig& c) {
   pr->jit_cfg[which] = c;
   pr->jit_cfg_set[which] = true;
   pr->jit_cfg_user[which] = true;
+  if (which < 2) SG_TRY(fp32_values(pr));
   if (!jit_eligible(pr)) return SG_OK;
   return jit_apply_build(pr, which);
 }

@@ -317,6 +317,7 @@ sg_status sg_precond_setup(sg_problem* pr, const sg_precond_opts* o, void* strea
   // the FP32 V-cycle keeps its phase kernels where coarse solves keep the slot form
   pc.amg_fold = o->amg_kernel == 0 && coarse_edge_form(pr) && pr->P <= kFoldModes;
   sg_status s = precond_setup_host(pr, pc);
+  if (s == SG_OK) s = fp32_values(pr);
   pc.amg.fused = o->amg_kernel == 0;
   pc.wait_limit = pr->wait_limit;
   if (s == SG_OK && pc.ras_kernel == 2) s = ras_inverse_build(pr, pc, st);

@@ -516,3 +516,29 @@ def test_edge_form_chosen_on_a_fresh_handle(gpu, solved_before):
     fresh = solve([1], solved_before)
     assert not torch.equal(slot, edge)
     assert torch.equal(fresh, edge)
+
+
+@pytest.mark.parametrize("choice", ["flux", "config", "kernel", "large"])
+def test_first_slot_form_apply_can_be_captured(gpu, choice):
+    """Handles on the slot form hold its FP32 values when the form is chosen
+    (P > 128: from sg_setup on): the first apply is captured into a graph and
+    gives the bits of a later eager one."""
+    import torch
+    import paper_2310_14649_gb300 as sg
+    prob, ref = setup_pair(*((6, 9, 3, 2) if choice == "large" else (20, 3, 2, 4)))
+    if choice == "flux":
+        sg.sg_apply_flux(prob, 0)
+    elif choice == "config":
+        sg.sg_apply_config(prob, 1, 1, 1, 1, 16, 1)
+    elif choice == "kernel":
+        sg.sg_set_apply_kernel(prob, 1)
+    X = to_dev(random_block(ref.n, ref.P, seed=94), torch.float32)
+    Y, Z = torch.zeros_like(X), torch.zeros_like(X)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        sg.sg_apply(prob, X, Y)
+    graph.replay()
+    sg.sg_apply(prob, X, Z)
+    torch.cuda.synchronize()
+    assert torch.equal(Y, Z) and bool(Z.any())
+    prob.close()
