@@ -248,8 +248,14 @@ sg_status sg_apply_config(sg_problem* prob, int which, int rows, int groups, int
  * autotuner (sg_apply_autotune, fine FP32 family) may choose the edge form;
  * -1: no change.  on (may be NULL) receives 1 when fine FP32 applies use the
  * edge form.  sg_apply_config selects the slot form of its family.  FP64
- * applies are unaffected.  A change drops recorded coarse-solve graphs;
- * recorded batches of this problem then refuse to run.
+ * applies are unaffected.  The coarse operator (and with it the form of the
+ * FP32 V-cycle) takes its untuned form in sg_precond_setup: the edge form
+ * where solves run on it then and, unless the fine family was configured or
+ * tuned, N p <= 800 (a coarse solve to 1e-5 shows the rounding of its operator
+ * beyond); a choice made later for the fine operator leaves it as it is.
+ * sg_apply_config and sg_apply_autotune set it directly (which = 1).  A change
+ * drops recorded coarse-solve graphs; recorded batches of this problem then
+ * refuse to run.
  * Errors: SG_ERR_ARG (mode out of range; mode 1 without the specialised
  * kernel), SG_ERR_NOMEM, SG_ERR_CUDA. */
 sg_status sg_apply_flux(sg_problem* prob, int mode, int* on);

@@ -345,8 +345,9 @@ sg_status jit_edge_launch(sg_problem* pr, int which, const EdgeVals& A, const T*
 // several times faster (345 us against 2.1 ms an apply): sg_apply_flux(prob,
 // 1) selects it.
 bool solver_edge(const sg_problem* pr);
-// whether coarse solves use the coarse edge form and the folded V-cycle: in
-// solves that use the edge form, and (untuned) while N p <= 800.  A coarse
+// whether coarse solves use the coarse edge form and the folded V-cycle
+// (sg_precond_setup decides it once, Precond::coarse_edge): in solves that use
+// the edge form, and (untuned) while N p <= 800.  A coarse
 // solve to the default tolerance (1e-5) in FP32 returns the rounding error of
 // its operator amplified by the condition of the coarse matrix: the two
 // forms' corrections differ by 1.2e-5 at 256^2, p = 3, 1.5e-5 at 320^2, p = 3

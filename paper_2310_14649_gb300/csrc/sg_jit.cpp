@@ -893,7 +893,7 @@ JitConfig jit_default_config(const sg_problem* pr, int which) {
   // applies run on the shared-memory kernel): it reports the slot shape
   if (jit_eligible(pr)) {
     if ((which == 0 && pr->flux_allowed) || which == 4) return edge_default(pr, pr->N, false);
-    if (which == 1 && coarse_edge_form(pr)) return edge_default(pr, pr->N / 2, false);
+    if (which == 1 && coarse_edge_default(pr)) return edge_default(pr, pr->N / 2, false);
     if (which == 5) return edge_default(pr, pr->N, true);
   }
   const bool fp64 = which == 2 || which == 3;

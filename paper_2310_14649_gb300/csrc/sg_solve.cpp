@@ -15,6 +15,9 @@ namespace sg {
 const Ell& coarse_ell(const sg_problem* pr) { return pr->solver->pc.co.ell; }
 const TripleTables& coarse_tri(const sg_problem* pr) { return pr->solver->pc.co.tri; }
 const EdgeVals& coarse_edge(const sg_problem* pr) { return pr->solver->pc.co.edge; }
+bool coarse_edge_default(const sg_problem* pr) {
+  return pr->solver ? pr->solver->pc.coarse_edge : coarse_edge_form(pr);
+}
 AsmBlocks& coarse_asm(sg_problem* pr) { return pr->solver->pc.co.asm_c; }
 
 // Recorded graphs (the coarse-solve graphs of the solver contexts) hold the
@@ -314,8 +317,16 @@ sg_status sg_precond_setup(sg_problem* pr, const sg_precond_opts* o, void* strea
   pc.ras_kernel = o->ras_kernel;
   pc.inner_passes = o->inner_orth_passes > 0 ? o->inner_orth_passes : 1;
   SG_TRY(kernel_attrs_init());
+  // one form for the life of the preconditioner, whatever is chosen for the
+  // fine operator later and whether or not a coarse solve has run by then
+  pc.coarse_edge = coarse_edge_form(pr);
+  if (pr->jit_cfg_set[1] && !pr->jit_cfg_user[1] && (pr->jit_cfg[1].flux != 0) != pc.coarse_edge) {
+    SG_CUDA(cudaDeviceSynchronize());
+    jit_free(pr, 1);
+    pr->jit_cfg_set[1] = false;
+  }
   // the FP32 V-cycle keeps its phase kernels where coarse solves keep the slot form
-  pc.amg_fold = o->amg_kernel == 0 && coarse_edge_form(pr) && pr->P <= kFoldModes;
+  pc.amg_fold = o->amg_kernel == 0 && pc.coarse_edge && pr->P <= kFoldModes;
   sg_status s = precond_setup_host(pr, pc);
   if (s == SG_OK) s = fp32_values(pr);
   pc.amg.fused = o->amg_kernel == 0;

@@ -137,6 +137,7 @@ struct Precond {
   Harvest harvest;
   int inner_its_last = 0, inner_its_total = 0, inner_calls = 0;
   bool device_loops = true;                // coarse GMRES as one CUDA graph launch
+  bool coarse_edge = false;                // untuned form of the coarse FP32 operator (coarse_edge_form at setup)
   bool amg_fold = false;                   // build the folded FP32 V-cycle
   int last_coarse_dtype = -1;              // 0 FP64, 1 FP32: context of the last graph solve
 };
@@ -161,6 +162,8 @@ sg_status amg_setup_fine(const sg_problem* pr, AmgHier& h);
 const Ell& coarse_ell(const sg_problem* pr);
 const TripleTables& coarse_tri(const sg_problem* pr);
 const EdgeVals& coarse_edge(const sg_problem* pr);
+// the coarse operator's untuned form: the preconditioner's, or what it will be
+bool coarse_edge_default(const sg_problem* pr);
 AsmBlocks& coarse_asm(sg_problem* pr);
 // drops the solver contexts and their recorded graphs after a change of
 // apply kernel (recorded batches of the problem then refuse to run)

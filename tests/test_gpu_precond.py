@@ -517,3 +517,36 @@ def test_amg_fold_is_the_cycle_that_runs(gpu, N, L, p, q, launches):
     tol = 2 * (min(nc, 2048) / 8 + 64) * 2.0 ** -24
     assert np.max(np.abs(Y32 - Y64)) <= tol * np.max(np.abs(S64))
     prob.close()
+
+
+def test_coarse_form_is_the_preconditioners(gpu):
+    """The coarse operator's untuned form is the one chosen by
+    sg_precond_setup: a later choice for the fine operator changes no bit of a
+    coarse correction, whether one has run before or not, and the next
+    sg_precond_setup follows it."""
+    import torch
+    import paper_2310_14649_gb300 as sg
+
+    def correction(prob):
+        R = torch.from_numpy(random_block(prob.n, prob.P, seed=44).T.copy()).float().cuda()
+        Z = torch.zeros_like(R)
+        sg.sg_precond_apply(prob, sg.PC_COARSE, R, Z)
+        return Z
+
+    def handle():
+        return sg.sg_setup(64, 3, 2, 4, sigma2=0.3, bx=0.5, by=0.5)
+
+    late, early, before = handle(), handle(), handle()
+    sg.sg_precond_setup(late, 3, 3, 1)
+    edge = correction(late)
+    for prob in (late, early):
+        if prob is early:
+            sg.sg_precond_setup(prob, 3, 3, 1)
+        sg.sg_apply_flux(prob, 0)
+        assert torch.equal(correction(prob), edge), prob is late
+    sg.sg_apply_flux(before, 0)
+    for prob in (late, early, before):
+        sg.sg_precond_setup(prob, 3, 3, 1)
+    slot = correction(before)
+    assert not torch.equal(slot, edge)
+    assert torch.equal(correction(late), slot) and torch.equal(correction(early), slot)
