@@ -537,8 +537,10 @@ sg_status fp32_values(sg_problem* pr) {
   const bool generated = pr->apply_mode != 1 && jit_eligible(pr);
   if (!generated || !jit_config(pr, 0).flux || (pr->solver && !solver_edge(pr)))
     SG_TRY(ell_f32(pr->fine, pr->K, nullptr));
-  if (pr->solver && (!generated || !jit_config(pr, 1).flux)) SG_TRY(ell_f32(coarse_ell(pr), pr->K, nullptr));
-  return SG_OK;
+  if (!pr->solver) return SG_OK;
+  const bool edge = jit_eligible(pr) && jit_config(pr, 1).flux;
+  if (edge) SG_TRY(coarse_edge_prepare(pr));
+  return edge && generated ? SG_OK : ell_f32(coarse_ell(pr), pr->K, nullptr);
 }
 
 sg_status apply_prepare32(sg_problem* pr, bool coarse, cudaStream_t st) {

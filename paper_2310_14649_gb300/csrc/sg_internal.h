@@ -354,7 +354,8 @@ bool solver_edge(const sg_problem* pr);
 // and 1.6e-5 at 256^2, p = 4 (1.0e-5 at 200^2, p = 3, 5e-6 at 256^2, p = 2),
 // and beyond the line by more than FP32 results may move.
 bool coarse_edge_form(const sg_problem* pr);
-// the FP32 slot values of the operators that run on the slot form, with the
+// the FP32 slot values of the operators that run on the slot form (and the
+// coarse conductances where that operator runs on the edge form), with the
 // handle, its preconditioner or the choice of the form: a first apply may be
 // captured and neither allocates nor waits.  Synchronous.
 sg_status fp32_values(sg_problem* pr);

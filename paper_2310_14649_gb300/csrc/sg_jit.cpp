@@ -1018,6 +1018,10 @@ template <typename T>
 static sg_status launch_edge(cudaKernel_t kern, const JitConfig& c, size_t smem, const EdgeVals& A, const T* X,
                              int64_t ldx, const T* F, int64_t ldf, T* Y, int64_t ldy, cudaStream_t st) {
   const T* V = sizeof(T) == 8 ? reinterpret_cast<const T*>(A.v64.ptr) : reinterpret_cast<const T*>(A.v32.ptr);
+  if (!V) {
+    set_error("the edge form's conductances are not on the device");
+    return SG_ERR_ARG;
+  }
   long long lx = ldx, lf = ldf, ly = ldy;
   int N = A.N;
   void* args[] = {(void*)&V, &N, (void*)&X, &lx, (void*)&F, &lf, (void*)&Y, &ly};
@@ -1180,7 +1184,12 @@ sg_status jit_autotune(sg_problem* pr, int which, int force, double* best_ms) {
     cudaKernel_t kern = nullptr;
     if (jit_compile(family_source(pr, c, fp64), &lib, &kern, nullptr, nullptr, pr->device, fp64) != SG_OK) continue;
     const size_t sm = jit_smem_bytes(pr, c, fp64);
-    if (!fp64 && !c.flux && (status = ell_f32(A, pr->K, nullptr)) != SG_OK) break;
+    if (coarse && c.flux) status = coarse_edge_prepare(pr);
+    else if (!fp64 && !c.flux) status = ell_f32(A, pr->K, nullptr);
+    if (status != SG_OK) {
+      cudaLibraryUnload(lib);
+      break;
+    }
     auto run = [&]() {
       if (c.flux)
         return launch_edge<float>(kern, c, sm, coarse ? coarse_edge(pr) : pr->edge, dp<float>(X), A.ldr, nullptr, 0, dp<float>(Y),

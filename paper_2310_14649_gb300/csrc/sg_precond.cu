@@ -1482,7 +1482,6 @@ sg_status precond_setup_coarse_plan(sg_problem* pr, Precond& pc, const CoarsePla
   SG_CUDA(cudaGetLastError());
   SG_CUDA(cudaDeviceSynchronize());
   SG_TRY(build_triple_tables(pr, C.tri, S));
-  if (jit_eligible(pr)) SG_TRY(coarse_edge_build(pr, C.edge));
   return SG_OK;
 }
 

@@ -15,6 +15,14 @@ namespace sg {
 const Ell& coarse_ell(const sg_problem* pr) { return pr->solver->pc.co.ell; }
 const TripleTables& coarse_tri(const sg_problem* pr) { return pr->solver->pc.co.tri; }
 const EdgeVals& coarse_edge(const sg_problem* pr) { return pr->solver->pc.co.edge; }
+sg_status coarse_edge_prepare(sg_problem* pr) {
+  EdgeVals& E = pr->solver->pc.co.edge;
+  if (E.v32.ptr) return SG_OK;
+  EdgeVals v;
+  SG_TRY(coarse_edge_build(pr, v));
+  E = std::move(v);
+  return SG_OK;
+}
 bool coarse_edge_default(const sg_problem* pr) {
   return pr->solver ? pr->solver->pc.coarse_edge : coarse_edge_form(pr);
 }

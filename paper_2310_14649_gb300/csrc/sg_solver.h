@@ -96,7 +96,7 @@ struct CoarseData {
   int64_t nc = 0, ldc = 0;
   std::vector<int32_t> rowptr, colidx;     // coarse CSR pattern (host)
   Ell ell;                                 // coarse A_k in ELL form (device)
-  EdgeVals edge;                           // the same in the edge form (FP32 conductances)
+  EdgeVals edge;                           // the same in the edge form (FP32 conductances; coarse_edge_prepare)
   TripleTables tri;
   DevCsr RT, R;                            // interpolation (n x nc) and restriction
   AsmBlocks asm_c;                         // assembled FP64 blocks of the coarse operator
@@ -162,6 +162,9 @@ sg_status amg_setup_fine(const sg_problem* pr, AmgHier& h);
 const Ell& coarse_ell(const sg_problem* pr);
 const TripleTables& coarse_tri(const sg_problem* pr);
 const EdgeVals& coarse_edge(const sg_problem* pr);
+// its FP32 conductances, where the coarse family runs on the edge form (or is
+// timed on it); synchronous when they are not there yet
+sg_status coarse_edge_prepare(sg_problem* pr);
 // the coarse operator's untuned form: the preconditioner's, or what it will be
 bool coarse_edge_default(const sg_problem* pr);
 AsmBlocks& coarse_asm(sg_problem* pr);

@@ -550,3 +550,24 @@ def test_coarse_form_is_the_preconditioners(gpu):
     slot = correction(before)
     assert not torch.equal(slot, edge)
     assert torch.equal(correction(late), slot) and torch.equal(correction(early), slot)
+
+
+def test_coarse_conductances_only_where_they_are_read(gpu):
+    """A handle whose coarse operator runs on the slot form (P > 48, untuned)
+    holds no coarse conductances (K x 2 (N/2) (N/2 - 1) FP32 values, 15 MB
+    here); tuning the coarse family makes them, and the operator agrees."""
+    import torch
+    import paper_2310_14649_gb300 as sg
+    N = 128
+    prob = sg.sg_setup(N, 5, 3, 6, sigma2=0.3, bx=0.5, by=0.5)
+    sg.sg_precond_setup(prob, 6, 6, 1, omega=0.3)
+    R = torch.from_numpy(random_block(prob.nc, prob.P, seed=45).T.copy()).float().cuda()
+    Z, Y = torch.zeros_like(R), torch.zeros_like(R)
+    sg.sg_precond_apply(prob, sg.PC_COARSE_APPLY, R, Z)
+    sg.sg_set_apply_fp64(prob, 1)                    # drops the solver's vectors, as tuning does
+    before = torch.cuda.mem_get_info()[0]
+    sg.sg_apply_autotune(prob, which=1)
+    assert before - torch.cuda.mem_get_info()[0] >= 0.9 * prob.K * 2 * (N // 2) * (N // 2 - 1) * 4
+    sg.sg_precond_apply(prob, sg.PC_COARSE_APPLY, R, Y)
+    assert (Y - Z).norm() <= 1e-5 * Z.norm()
+    prob.close()
