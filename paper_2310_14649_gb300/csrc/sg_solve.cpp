@@ -229,14 +229,11 @@ using namespace sg;
 template <typename T>
 static sg_status precond_apply_t(sg_problem* pr, int which, const T* Rin, int64_t ldr, T* Zout, int64_t ldz,
                                  cudaStream_t st) {
-  SolverCtx<T>* c = nullptr;
-  SG_TRY(get_ctx<T>(pr, c));
   SolverState& S = *pr->solver;
   const int P = pr->P;
   const bool coarse_in = which == 3 || which == 4 || which == 6;
   const bool coarse_out = which == 3 || which == 4 || which == 5;
-  const int64_t nin = coarse_in ? S.pc.co.nc : pr->n, ldin = coarse_in ? c->ldc : c->ld;
-  const int64_t nout = coarse_out ? S.pc.co.nc : pr->n, ldout = coarse_out ? c->ldc : c->ld;
+  const int64_t nin = coarse_in ? S.pc.co.nc : pr->n, nout = coarse_out ? S.pc.co.nc : pr->n;
   SG_ARG(ldr >= nin && ldz >= nout, "sg_precond_apply: leading dimension too small");
   const bool learned = which == 8 || which == 9;
   if (learned) {
@@ -251,7 +248,8 @@ static sg_status precond_apply_t(sg_problem* pr, int which, const T* Rin, int64_
     ~Restore() { pc.use_cnn = v; }
   } restore{S.pc, prev_cnn};
   // the explicit inverses read and write blocks of any leading dimension: the
-  // four passes over a block below were 35 of 181 us at 256^2, P = 35
+  // four passes over a block below were 35 of 181 us at 256^2, P = 35, and a
+  // program that only smooths needs none of the solver's vectors
   if constexpr (sizeof(T) == 4)
     if ((which == 7 || (which == 1 && !S.pc.use_cnn && !S.pc.harvest.on)) && S.pc.ras_kernel == 2 &&
         S.pc.ras.d_inv.ptr && ras_inverse_disjoint(P, Rin, ldr, Zout, ldz)) {
@@ -264,6 +262,9 @@ static sg_status precond_apply_t(sg_problem* pr, int which, const T* Rin, int64_
       if (timed) SG_TRY(prof->end(slot, st));
       return SG_OK;
     }
+  SolverCtx<T>* c = nullptr;
+  SG_TRY(get_ctx<T>(pr, c));
+  const int64_t ldin = coarse_in ? c->ldc : c->ld, ldout = coarse_out ? c->ldc : c->ld;
   T* in = coarse_in ? dp<T>(c->coarse.tmp) : dp<T>(c->fine.tmp);
   T* out = coarse_out ? dp<T>(c->coarse.tmp2) : dp<T>(c->fine.tmp2);
   SG_CUDA(cudaMemsetAsync(in, 0, size_t(P) * ldin * sizeof(T), st));

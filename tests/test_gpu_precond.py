@@ -571,3 +571,24 @@ def test_coarse_conductances_only_where_they_are_read(gpu):
     sg.sg_precond_apply(prob, sg.PC_COARSE_APPLY, R, Y)
     assert (Y - Z).norm() <= 1e-5 * Z.norm()
     prob.close()
+
+
+def test_smoother_alone_allocates_no_solver_vectors(gpu):
+    """The explicit local inverses work on the caller's blocks: a program that
+    only smooths allocates none of the solver's 62 vectors (2 MB each here),
+    and an operator that needs them still finds them."""
+    import torch
+    import paper_2310_14649_gb300 as sg
+    prob = sg.sg_setup(128, 4, 3, 6, sigma2=0.3, bx=0.5, by=0.5)
+    sg.sg_precond_setup(prob, 5, 5, 1, omega=0.3, ras_kernel=2)
+    R = torch.from_numpy(random_block(prob.n, prob.P, seed=46).T.copy()).float().cuda()
+    Z, Y = torch.zeros_like(R), torch.zeros_like(R)
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    for which in (sg.PC_SMOOTH, sg.PC_RAS_LOCAL):
+        sg.sg_precond_apply(prob, which, R, Z)
+    torch.cuda.synchronize()
+    assert before - torch.cuda.mem_get_info()[0] < 62 * R.numel() * 4 // 8
+    sg.sg_precond_apply(prob, sg.PC_TWOLEVEL, R, Y)
+    assert bool(torch.isfinite(Y).all()) and bool(Y.any())
+    prob.close()
