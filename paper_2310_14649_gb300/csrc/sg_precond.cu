@@ -4,6 +4,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "sg_df.h"
 #include "sg_kernels.h"
 #include "sg_solver.h"
 
@@ -719,8 +720,6 @@ struct AmgPhase {
   T* Y = nullptr;         // t (kDown, kResid), b_{l+1}, x (kProlong, +=), out (kFinal)
   int64_t ldy = 0;
   T* Y2 = nullptr;        // kDown: x = D^{-1} b (ld ldy)
-  const int* j = nullptr; // kRestrict: the gathered vector is block *j of X, xstride apart
-  int64_t xstride = 0;
 };
 
 // MB modes per thread group: the row's pattern and values are read once
@@ -733,7 +732,6 @@ __global__ void __launch_bounds__(128) k_amg_phase(const __grid_constant__ AmgPh
   const int64_t a0 = int64_t(blockIdx.y) * MB;
   const int nm = int(min(int64_t(MB), int64_t(p.P) - a0));
   const bool live = i < p.n;
-  const T* X0 = OP == kRestrict && p.j ? p.X + int64_t(*p.j) * p.xstride : p.X;
   T acc[MB];
 #pragma unroll
   for (int m = 0; m < MB; ++m) acc[m] = T(0);
@@ -747,7 +745,7 @@ __global__ void __launch_bounds__(128) k_amg_phase(const __grid_constant__ AmgPh
 #pragma unroll
       for (int m = 0; m < MB; ++m) {
         if (m < nm) {
-          const T* X = X0 + (a0 + m) * p.ldx;
+          const T* X = p.X + (a0 + m) * p.ldx;
           T g;
           if (OP == kDown)
             g = dj * X[j];
@@ -785,15 +783,17 @@ __global__ void __launch_bounds__(128) k_amg_phase(const __grid_constant__ AmgPh
   }
 }
 
-// the phase kernel with the largest MB in {1, 2, 4, 8} that still leaves
-// about one wave of resident threads (152 SMs x 2048) of (row, mode group)
-// lane groups
+// the largest mode group MB in {1, 2, 4, 8} that still leaves about one wave
+// of resident threads (152 SMs x 2048) of (row, mode group) lane groups
+int mode_group(int n, int G, int P) {
+  int MB = 8;
+  while (MB > 1 && int64_t(n) * G * ((P + MB - 1) / MB) < 152 * 2048) MB >>= 1;
+  return MB;
+}
+
 template <typename T, int OP>
 cudaError_t amg_phase_launch(const AmgPhase<T>& p, cudaStream_t st) {
-  const int rows = 128 / p.G;
-  const int64_t lanes_per_mode_group = int64_t(p.n) * p.G;
-  int MB = 8;
-  while (MB > 1 && lanes_per_mode_group * ((p.P + MB - 1) / MB) < 152 * 2048) MB >>= 1;
+  const int rows = 128 / p.G, MB = mode_group(p.n, p.G, p.P);
   const dim3 grid(unsigned((p.n + rows - 1) / rows), unsigned((p.P + MB - 1) / MB));
   switch (MB) {
     case 8: k_amg_phase<T, OP, 8><<<grid, 128, 0, st>>>(p); break;
@@ -1156,40 +1156,109 @@ sg_status amg_vcycle(const AmgHier& H, AmgWork<T>& w, int P, cudaStream_t st, T*
 // ---------------------------------------------------------------------------
 // Folded FP32 V-cycle (AmgFold).  A cycle of four levels took 13 launches of
 // 4.5 to 14 us, bound by launch latency and short dependent loads; folded it
-// takes three (down, dense, up), and in the recorded coarse solves the copy of
-// the input and the Kronecker factor, two launches more, are part of the
-// first and the last.  256^2, P = 35 (16,129 coarse unknowns): 83 us of
-// kernels a cycle, now 34 (9.2 + 6.8 + 17.8); a coarse solve at tolerance
-// 1e-5 3.02 ms, now 2.58.  A hierarchy of one level is the dense product alone
-// (32^2, 225 unknowns: 35 us, now 6).
+// takes two per sparse level and the dense product, and in the recorded coarse
+// solves the copy of the input and the Kronecker factor, two launches more,
+// are part of the first and the last.
+// Every sum is carried in double-FP32 (of products rounded to FP32; in large
+// dense parts of FP32 partial sums of 16 or 32 terms): in plain FP32 the
+// longer rows and the dense part, which takes the place of the coarsest
+// level's FP64 inverse, cost accuracy.  Relative L2 error against the FP64
+// cycle for random blocks, one kernel per level operation / folded in plain
+// FP32 / now: 32^2 2.6e-8 / 1.4e-7 / 2.6e-8, 96^2 8.7e-8 / 1.0e-7 / 6.2e-8,
+// 200^2 8.7e-8 / 1.6e-7 / 6.6e-8, 256^2 9.2e-8 / 1.0e-7 / 6.7e-8.
+// Bound by the latency of the gathers: 256^2, P = 35 (16,129 coarse unknowns,
+// two sparse levels), us of the five kernels under ncu, in plain FP32 with one
+// entry's gathers in flight and now with four: 12.3 + 6.3 + 6.3 + 20.0 + 15.5,
+// 12.9 + 7.0 + 6.1 + 13.3 + 11.2; a coarse solve at tolerance 1e-5 3.02 ms
+// unfolded, 2.58 and 2.43 ms.  A hierarchy of one level is the dense product
+// alone (32^2, 225 unknowns: 35 us unfolded, 5.6 in plain FP32, now 7.1).
 // ---------------------------------------------------------------------------
 namespace {
 
-constexpr int kDenseRows = 64, kDenseSplit = 8, kDenseModes = 48, kDenseLd = 52;
+constexpr int kDenseRows = 64, kDenseSplit = 8;
 
-// X = B b for the dense part: a cluster of eight CTAs per 64 rows and 48
+struct FoldDown {
+  int n = 0, G = 1, P = 0;
+  const int *rp = nullptr, *ci = nullptr;
+  const float* v = nullptr;
+  const float* b = nullptr;   // block *j of b when j
+  int64_t ldb = 0, bstride = 0;
+  const int* j = nullptr;
+  float* out = nullptr;
+  int64_t ldo = 0;
+};
+
+// b_{l+1} = R' b_l: a group of G lanes per row and MB modes (k_amg_phase)
+template <int MB>
+__global__ void __launch_bounds__(128) k_fold_down(const __grid_constant__ FoldDown p) {
+  const int G = p.G;
+  const int grp = threadIdx.x / G, lane = threadIdx.x - grp * G;
+  const int i = blockIdx.x * (128 / G) + grp;
+  const int64_t a0 = int64_t(blockIdx.y) * MB;
+  const int nm = int(min(int64_t(MB), int64_t(p.P) - a0));
+  const bool live = i < p.n;
+  const float* b = p.b + (p.j ? int64_t(*p.j) * p.bstride : 0) + a0 * p.ldb;
+  Df acc[MB];
+#pragma unroll
+  for (int m = 0; m < MB; ++m) acc[m] = Df{0.f, 0.f};
+  if (live) {
+    const int e1 = p.rp[i + 1];
+    for (int e = p.rp[i] + lane; e < e1; e += G) {
+      const int c = p.ci[e];
+      const float v = p.v[e];
+#pragma unroll
+      for (int m = 0; m < MB; ++m)
+        if (m < nm) df_accumulate(acc[m], __fmul_rn(v, b[m * p.ldb + c]));
+    }
+  }
+#pragma unroll
+  for (int m = 0; m < MB; ++m)
+    for (int o = G >> 1; o > 0; o >>= 1)
+      acc[m] = df_add(acc[m], Df{__shfl_xor_sync(0xffffffffu, acc[m].h, o), __shfl_xor_sync(0xffffffffu, acc[m].l, o)});
+  if (!live || lane != 0) return;
+#pragma unroll
+  for (int m = 0; m < MB; ++m)
+    if (m < nm) p.out[(a0 + m) * p.ldo + i] = df_value(acc[m]);
+}
+
+// x = B b for the dense part: a cluster of eight CTAs per 64 rows and 4 MT
 // modes, each a slice of the sum (its matrix and vector slices brought to
 // shared memory in one round of 16-byte copies), the partial sums added over
 // the cluster in rank order through distributed shared memory.  At n = 1,849
-// the matrix is 13.7 MB, read once from L2.  b, x: mode-major.
+// the matrix is 13.7 MB, read once from L2.  b, x: mode-major.  A warp holds
+// 64 rows of MT modes: 3 up to n = 1,024 or 12 modes, where smaller tiles fill
+// the GPU (n = 687, 35 modes: 12 a warp 10.6 us, 3 a warp 7.6), else 12, which
+// reads the matrix once for 48 modes (n = 1,674, 35 modes: 19.3 us, 3 a warp 30.3).
+// EXACT (n <= kFoldExact, where the dense part replaces little but the FP64
+// inverse of the coarsest level): the matrix as hi + lo, every product and
+// sum in double-FP32, so the result is the FP64 one rounded.  Else C products
+// at a time in FP32 and these sums in double-FP32 (n = 1,674, 15 modes, 12 a
+// warp: 17.1 us with no double-FP32, 20.7 with C = 16, 18.3 with 32).
+template <bool EXACT, int MT>
 __global__ void __cluster_dims__(kDenseSplit, 1, 1) __launch_bounds__(128)
-    k_fold_dense(int n, int64_t ldd, const float* __restrict__ B, const float* __restrict__ b, int64_t ldb, int P,
-                 float* __restrict__ x, int64_t ldx, int slice, const int* __restrict__ j, int64_t bstride) {
+    k_fold_dense(int n, int64_t ldd, const float* __restrict__ B, const float* __restrict__ Blo,
+                 const float* __restrict__ b, int64_t ldb, int P, float* __restrict__ x, int64_t ldx, int slice,
+                 const int* __restrict__ j, int64_t bstride) {
+  constexpr int M = 4 * MT, C = MT == 12 ? 32 : 16;
+  constexpr int LD = MT == 12 ? 52 : 13;               // a mode's store along k meets 8 or 32 banks
   extern __shared__ __align__(16) float sm_fold[];
-  float* Bs = sm_fold;                       // [slice][64]
-  float* bs = Bs + slice * kDenseRows;       // [slice][52]: a mode's store along k meets 8 banks
-  const int rank = blockIdx.x, row0 = blockIdx.y * kDenseRows, a0 = blockIdx.z * kDenseModes;
-  const int k0 = rank * slice, kn = max(0, min(slice, n - k0)), nm = min(kDenseModes, P - a0);
+  float* Bs = sm_fold;                                 // [slice][64]
+  float* Ls = Bs + slice * kDenseRows;                 // EXACT: [slice][64]
+  float* bs = Ls + (EXACT ? slice * kDenseRows : 0);   // [slice][LD]
+  const int rank = blockIdx.x, row0 = blockIdx.y * kDenseRows, a0 = blockIdx.z * M;
+  const int k0 = rank * slice, kn = max(0, min(slice, n - k0)), nm = min(M, P - a0);
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   if (j) b += int64_t(*j) * bstride;
   for (int q = tid; q < kn * (kDenseRows / 4); q += 128) {
     const int k = q / (kDenseRows / 4), c = q % (kDenseRows / 4);
     // columns row0 .. row0 + 63 of row k (the matrix is symmetric; ldd covers whole tiles)
-    cp_async16(Bs + k * kDenseRows + 4 * c, B + int64_t(k0 + k) * ldd + row0 + 4 * c);
+    const int64_t at = int64_t(k0 + k) * ldd + row0 + 4 * c;
+    cp_async16(Bs + k * kDenseRows + 4 * c, B + at);
+    if (EXACT) cp_async16(Ls + k * kDenseRows + 4 * c, Blo + at);
   }
   for (int k = tid; k < kn; k += 128)
-    for (int m = 0; m < kDenseModes; ++m) {
-      float* dst = bs + k * kDenseLd + m;
+    for (int m = 0; m < M; ++m) {
+      float* dst = bs + k * LD + m;
       if (m < nm)
         asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(
                          static_cast<uint32_t>(__cvta_generic_to_shared(dst))),
@@ -1201,45 +1270,92 @@ __global__ void __cluster_dims__(kDenseSplit, 1, 1) __launch_bounds__(128)
   cp_async_commit();
   cp_async_wait_all();
   __syncthreads();
-  // thread: rows 2 lane, 2 lane + 1, modes 12 w .. 12 w + 11
-  float acc[2][12];
+  // thread: rows 2 lane, 2 lane + 1, modes MT w .. MT w + MT - 1
+  Df sum[2][MT];
 #pragma unroll
-  for (int m = 0; m < 12; ++m) acc[0][m] = acc[1][m] = 0.f;
+  for (int m = 0; m < MT; ++m) sum[0][m] = sum[1][m] = Df{0.f, 0.f};
+  auto vec = [&](int k, float (&e)[MT]) {
+    const float* v = bs + k * LD + MT * w;
+    if constexpr (MT % 4 == 0) {
+#pragma unroll
+      for (int u = 0; u < MT; u += 4) {
+        const float4 t = *reinterpret_cast<const float4*>(v + u);
+        e[u] = t.x;
+        e[u + 1] = t.y;
+        e[u + 2] = t.z;
+        e[u + 3] = t.w;
+      }
+    } else {
+#pragma unroll
+      for (int u = 0; u < MT; ++u) e[u] = v[u];
+    }
+  };
+  if (MT * w >= nm) {
+    // no modes for this warp
+  } else if constexpr (EXACT) {
+    auto add = [](Df& s, float hi, float lo, float v) {
+      const float p = __fmul_rn(hi, v);
+      const float e = fmaf(lo, v, fmaf(hi, v, -p));
+      const Df t = two_sum(s.h, p);
+      s = Df{t.h, __fadd_rn(s.l, __fadd_rn(t.l, e))};
+    };
+    for (int k = 0; k < kn; ++k) {
+      const float2 r = *reinterpret_cast<const float2*>(Bs + k * kDenseRows + 2 * lane);
+      const float2 l = *reinterpret_cast<const float2*>(Ls + k * kDenseRows + 2 * lane);
+      float e[MT];
+      vec(k, e);
+#pragma unroll
+      for (int m = 0; m < MT; ++m) {
+        add(sum[0][m], r.x, l.x, e[m]);
+        add(sum[1][m], r.y, l.y, e[m]);
+      }
+    }
+  } else {
+    for (int kc = 0; kc < kn; kc += C) {
+      float acc[2][MT];
+#pragma unroll
+      for (int m = 0; m < MT; ++m) acc[0][m] = acc[1][m] = 0.f;
+      const int ke = min(kc + C, kn);
 #pragma unroll 4
-  for (int k = 0; k < kn; ++k) {
-    const float2 r = *reinterpret_cast<const float2*>(Bs + k * kDenseRows + 2 * lane);
-    const float4* v = reinterpret_cast<const float4*>(bs + k * kDenseLd + 12 * w);
+      for (int k = kc; k < ke; ++k) {
+        const float2 r = *reinterpret_cast<const float2*>(Bs + k * kDenseRows + 2 * lane);
+        float e[MT];
+        vec(k, e);
 #pragma unroll
-    for (int u = 0; u < 3; ++u) {
-      const float4 t = v[u];
-      const float e[4] = {t.x, t.y, t.z, t.w};
+        for (int m = 0; m < MT; ++m) {
+          acc[0][m] = fmaf(r.x, e[m], acc[0][m]);
+          acc[1][m] = fmaf(r.y, e[m], acc[1][m]);
+        }
+      }
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        acc[0][4 * u + i] = fmaf(r.x, e[i], acc[0][4 * u + i]);
-        acc[1][4 * u + i] = fmaf(r.y, e[i], acc[1][4 * u + i]);
+      for (int m = 0; m < MT; ++m) {
+        df_accumulate(sum[0][m], acc[0][m]);
+        df_accumulate(sum[1][m], acc[1][m]);
       }
     }
   }
   __syncthreads();
-  float* part = sm_fold;                     // [48][64]
+  float2* part = reinterpret_cast<float2*>(sm_fold);   // [M][64]
 #pragma unroll
-  for (int m = 0; m < 12; ++m)
-    *reinterpret_cast<float2*>(part + (12 * w + m) * kDenseRows + 2 * lane) = make_float2(acc[0][m], acc[1][m]);
+  for (int m = 0; m < MT; ++m)
+    *reinterpret_cast<float4*>(part + (MT * w + m) * kDenseRows + 2 * lane) =
+        make_float4(sum[0][m].h, sum[0][m].l, sum[1][m].h, sum[1][m].l);
   asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
-  // this CTA sums modes 6 rank .. 6 rank + 5 over the cluster
+  // this CTA sums an eighth of the tile's results over the cluster
+  constexpr int E = M * kDenseRows / kDenseSplit;
   const uint32_t base = static_cast<uint32_t>(__cvta_generic_to_shared(part));
-  for (int q = tid; q < (kDenseModes / kDenseSplit) * kDenseRows; q += 128) {
-    const int m = rank * (kDenseModes / kDenseSplit) + q / kDenseRows, r = q % kDenseRows;
-    float s = 0.f;
+  for (int q = rank * E + tid; q < (rank + 1) * E; q += 128) {
+    const int m = q / kDenseRows, r = q % kDenseRows;
+    Df s{0.f, 0.f};
 #pragma unroll
     for (int c = 0; c < kDenseSplit; ++c) {
       uint32_t addr;
-      float v;
-      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(addr) : "r"(base + 4u * (m * kDenseRows + r)), "r"(c));
-      asm volatile("ld.shared::cluster.f32 %0, [%1];\n" : "=f"(v) : "r"(addr) : "memory");
-      s += v;
+      Df v;
+      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(addr) : "r"(base + 8u * q), "r"(c));
+      asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];\n" : "=f"(v.h), "=f"(v.l) : "r"(addr) : "memory");
+      s = df_add(s, v);
     }
-    if (m < nm && row0 + r < n) x[int64_t(a0 + m) * ldx + row0 + r] = s;
+    if (m < nm && row0 + r < n) x[int64_t(a0 + m) * ldx + row0 + r] = df_value(s);
   }
   // no CTA leaves while another reads its partial sums
   asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
@@ -1280,27 +1396,39 @@ __global__ void __launch_bounds__(128) k_fold_up(const __grid_constant__ FoldUp 
       const int c = e / (4 * MW), a = e - c * 4 * MW;
       Ms[e] = a < p.P ? p.M[a * p.P + c] : 0.f;
     }
+  Df sum[MW];
+#pragma unroll
+  for (int m = 0; m < MW; ++m) sum[m] = Df{0.f, 0.f};
+  // U entries' gathers in flight, two products to a sum
+  constexpr int U = MW <= 12 ? 4 : 2;
+  auto row = [&](const int* __restrict__ rp, const int* __restrict__ ci, const float* __restrict__ vals,
+                 const float* __restrict__ x, int64_t ld) {
+    const int e1 = rp[r + 1];
+    for (int e = rp[r]; e < e1; e += U) {
+      int c[U];
+      float v[U], g[U][MW];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        c[u] = e + u < e1 ? ci[e + u] : -1;
+        v[u] = e + u < e1 ? vals[e + u] : 0.f;
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int m = 0; m < MW; ++m) g[u][m] = c[u] >= 0 && a0 + m < p.P ? x[int64_t(a0 + m) * ld + c[u]] : 0.f;
+#pragma unroll
+      for (int u = 0; u < U; u += 2)
+#pragma unroll
+        for (int m = 0; m < MW; ++m) df_accumulate(sum[m], fmaf(v[u + 1], g[u + 1][m], __fmul_rn(v[u], g[u][m])));
+    }
+  };
+  if (live) {
+    row(p.rpS, p.ciS, p.vS, b, p.ldb);
+    row(p.rpP, p.ciP, p.vP, p.xc, p.ldc);
+  }
   float acc[MW];
 #pragma unroll
-  for (int m = 0; m < MW; ++m) acc[m] = 0.f;
-  if (live) {
-    const int e1 = p.rpS[r + 1];
-    for (int e = p.rpS[r]; e < e1; ++e) {
-      const int c = p.ciS[e];
-      const float v = p.vS[e];
-#pragma unroll
-      for (int m = 0; m < MW; ++m)
-        if (a0 + m < p.P) acc[m] = fmaf(v, b[int64_t(a0 + m) * p.ldb + c], acc[m]);
-    }
-    const int f1 = p.rpP[r + 1];
-    for (int e = p.rpP[r]; e < f1; ++e) {
-      const int c = p.ciP[e];
-      const float v = p.vP[e];
-#pragma unroll
-      for (int m = 0; m < MW; ++m)
-        if (a0 + m < p.P) acc[m] = fmaf(v, p.xc[int64_t(a0 + m) * p.ldc + c], acc[m]);
-    }
-  }
+  for (int m = 0; m < MW; ++m) acc[m] = df_value(sum[m]);
   if (p.M) {
 #pragma unroll
     for (int m = 0; m < MW; ++m)
@@ -1331,9 +1459,13 @@ __global__ void __launch_bounds__(128) k_fold_up(const __grid_constant__ FoldUp 
     }
 }
 
-__global__ void k_fold_round(const double* __restrict__ x, int64_t ldx, int n, float* __restrict__ B, int64_t ldd) {
+__global__ void k_fold_round(const double* __restrict__ x, int64_t ldx, int n, float* __restrict__ B,
+                             float* __restrict__ lo, int64_t ldd) {
   const int c = blockIdx.x * blockDim.x + threadIdx.x, r = blockIdx.y;
-  if (c < n) B[int64_t(r) * ldd + c] = float(x[int64_t(r) * ldx + c]);
+  if (c >= n) return;
+  const double v = x[int64_t(r) * ldx + c];
+  B[int64_t(r) * ldd + c] = float(v);
+  if (lo) lo[int64_t(r) * ldd + c] = float(v - double(float(v)));
 }
 __global__ void k_fold_units(double* __restrict__ b, int64_t ld, int n) {
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1341,9 +1473,10 @@ __global__ void k_fold_units(double* __restrict__ b, int64_t ld, int n) {
 }
 
 int fold_slice(int64_t n) { return int(round_up((n + kDenseSplit - 1) / kDenseSplit, 4)); }
+// the largest over both mode tiles
 size_t fold_dense_smem(int64_t n) {
-  const size_t s = size_t(fold_slice(n)) * (kDenseRows + kDenseLd), part = size_t(kDenseModes) * kDenseRows;
-  return std::max(s, part) * sizeof(float);
+  const size_t s = size_t(fold_slice(n)) * (kDenseRows * (n <= kFoldExact ? 2 : 1) + 52) * sizeof(float);
+  return std::max(s, size_t(48) * kDenseRows * sizeof(float2));
 }
 
 template <int MW>
@@ -1358,8 +1491,14 @@ sg_status fold_up_launch(const FoldUp& p, cudaStream_t st) {
 }  // namespace
 
 sg_status fold_attrs_init() {
-  SG_CUDA(cudaFuncSetAttribute(k_fold_dense, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  SG_CUDA(cudaFuncSetAttribute(k_fold_dense<false, 12>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                int(fold_dense_smem(kFoldMax))));
+  SG_CUDA(cudaFuncSetAttribute(k_fold_dense<false, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               int(fold_dense_smem(kFoldMax))));
+  SG_CUDA(cudaFuncSetAttribute(k_fold_dense<true, 12>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               int(fold_dense_smem(kFoldExact))));
+  SG_CUDA(cudaFuncSetAttribute(k_fold_dense<true, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               int(fold_dense_smem(kFoldExact))));
   SG_CUDA(cudaFuncSetAttribute(k_fold_up<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024));
   return SG_OK;
 }
@@ -1385,7 +1524,9 @@ sg_status amg_fold_dense(AmgHier& H) {
   SG_TRY(amg_vcycle<double>(H, w, n, nullptr, nullptr, 0, F.lf));
   F.ldd = round_up(n, kDenseRows);
   SG_TRY(F.dense.alloc(size_t(n) * F.ldd * 4));
-  k_fold_round<<<dim3(unsigned((n + 127) / 128), unsigned(n)), 128>>>(w.x[F.lf], ld, n, F.dense.as<float>(), F.ldd);
+  if (n <= kFoldExact) SG_TRY(F.dense_lo.alloc(size_t(n) * F.ldd * 4));
+  k_fold_round<<<dim3(unsigned((n + 127) / 128), unsigned(n)), 128>>>(w.x[F.lf], ld, n, F.dense.as<float>(),
+                                                                      F.dense_lo.as<float>(), F.ldd);
   note_launch();
   SG_CUDA(cudaGetLastError());
   SG_CUDA(cudaDeviceSynchronize());
@@ -1402,29 +1543,41 @@ sg_status amg_fold_apply(const AmgHier& H, AmgWork<float>& w, int P, const float
     const int64_t avg = R.n > 0 ? (R.nnz + R.n - 1) / R.n : 1;
     int G = 1;
     while (G < 32 && 2 * G < avg && R.n * int64_t(P) * (2 * G) <= 2 * 152 * 2048) G <<= 1;
-    AmgPhase<float> p;
+    FoldDown p;
     p.n = int(R.n);
-    p.P = P;
     p.G = G;
+    p.P = P;
     p.rp = R.rowptr.as<int>();
     p.ci = R.col.as<int>();
     p.v = R.v32.as<float>();
-    p.X = l ? w.b[l] : b;
-    p.ldx = l ? H[l].ld : ldb;
+    p.b = l ? w.b[l] : b;
+    p.ldb = l ? H[l].ld : ldb;
     p.j = l ? nullptr : j;
-    p.xstride = bstride;
-    p.Y = w.b[l + 1];
-    p.ldy = H[l + 1].ld;
-    SG_CUDA((amg_phase_launch<float, kRestrict>(p, st)));
+    p.bstride = bstride;
+    p.out = w.b[l + 1];
+    p.ldo = H[l + 1].ld;
+    const int MB = mode_group(p.n, G, P), rows = 128 / G;
+    const dim3 grid(unsigned((p.n + rows - 1) / rows), unsigned((P + MB - 1) / MB));
+    switch (MB) {
+      case 8: k_fold_down<8><<<grid, 128, 0, st>>>(p); break;
+      case 4: k_fold_down<4><<<grid, 128, 0, st>>>(p); break;
+      case 2: k_fold_down<2><<<grid, 128, 0, st>>>(p); break;
+      default: k_fold_down<1><<<grid, 128, 0, st>>>(p); break;
+    }
+    note_launch();
+    SG_CUDA(cudaGetLastError());
   }
   {
     const AmgLevel& L = H[F.lf];
     const int n = int(L.n);
-    const dim3 grid(kDenseSplit, unsigned((n + kDenseRows - 1) / kDenseRows), unsigned((P + kDenseModes - 1) / kDenseModes));
+    const int modes = P <= 12 || n <= 1024 ? 12 : 48;
+    const dim3 grid(kDenseSplit, unsigned((n + kDenseRows - 1) / kDenseRows), unsigned((P + modes - 1) / modes));
     const bool all = F.lf == 0;  // the whole cycle
-    k_fold_dense<<<grid, 128, fold_dense_smem(n), st>>>(n, F.ldd, F.dense.as<float>(), all ? b : w.b[F.lf],
-                                                        all ? ldb : L.ld, P, all ? out : w.x[F.lf], all ? ldo : L.ld,
-                                                        fold_slice(n), all ? j : nullptr, bstride);
+    const auto dense = n <= kFoldExact ? (modes == 12 ? k_fold_dense<true, 3> : k_fold_dense<true, 12>)
+                                       : (modes == 12 ? k_fold_dense<false, 3> : k_fold_dense<false, 12>);
+    dense<<<grid, 128, fold_dense_smem(n), st>>>(n, F.ldd, F.dense.as<float>(), F.dense_lo.as<float>(),
+                                                 all ? b : w.b[F.lf], all ? ldb : L.ld, P, all ? out : w.x[F.lf],
+                                                 all ? ldo : L.ld, fold_slice(n), all ? j : nullptr, bstride);
     note_launch();
     SG_CUDA(cudaGetLastError());
     if (all) return M ? node_transform<float>(out, ldo, n, P, M, st, Z2, stride2, Z2 ? j : nullptr) : SG_OK;

@@ -621,7 +621,9 @@ static sg_status setup_amg(AmgHier& H, const HCsr& A0c, bool fold) {
   AmgFold& F = H.fold;
   F.lf = As.size() > 1 ? 1 : 0;
   while (As[F.lf].n > kFoldMax && F.lf + 1 < int(As.size())) ++F.lf;
-  if (As[F.lf].n > kFoldMax) return SG_OK;  // the coarsening stalled: no dense part
+  // no dense part where the coarsening stalled (a single level beyond
+  // kFoldExact keeps the FP64 inverse)
+  if (As[F.lf].n > (F.lf == 0 ? kFoldExact : kFoldMax)) return SG_OK;
   F.Rp.resize(F.lf);
   F.Pp.resize(F.lf);
   F.S.resize(F.lf);

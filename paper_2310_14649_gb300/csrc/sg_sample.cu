@@ -14,6 +14,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "sg_df.h"
 #include "sg_internal.h"
 
 namespace sg {
@@ -23,26 +24,10 @@ constexpr int kSampThreads = 512;      // most threads of a CTA
 constexpr int kSampMaxNodes = 10240;   // meshes up to N = 102
 constexpr int kSampMaxRun = 21;        // most nodes of a thread (m = 101: 5 runs of a column)
 
-// Double-FP32 number hi + lo (48 significant bits).  The sums over a block
-// and the scalars of the CG recurrence are carried in it: GB300 runs FP64 at
-// 1/64 of its FP32 rate, and the FP64 sums this replaces (every thread
-// adding 64 partial sums per reduction) were 90 % of an iteration.
-struct Df {
-  float h, l;
-};
-
-// exact sum of two floats as hi + lo (TwoSum, Knuth)
-__device__ __forceinline__ Df two_sum(float a, float b) {
-  const float s = __fadd_rn(a, b);
-  const float bb = __fsub_rn(s, a);
-  return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb))};
-}
-// a + b with the rounding error gathered in the low word; symmetric in its
-// arguments, so a butterfly gives every lane the same bits
-__device__ __forceinline__ Df df_add(Df a, Df b) {
-  const Df s = two_sum(a.h, b.h);
-  return {s.h, __fadd_rn(__fadd_rn(a.l, b.l), s.l)};
-}
+// The sums over a block and the scalars of the CG recurrence are carried in
+// double-FP32: GB300 runs FP64 at 1/64 of its FP32 rate, and the FP64 sums
+// this replaces (every thread adding 64 partial sums per reduction) were 90 %
+// of an iteration.
 // float(a / b): the quotient of the high words corrected by its remainder
 __device__ __forceinline__ float df_div(Df a, Df b) {
   const float q = __fdiv_rn(a.h, b.h);

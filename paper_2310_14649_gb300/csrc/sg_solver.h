@@ -36,12 +36,13 @@ struct AmgLevel {
 // (A symmetric), so a level costs two launches instead of four and the
 // levels from the first with at most kFoldMax unknowns one dense product.
 constexpr int kFoldMax = 2048;
+constexpr int kFoldExact = 256;  // dense parts up to this size keep their values in 48 bits
 constexpr int kFoldModes = 128;  // modes of the kernel with the Kronecker factor
 struct AmgFold {
   bool ready = false;
   int lf = 0;                       // first level of the dense part
   std::vector<DevCsr> Rp, Pp, S;    // levels 0 .. lf - 1
-  DevBuf dense;                     // float n_lf x ldd, symmetric
+  DevBuf dense, dense_lo;           // float n_lf x ldd, symmetric; the remainders (n_lf <= kFoldExact)
   int64_t ldd = 0;
 };
 

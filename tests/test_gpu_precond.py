@@ -592,3 +592,31 @@ def test_smoother_alone_allocates_no_solver_vectors(gpu):
     sg.sg_precond_apply(prob, sg.PC_TWOLEVEL, R, Y)
     assert bool(torch.isfinite(Y).all()) and bool(Y.any())
     prob.close()
+
+
+@pytest.mark.parametrize("N,L,p", [(32, 2, 2), (36, 3, 2), (58, 3, 2), (66, 3, 3), (96, 4, 3), (200, 3, 2), (256, 4, 2)])
+def test_amg_fold_is_no_less_accurate(gpu, N, L, p):
+    """The folded FP32 V-cycle is as close to the FP64 cycle as the cycle of
+    one kernel per level operation with its FP64 coarsest solve (5 % for the
+    scatter of roundings), for rough and for smooth right-hand sides: one
+    level (both are the FP64 result rounded), two and three, dense parts of
+    both kinds."""
+    import torch
+    import paper_2310_14649_gb300 as sg
+    prob = sg.sg_setup(N, L, p, 2 * p, sigma2=0.3, bx=0.5, by=0.5)
+    m = N // 2 - 1
+    t = np.pi * np.arange(1, m + 1) / (m + 1.0)
+    smooth = 1.0 + np.sin(t)[:, None] * np.sin(2 * t)[None, :]
+    blocks = {"rough": random_block(m * m, prob.P, seed=38),
+              "smooth": smooth.reshape(-1, 1) * (1.0 + 0.1 * np.arange(prob.P))[None, :]}
+    err = {}
+    for kernel in (0, 1):
+        sg.sg_precond_setup(prob, 3, 3, 1, omega=0.3, amg_kernel=kernel)
+        for name, B in blocks.items():
+            B = B.astype(np.float32).astype(np.float64)
+            Y64, _ = run(prob, sg.PC_AMG, B, m * m, torch.float64)
+            Y32, _ = run(prob, sg.PC_AMG, B, m * m, torch.float32)
+            err[name, kernel] = np.linalg.norm(Y32 - Y64) / np.linalg.norm(Y64)
+    for name in blocks:
+        assert err[name, 0] <= 1.05 * err[name, 1], err
+    prob.close()
