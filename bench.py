@@ -406,6 +406,15 @@ def ev_time(torch, stream, fn):
     return a.elapsed_time(b), r
 
 
+def apply_bytes(prob, flux):
+    """Algorithmic bytes of one fine FP32 operator apply: the edge form reads
+    one conductance per edge and input term, the five-slot form the values
+    and the pattern; the two blocks once."""
+    n, P, K, nnz, N = prob.n, prob.P, prob.K, prob.nnzA, math.isqrt(prob.n) + 1
+    values = K * 2 * N * (N - 1) * 4 if flux else K * nnz * 4 + nnz * 4 + (n + 1) * 4
+    return values + 2 * n * P * 4
+
+
 def large_workload(sg, torch, stream, reps=3):
     """The 512x512 mesh, L=6, p=3 (P=84, K=924, 21.9M unknowns): mixed and
     plain FP64 solves, the apply's roofline (per-launch events in a separate
@@ -420,7 +429,7 @@ def large_workload(sg, torch, stream, reps=3):
     sg.sg_precond_setup(prob, c["sx"], c["sy"], c["overlap"], inner_rtol=INNER_RTOL, ras_kernel=RAS_KERNEL)
     for which in (1, 2, 3):
         sg.sg_apply_autotune(prob, which=which)
-    n, P, K, nnz = prob.n, prob.P, prob.K, prob.nnzA
+    n, P, K = prob.n, prob.P, prob.K
     X = torch.zeros((P, n), dtype=torch.float64, device="cuda")
 
     def solve(mode):
@@ -437,7 +446,8 @@ def large_workload(sg, torch, stream, reps=3):
     cnt, kms = sg.sg_profile_read(prob, 0)
     rcnt, rms = sg.sg_profile_read(prob, 4)
     sg.sg_profile(prob, False)
-    bytes_f32 = K * nnz * 4 + nnz * 4 + (n + 1) * 4 + 2 * n * P * 4
+    flux_on = sg.sg_apply_flux(prob, -1)
+    bytes_f32 = apply_bytes(prob, flux_on)
     avg = kms / max(cnt, 1)
     peak, peak_kind = peaks()
     out = {"workload": "poisson512_L6_p3", "N": c["N"], "L": c["L"], "P": P, "K": K, "unknowns": n * P,
@@ -445,7 +455,8 @@ def large_workload(sg, torch, stream, reps=3):
            "mixed_ms": round(ms32, 2), "mixed_outer_it": info32["outer_it"], "mixed_relres": info32["relres"],
            "plain_fp64_ms": round(ms64, 2), "plain_fp64_outer_it": info64["outer_it"],
            "speedup_mixed": round(ms64 / ms32, 3),
-           "roofline": {"kernel": "sg_apply FP32 (fine Galerkin operator, five-slot form)", "bound": "hbm",
+           "roofline": {"kernel": "sg_apply FP32 (fine Galerkin operator, %s form)" % ("edge-flux" if flux_on else
+                                                                                       "five-slot"), "bound": "hbm",
                         "achieved": round(bytes_f32 / (avg * 1e-3) / 1e9, 1), "peak": peak, "unit": "GB/s",
                         "frac": round(bytes_f32 / (avg * 1e-3) / 1e9 / peak, 4), "peak_source": peak_kind,
                         "bytes_per_launch": bytes_f32, "avg_launch_ms": avg, "launches": cnt},
@@ -683,15 +694,9 @@ def main():
         kinds[name] = (cnt, kms)
     sg.sg_profile(prob, False)
 
-    # roofline of the fine FP32 operator apply: algorithmic bytes per launch
-    # (five-slot form: values, pattern and blocks read once; edge form: one
-    # conductance per edge and term)
-    K, nnz = prob.K, prob.nnzA
+    # roofline of the fine FP32 operator apply
     flux_on = sg.sg_apply_flux(prob, -1)
-    N_ = c["N"]
-    bytes_slot = K * nnz * 4 + nnz * 4 + (n + 1) * 4 + 2 * n * P * 4
-    bytes_flux = K * 2 * N_ * (N_ - 1) * 4 + 2 * n * P * 4
-    bytes_f32 = bytes_flux if flux_on else bytes_slot
+    bytes_f32 = apply_bytes(prob, flux_on)
     cnt, kms = kinds["apply_fine_f32"]
     avg_ms = kms / max(cnt, 1)
     achieved = bytes_f32 / (avg_ms * 1e-3) / 1e9 if cnt else None
@@ -774,7 +779,7 @@ def main():
         for _ in range(3):
             sg.sg_apply(prob, Xa, Ya)
         ms_a, _ = ev_time(torch, stream, lambda: [sg.sg_apply(prob, Xa, Ya) for _ in range(20)])
-        byt = bytes_flux if mode else bytes_slot
+        byt = apply_bytes(prob, mode)
         apply_forms[form] = {"ms": round(ms_a / 20, 5), "bytes": byt, "gbs": round(byt / (ms_a / 20 * 1e-3) / 1e9, 1)}
     sg.sg_apply_flux(prob, 2)
     sg.sg_apply_autotune(prob)                 # the tuned choice again (cached)
