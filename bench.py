@@ -695,6 +695,7 @@ def main():
     sg.sg_profile(prob, False)
 
     # roofline of the fine FP32 operator apply
+    K, N_ = prob.K, c["N"]
     flux_on = sg.sg_apply_flux(prob, -1)
     bytes_f32 = apply_bytes(prob, flux_on)
     cnt, kms = kinds["apply_fine_f32"]
