@@ -224,7 +224,7 @@ sg_status sg_residual_refine(sg_problem* prob, const double* F_dev, int64_t ldf,
  * warps (1, 2 or 4 warps per group, i.e. 32, 64 or 128 rows per tile: narrow
  * groups let many slot or input groups share one CTA without capping its
  * registers; fewer than 4 only without staging or separate CTAs).
- * Recompiles.
+ * The shape that sg_apply_info reports is always accepted.  Recompiles.
  * Errors: SG_ERR_ARG out of range, SG_ERR_CUDA compile failure. */
 sg_status sg_apply_config(sg_problem* prob, int which, int rows, int groups, int igroups, int sgroups,
                           int prefetch, int min_blocks, int stages, int cgroups, int warps);

@@ -114,6 +114,13 @@ sg_status sg_apply_config(sg_problem* pr, int which, int rows, int groups, int i
   c.stages = stages;
   c.cgroups = cgroups;
   c.warps = warps;
+  // the shape that sg_apply_info reports for an edge form whose outputs are
+  // split (P > 110) is none of the slot form, whose own shape it stands for
+  const JitConfig e = jit_config(pr, which);
+  if (e.flux && e.cgroups > 1 && rows == e.rows && groups == e.groups && igroups == e.igroups &&
+      sgroups == e.sgroups && prefetch == e.prefetch && min_blocks == e.min_blocks && stages == e.stages &&
+      cgroups == e.cgroups && warps == e.warps)
+    c = jit_slot_config(pr, which);
   return jit_configure(pr, which, c);
 }
 

@@ -312,6 +312,7 @@ sg_status apply_ell(const Ell& A, const TripleTables& tri, int P, int K, const T
 std::string jit_apply_source(const sg_problem* pr, const JitConfig& c, bool fp64 = false);
 std::string jit_edge_source(const sg_problem* pr, const JitConfig& c, bool fp64);
 JitConfig jit_default_config(const sg_problem* pr, int which);
+JitConfig jit_slot_config(const sg_problem* pr, int which);  // the same in the five-slot form
 // turns of the edge form's loop, and the input term at each position of its
 // conductance blocks
 int jit_edge_rotations(const sg_problem* pr);

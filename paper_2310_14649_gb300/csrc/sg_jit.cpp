@@ -896,6 +896,10 @@ JitConfig jit_default_config(const sg_problem* pr, int which) {
     if (which == 1 && coarse_edge_default(pr)) return edge_default(pr, pr->N / 2, false);
     if (which == 5) return edge_default(pr, pr->N, true);
   }
+  return jit_slot_config(pr, which);
+}
+
+JitConfig jit_slot_config(const sg_problem* pr, int which) {
   const bool fp64 = which == 2 || which == 3;
   JitConfig c;
   c.rows = 1;

@@ -542,3 +542,20 @@ def test_first_slot_form_apply_can_be_captured(gpu, choice):
     torch.cuda.synchronize()
     assert torch.equal(Y, Z) and bool(Z.any())
     prob.close()
+
+
+@pytest.mark.parametrize("L,p,q", [(3, 2, 4), (5, 4, 4)])
+def test_reported_shape_is_accepted(gpu, L, p, q):
+    """sg_apply_config takes what sg_apply_info reports, also for an edge form
+    with split outputs (P = 126), and selects the slot form."""
+    import torch
+    import paper_2310_14649_gb300 as sg
+    prob, ref = setup_pair(9, L, p, q)
+    X = random_block(ref.n, ref.P, seed=95)
+    for which in (0, 2):
+        shape = sg.sg_apply_info(prob, which=which)
+        sg.sg_apply_config(prob, which=which, **{k: shape[k] for k in (
+            "rows", "groups", "igroups", "sgroups", "prefetch", "min_blocks", "stages", "cgroups", "warps")})
+        check_apply(prob, ref, X, torch.float64 if which else torch.float32)
+    assert sg.sg_apply_flux(prob, -1) == 0
+    prob.close()
