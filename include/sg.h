@@ -160,10 +160,11 @@ sg_status sg_apply(sg_problem* prob, sg_dtype dtype, const void* X_dev, int64_t 
 sg_status sg_set_apply_kernel(sg_problem* prob, int mode);
 
 /* FP64 applies (Sec. 2.1, Eq. Galerkin_L_exp) over assembled blocks: the K
- * values of each stencil edge summed once into its symmetric P x P block,
- * C_ab = sum_k g_kab v_k (P (P + 1) / 2 doubles per edge, S per row), so an
- * FP64 apply costs P^2 FMAs per edge instead of two FP64 operations per
- * triple (GB300's FP64 units bound the FP64 applies).  mode 0 (default):
+ * values of each edge summed once into its symmetric P x P block, B_ab =
+ * sum_k g_kab w_k (P (P + 1) / 2 doubles per edge, 2.1 to 3 edges per row),
+ * and each edge's flux formed once for both its nodes, so an FP64 apply costs
+ * P^2 FMAs per edge instead of two FP64 operations per triple (GB300's FP64
+ * units bound the FP64 applies).  mode 0 (default):
  * built on the first FP64 apply of the fine and of the coarse operator
  * when the blocks take at most a quarter of the free device memory; 1:
  * never (the generated or shared-memory kernel); 2: always, built now
@@ -312,11 +313,12 @@ typedef struct {
                           coarse GMRES: 1 (<= 0) = classical, the
                           PETSc default the paper's runs used (Sec. 5);
                           2 = classical with one re-orthogonalisation   */
-  int amg_kernel;      /* AMG V-cycle kernels: 0 = level 0 as three
-                          GPU-wide kernels and all coarser levels in one
-                          launch (one CTA per PCE mode, level vectors in
-                          shared memory); 1 = one launch per level
-                          operation                                      */
+  int amg_kernel;      /* AMG V-cycle kernels: 0 = FP32 cycles of a coarse
+                          operator in the edge form (sg_apply_flux) folded,
+                          the Jacobi steps multiplied into the transfers and
+                          the lower levels one dense product, others as
+                          phase kernels with lane groups per sparse row;
+                          1 = one launch per level operation             */
   int ras_stages;      /* line steps whose matrices the RAS kernel keeps in
                           flight or resident (2..8); 0 = automatic       */
   int ras_kernel;      /* RAS local solves on FP32 data: 0 = FMA kernel;

@@ -337,14 +337,14 @@ template <typename T>
 sg_status jit_edge_launch(sg_problem* pr, int which, const EdgeVals& A, const T* X, int64_t ldx, const T* F,
                           int64_t ldf, T* Y, int64_t ldy, cudaStream_t st);
 // Whether FP32 solves run on the edge form: what the program configured or
-// tuned for the fine family, else P <= 48.  Above that the five-slot form
-// was the default, and a mixed solve that stops at a relative residual of
-// 1e-8 carries the rounding error of its FP32 operator: 1.1e-9 of the
-// solution at 384^2, P = 70 (2e-11 in the edge form; below 2e-11 in either
-// form up to P = 35), so a change of form there would move the returned
-// solutions by more than their FP64 results may move.  The edge form is
-// several times faster (345 us against 2.1 ms an apply): sg_apply_flux(prob,
-// 1) selects it.
+// tuned for the fine family, else P <= 48.  A mixed solve that stops at a
+// relative residual of 1e-8 carries the rounding error of its FP32 operator:
+// 1.1e-9 of the solution at 384^2, P = 70 in the five-slot form, 2e-11 in the
+// edge form (below 2e-11 in either up to P = 35).  Above the line untuned
+// handles keep the five-slot form and with it the solutions they have
+// returned all along, digit for digit; the edge form is nearer the exact
+// solution and several times faster (345 us against 1.29 ms an apply at that
+// size), and sg_apply_flux(prob, 1) selects it.
 bool solver_edge(const sg_problem* pr);
 // whether coarse solves use the coarse edge form and the folded V-cycle
 // (sg_precond_setup decides it once, Precond::coarse_edge): in solves that use
