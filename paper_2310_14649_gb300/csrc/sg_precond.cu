@@ -1229,7 +1229,7 @@ __global__ void __launch_bounds__(128) k_fold_down(const __grid_constant__ FoldD
 // 64 rows of MT modes: 3 up to n = 1,024 or 12 modes, where smaller tiles fill
 // the GPU (n = 687, 35 modes: 12 a warp 10.6 us, 3 a warp 7.6), else 12, which
 // reads the matrix once for 48 modes (n = 1,674, 35 modes: 19.3 us, 3 a warp 30.3).
-// EXACT (n <= kFoldExact, where the dense part replaces little but the FP64
+// EXACT (n <= kFoldExact, 3 modes a warp, where the dense part replaces little but the FP64
 // inverse of the coarsest level): the matrix as hi + lo, every product and
 // sum in double-FP32, so the result is the FP64 one rounded.  Else C products
 // at a time in FP32 and these sums in double-FP32 (n = 1,674, 15 modes, 12 a
@@ -1495,8 +1495,6 @@ sg_status fold_attrs_init() {
                                int(fold_dense_smem(kFoldMax))));
   SG_CUDA(cudaFuncSetAttribute(k_fold_dense<false, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                int(fold_dense_smem(kFoldMax))));
-  SG_CUDA(cudaFuncSetAttribute(k_fold_dense<true, 12>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               int(fold_dense_smem(kFoldExact))));
   SG_CUDA(cudaFuncSetAttribute(k_fold_dense<true, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                int(fold_dense_smem(kFoldExact))));
   SG_CUDA(cudaFuncSetAttribute(k_fold_up<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024));
@@ -1573,8 +1571,9 @@ sg_status amg_fold_apply(const AmgHier& H, AmgWork<float>& w, int P, const float
     const int modes = P <= 12 || n <= 1024 ? 12 : 48;
     const dim3 grid(kDenseSplit, unsigned((n + kDenseRows - 1) / kDenseRows), unsigned((P + modes - 1) / modes));
     const bool all = F.lf == 0;  // the whole cycle
-    const auto dense = n <= kFoldExact ? (modes == 12 ? k_fold_dense<true, 3> : k_fold_dense<true, 12>)
-                                       : (modes == 12 ? k_fold_dense<false, 3> : k_fold_dense<false, 12>);
+    const auto dense = n <= kFoldExact ? k_fold_dense<true, 3>
+                       : modes == 12   ? k_fold_dense<false, 3>
+                                       : k_fold_dense<false, 12>;
     dense<<<grid, 128, fold_dense_smem(n), st>>>(n, F.ldd, F.dense.as<float>(), F.dense_lo.as<float>(),
                                                  all ? b : w.b[F.lf], all ? ldb : L.ld, P, all ? out : w.x[F.lf],
                                                  all ? ldo : L.ld, fold_slice(n), all ? j : nullptr, bstride);
